@@ -64,7 +64,7 @@ struct AdjArgs {
     int n[3];             // kernel-axis extents
     int bc_lo[3], bc_hi[3];
     T gamma, gm1;
-    T dxk[3];             // per kernel axis: dx (FP64) or 1/dx (FP32)
+    width_t<T> dxk[3];    // per kernel axis
     // z faces of kind BC_HALO (a slab of a decomposed mesh): the ghost planes
     // of Uc below / above the slab ([5][2][ny][nx], z fastest-but-one) and the
     // accumulators of the primitive cotangent the faces scatter onto them
@@ -228,7 +228,7 @@ __device__ void hllc_vjp(const T WL[NF], const T WR[NF], T gamma, const T Fb[NF]
 // primitives (reflections not yet undone) and the face's explicit d/dgamma.
 template <typename T, int PA>
 __device__ __forceinline__ void face_vjp_core(const T q[4][NF], const T ll[NF], const T lr[NF],
-                                              T dxk, T gamma, T qb[4][NF], T& gb) {
+                                              width_t<T> dxk, T gamma, T qb[4][NF], T& gb) {
     using R = Rot<PA>;
     // face flux cotangent (lambda_m - lambda_{m-1}) / dx
     T Fb[NF];
@@ -244,8 +244,8 @@ __device__ __forceinline__ void face_vjp_core(const T q[4][NF], const T ll[NF], 
         s2[f] = minmod_sel(d1, d2);
         const T m1 = s1[f] == 1 ? d0 : (s1[f] == 2 ? d1 : T(0));
         const T m2 = s2[f] == 1 ? d1 : (s2[f] == 2 ? d2 : T(0));
-        qL[f] = madd(T(0.5), m1, q[1][f]);
-        qR[f] = madd(T(-0.5), m2, q[2][f]);
+        qL[f] = add_half(q[1][f], m1);
+        qR[f] = sub_half(q[2][f], m2);
     }
     const T WL[NF] = {qL[0], qL[R::n], qL[R::t1], qL[R::t2], qL[4]};
     const T WR[NF] = {qR[0], qR[R::n], qR[R::t1], qR[R::t2], qR[4]};

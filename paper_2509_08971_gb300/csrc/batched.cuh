@@ -55,13 +55,12 @@ __device__ __forceinline__ StageArgs<T> batch_stage_args(const BatchProblem& P, 
     A.gamma = (T)P.gamma;
     A.gm1 = (T)(P.gamma - 1.0);
     A.igm1 = (T)(1.0 / (P.gamma - 1.0));
-    const bool f64 = sizeof(T) == 8;
-    A.dxk[0] = f64 ? (T)dx : (T)(1.0 / dx);
-    A.dxk[1] = f64 ? (T)dy : (T)(1.0 / dy);
-    A.dxk[2] = T(1);
+    A.dxk[0] = make_width<T>(dx);
+    A.dxk[1] = make_width<T>(dy);
+    A.dxk[2] = make_width<T>(1.0);
     A.rdx[0] = A.dxk[0];
     A.rdx[1] = A.dxk[1];
-    A.rdx[2] = T(1);
+    A.rdx[2] = A.dxk[2];
     A.act[0] = true;
     A.act[1] = two_d;
     A.act[2] = false;

@@ -24,11 +24,6 @@ using T = HH_T;
 
 template <typename V> __host__ __device__ inline V cdiv(V a, V b) { return (a + b - 1) / b; }
 
-inline T width_param(double dx) {
-    // FP64 kernels divide by dx; FP32 kernels multiply by 1/dx
-    return sizeof(T) == 8 ? (T)dx : (T)(1.0 / dx);
-}
-
 StageArgs<T> make_args(const MeshDesc& m, const TileDesc& td, const StageCall& c) {
     StageArgs<T> A;
     A.U0 = static_cast<const T*>(c.U0);
@@ -39,8 +34,8 @@ StageArgs<T> make_args(const MeshDesc& m, const TileDesc& td, const StageCall& c
         A.n[a] = m.n[a];
         A.bc_lo[a] = m.bc_lo[a];
         A.bc_hi[a] = m.bc_hi[a];
-        A.dxk[a] = width_param(m.dxk[a]);
-        A.rdx[a] = width_param(m.dx[a]);
+        A.dxk[a] = make_width<T>(m.dxk[a]);
+        A.rdx[a] = make_width<T>(m.dx[a]);
         A.act[a] = m.act[a];
     }
     A.gamma = (T)m.gamma;
@@ -269,15 +264,15 @@ __global__ void pointwise_stage_kernel(const T* U0, const T* Uc, T* Uo, long lon
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n5;
          q += (long long)gridDim.x * blockDim.x) {
         const T L = T(0);
-        Uo[q] = stage == 1 ? madd(d, L, Uc[q]) : madd(T(0.5), U0[q], T(0.5) * madd(d, L, Uc[q]));
+        Uo[q] = stage == 1 ? madd(d, L, Uc[q]) : add_half(T(0.5) * madd(d, L, Uc[q]), U0[q]);
     }
 }
 
 __global__ void rate_kernel(const T* __restrict__ U, long long N, T gamma, T gm1, bool a0,
-                            bool a1, bool a2, T r0, T r1, T r2, unsigned long long* slot,
+                            bool a1, bool a2, width_t<T> r0, width_t<T> r1, width_t<T> r2, unsigned long long* slot,
                             int* status) {
     const bool act[3] = {a0, a1, a2};
-    const T rdx[3] = {r0, r1, r2};
+    const width_t<T> rdx[3] = {r0, r1, r2};
     T rmax = T(0);
     bool bad = false;
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
@@ -437,7 +432,7 @@ AdjArgs<T> make_adj(const MeshDesc& m, const AdjointCall& c) {
         A.n[k] = m.n[k];
         A.bc_lo[k] = m.bc_lo[k];
         A.bc_hi[k] = m.bc_hi[k];
-        A.dxk[k] = width_param(m.dxk[k]);
+        A.dxk[k] = make_width<T>(m.dxk[k]);
     }
     A.gamma = (T)m.gamma;
     A.gm1 = (T)(m.gamma - 1.0);
@@ -494,7 +489,7 @@ cudaError_t HH_CAT(launch_rate_, HH_SUFFIX)(const MeshDesc& m, const void* U,
     if (blocks > 152 * 8) blocks = 152 * 8;
     rate_kernel<<<(int)blocks, 256, 0, s>>>(
         static_cast<const T*>(U), m.N, (T)m.gamma, (T)(m.gamma - 1.0), m.act[0], m.act[1],
-        m.act[2], width_param(m.dx[0]), width_param(m.dx[1]), width_param(m.dx[2]), rate_slot,
+        m.act[2], make_width<T>(m.dx[0]), make_width<T>(m.dx[1]), make_width<T>(m.dx[2]), rate_slot,
         status);
     return cudaGetLastError();
 }

@@ -32,8 +32,8 @@ struct StageArgs {
     int bc_lo[3], bc_hi[3];       // boundary kind per kernel axis
     T gamma, gm1;
     T igm1;                       // 1/(gamma-1), rounded once on the host (FP32 path)
-    T dxk[3];                     // per kernel axis: dx (FP64) or 1/dx (FP32)
-    T rdx[3];                     // per physical axis, same convention
+    width_t<T> dxk[3];            // per kernel axis (hydro_math.cuh)
+    width_t<T> rdx[3];            // per physical axis
     bool act[3];                  // per physical axis: active
     double dt;                    // used when dt_dev == nullptr
     const double* dt_dev;
@@ -295,8 +295,8 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, unsigned char*
                 for (int f = 0; f < NF; ++f) {
                     dcur[f] = qj[f] - qm1[f];
                     T d = minmod(dprev[f], dcur[f]);
-                    qR[f] = madd(T(-0.5), d, qm1[f]);
-                    qL[f] = madd(T(0.5), d, qm1[f]);
+                    qR[f] = sub_half(qm1[f], d);
+                    qL[f] = add_half(qm1[f], d);
                 }
                 if (cnt >= 3) hllc_axis<2>(qLp, qR, gamma, gm1, igm1, Fz);   // face j-3/2
 #pragma unroll
@@ -334,7 +334,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, unsigned char*
                     Uo[f] = madd(dt, L[f], uc);
                 } else {
                     T u0 = A.U0[f * A.N + c];
-                    Uo[f] = madd(T(0.5), u0, T(0.5) * madd(dt, L[f], uc));
+                    Uo[f] = add_half(T(0.5) * madd(dt, L[f], uc), u0);
                 }
                 A.Uo[f * A.N + c] = Uo[f];
             }

@@ -266,8 +266,8 @@ stage_tma_kernel(const __grid_constant__ StageArgs<T> A, const __grid_constant__
 #pragma unroll
                 for (int f = 0; f < NF; ++f) {
                     const T d = minmod(dprev[f], dcur[f]);
-                    qR[f] = madd(T(-0.5), d, qm1[f]);
-                    qL[f] = madd(T(0.5), d, qm1[f]);
+                    qR[f] = sub_half(qm1[f], d);
+                    qL[f] = add_half(qm1[f], d);
                 }
                 if (it >= 3) hllc_axis<2>(qLp, qR, gamma, gm1, igm1, Fz);  // face j-3/2
 #pragma unroll
@@ -397,8 +397,8 @@ stage_tma_kernel(const __grid_constant__ StageArgs<T> A, const __grid_constant__
                 const T uc = Sk[(f * HYC + ty + 2) * HXC + tx + 4];
                 Uo[f] = STAGE == 1
                             ? madd(dt, Lf, uc)
-                            : madd(T(0.5), u0s[(it & 1) * L::U0S + (f * TY + ty) * TX + tx],
-                                   T(0.5) * madd(dt, Lf, uc));
+                            : add_half(T(0.5) * madd(dt, Lf, uc),
+                                       u0s[(it & 1) * L::U0S + (f * TY + ty) * TX + tx]);
                 A.Uo[f * Nu + cell] = Uo[f];
             }
             cell += plane;

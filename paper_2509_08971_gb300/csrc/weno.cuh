@@ -36,9 +36,10 @@ constexpr int WENO_G = 3;                 // ghost layers
 
 // ---------------------------------------------------------------- WENO5-Z --
 __device__ __forceinline__ double weno5z(double v0, double v1, double v2, double v3, double v4) {
-    const double p0 = (2.0 * v0 - 7.0 * v1 + 11.0 * v2) / 6.0;
-    const double p1 = (-v1 + 5.0 * v2 + 2.0 * v3) / 6.0;
-    const double p2 = (2.0 * v2 + 5.0 * v3 - v4) / 6.0;
+    const double sixth = 1.0 / 6.0;                    // rounded: the reciprocal div_by wants
+    const double p0 = div_by(2.0 * v0 - 7.0 * v1 + 11.0 * v2, 6.0, sixth, true);
+    const double p1 = div_by(-v1 + 5.0 * v2 + 2.0 * v3, 6.0, sixth, true);
+    const double p2 = div_by(2.0 * v2 + 5.0 * v3 - v4, 6.0, sixth, true);
     const double s0 = v0 - 2.0 * v1 + v2, t0 = v0 - 4.0 * v1 + 3.0 * v2;
     const double s1 = v1 - 2.0 * v2 + v3, t1 = v1 - v3;
     const double s2 = v2 - 2.0 * v3 + v4, t2 = 3.0 * v2 - 4.0 * v3 + v4;
@@ -97,9 +98,11 @@ __device__ __forceinline__ void hll_normal(const double WL[NF], const double WR[
 #pragma unroll
         for (int f = 0; f < NF; ++f) F[f] = FR[f];
     } else {
+        const double D = SR - SL, y = __drcp_rn(D), SS = SL * SR;
+        const bool ok = mid_exponent(D);
 #pragma unroll
         for (int f = 0; f < NF; ++f)
-            F[f] = (SR * FL[f] - SL * FR[f] + SL * SR * (UR[f] - UL[f])) / (SR - SL);
+            F[f] = div_by(SR * FL[f] - SL * FR[f] + SS * (UR[f] - UL[f]), D, y, ok);
     }
 }
 __device__ __forceinline__ void hll_normal(const float WL[NF], const float WR[NF], float gamma,
@@ -453,7 +456,7 @@ weno_stage_kernel(const StageArgs<T> A) {
                     Uo[f] = madd(dt, L[f], uc);
                 } else {
                     const T u0 = A.U0[f * A.N + c];
-                    Uo[f] = madd(T(0.5), u0, T(0.5) * madd(dt, L[f], uc));
+                    Uo[f] = add_half(T(0.5) * madd(dt, L[f], uc), u0);
                 }
                 A.Uo[f * A.N + c] = Uo[f];
             }
@@ -527,7 +530,7 @@ struct AdvectArgs {
     long long N;
     int n[3];
     int bc_lo[3], bc_hi[3];
-    T dxk[3];            // per kernel axis: dx (FP64) or 1/dx (FP32)
+    width_t<T> dxk[3];   // per kernel axis
     double dt;
     int stage;
     int zchunk;
@@ -728,7 +731,7 @@ __global__ void __launch_bounds__(TX * TY) weno_advect_kernel(const AdvectArgs<T
         if (k >= 0 && own) {
             const long long c = ((long long)k * A.n[1] + y) * A.n[0] + x;
             const T ec = A.Ec[c];
-            A.Eo[c] = A.stage == 1 ? madd(dt, L, ec) : madd(T(0.5), A.E0[c], T(0.5) * madd(dt, L, ec));
+            A.Eo[c] = A.stage == 1 ? madd(dt, L, ec) : add_half(T(0.5) * madd(dt, L, ec), A.E0[c]);
         }
     }
 }

@@ -17,8 +17,6 @@ using T = HH_T;
 
 template <typename V> inline V wcdiv(V a, V b) { return (a + b - 1) / b; }
 
-inline T width_param_w(double dx) { return sizeof(T) == 8 ? (T)dx : (T)(1.0 / dx); }
-
 // The kernel arguments of one stage (the same fields the PLM kernels get).
 StageArgs<T> weno_args(const MeshDesc& m, int zchunk, const StageCall& c) {
     StageArgs<T> A{};
@@ -30,8 +28,8 @@ StageArgs<T> weno_args(const MeshDesc& m, int zchunk, const StageCall& c) {
         A.n[a] = m.n[a];
         A.bc_lo[a] = m.bc_lo[a];
         A.bc_hi[a] = m.bc_hi[a];
-        A.dxk[a] = width_param_w(m.dxk[a]);
-        A.rdx[a] = width_param_w(m.dx[a]);
+        A.dxk[a] = make_width<T>(m.dxk[a]);
+        A.rdx[a] = make_width<T>(m.dx[a]);
         A.act[a] = m.act[a];
     }
     A.gamma = (T)m.gamma;
@@ -128,7 +126,7 @@ cudaError_t HH_WCAT(launch_advect_E_stage_, HH_SUFFIX)(const MeshDesc& m, int st
         A.n[a] = m.n[a];
         A.bc_lo[a] = m.bc_lo[a];
         A.bc_hi[a] = m.bc_hi[a];
-        A.dxk[a] = width_param_w(m.dxk[a]);
+        A.dxk[a] = make_width<T>(m.dxk[a]);
     }
     A.dt = dt;
     A.stage = stage;

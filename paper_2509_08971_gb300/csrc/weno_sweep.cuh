@@ -276,7 +276,7 @@ weno_march_kernel(const StageArgs<T> A, T* __restrict__ L) {
                         T Uo[NF];
 #pragma unroll
                         for (int f = 0; f < NF; ++f) {
-                            Uo[f] = two ? madd(T(0.5), U0c[f], T(0.5) * madd(dt, D[f], Uc_[f]))
+                            Uo[f] = two ? add_half(T(0.5) * madd(dt, D[f], Uc_[f]), U0c[f])
                                         : madd(dt, D[f], Uc_[f]);
                             A.Uo[f * N + c] = Uo[f];
                         }
@@ -444,7 +444,7 @@ advect_march_kernel(const AdvectArgs<T> A, T* __restrict__ L) {
                     const T D = sub_over_dx(Lc, F - Fp, A.dxk[AX]);
                     if constexpr (LAST) {
                         const T ec = we[1];
-                        A.Eo[c] = two ? madd(T(0.5), E0c, T(0.5) * madd(dt, D, ec)) : madd(dt, D, ec);
+                        A.Eo[c] = two ? add_half(T(0.5) * madd(dt, D, ec), E0c) : madd(dt, D, ec);
                     } else {
                         L[c] = D;
                     }
