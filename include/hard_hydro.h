@@ -98,7 +98,8 @@ int hard_hydro_set_cells(hard_hydro_t h, double dx, double dy, double dz);
  * built-in default).  Tile ids index a table that depends on the number of
  * active axes of the handle's mesh: hard_hydro_tile_count returns its size
  * (or a negative error code) and hard_hydro_tile_info writes
- * {tile_x, tile_y, z_chunk, threads_per_block} of one entry. */
+ * {tile_x, tile_y, z_chunk, threads_per_block} of one entry (1D and 2D meshes:
+ * tile_y rows per warp, 28 cells of a row per warp). */
 int hard_hydro_set_kernel(hard_hydro_t h, int kernel, int tile);
 int hard_hydro_tile_count(hard_hydro_t h);
 int hard_hydro_tile_info(hard_hydro_t h, int tile, int out4[4]);
@@ -280,7 +281,7 @@ hard_batch_t hard_batch_create(int nprob, const int* nx, const int* ny, const in
 long long hard_batch_offset(hard_batch_t b, int p);
 long long hard_batch_elements(hard_batch_t b);
 int hard_batch_tile_count(void);
-/* tile id: {1D tile width, 2D tile} = 0: {256, 32x8}, 1: {128, 32x4}, 2: {512, 64x8} */
+/* tile id: warps per block = 0: 8, 1: 4, 2: 16 */
 int hard_batch_set_tile(hard_batch_t b, int tile);
 int hard_hydro_step_batched(hard_batch_t b, void* U_packed, int nsteps, double cfl, double* t_dev,
                             void* stream);

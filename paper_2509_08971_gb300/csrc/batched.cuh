@@ -10,14 +10,19 @@
 //         stage 1 over the problem's tiles: U -> W
 //         stage 2 over the problem's tiles: (U, W) -> U, signal rate fused
 //         r = block max of that rate;  t += dt         (FP64)
-// The tiles are evaluated by the same stage_tile code as the single-problem
-// kernel, so a problem advanced here matches the same problem advanced alone
-// bit for bit.  State is read through the coherent cache path because the
-// block rewrites it within the launch.  A block never waits on another block:
-// problems are disjoint and the rate reduction is block-local.
+// A problem's cells are evaluated by strip_rows, as on a single 1D or 2D mesh,
+// so a problem advanced here matches the same problem advanced alone bit for
+// bit: the block's warps take strips of 28 cells by a chunk of rows.  State is
+// read through the coherent cache path because the block rewrites it within
+// the launch.  A block never waits on another block: problems are disjoint and
+// the rate reduction is block-local.
+//
+// What bounds it: instruction issue (strip.cuh).  The FP64 scalars of a
+// problem (widths, dt, t) are one thread's work: a warp's FP64 instruction
+// holds the SM's pipe for 16 clocks.
 #pragma once
 #include "launch.h"
-#include "stage_kernel.cuh"
+#include "strip.cuh"
 
 namespace hh {
 
@@ -35,11 +40,18 @@ struct BatchArgs {
     int* status;
 };
 
+// What a problem's stages share, set up once by one thread.
 template <typename T>
-__device__ __forceinline__ StageArgs<T> batch_stage_args(const BatchProblem& P, T* U, T* W,
+struct BatchScalars {
+    T gamma, gm1, igm1;
+    width_t<T> dx, dy;
+};
+
+template <typename T>
+__device__ __forceinline__ StageArgs<T> batch_stage_args(const BatchProblem& P,
+                                                        const BatchScalars<T>& S, T* U, T* W,
                                                         int stage, double dt) {
     StageArgs<T> A;
-    const bool two_d = P.ny > 1;
     A.U0 = U;
     A.Uc = stage == 1 ? U : W;
     A.Uo = stage == 1 ? W : U;
@@ -51,18 +63,14 @@ __device__ __forceinline__ StageArgs<T> batch_stage_args(const BatchProblem& P, 
         A.bc_lo[a] = P.bc;
         A.bc_hi[a] = P.bc;
     }
-    const double dx = 1.0 / P.nx, dy = 1.0 / P.ny;
-    A.gamma = (T)P.gamma;
-    A.gm1 = (T)(P.gamma - 1.0);
-    A.igm1 = (T)(1.0 / (P.gamma - 1.0));
-    A.dxk[0] = make_width<T>(dx);
-    A.dxk[1] = make_width<T>(dy);
-    A.dxk[2] = make_width<T>(1.0);
-    A.rdx[0] = A.dxk[0];
-    A.rdx[1] = A.dxk[1];
-    A.rdx[2] = A.dxk[2];
+    A.gamma = S.gamma;
+    A.gm1 = S.gm1;
+    A.igm1 = S.igm1;
+    A.dxk[0] = A.rdx[0] = S.dx;
+    A.dxk[1] = A.rdx[1] = S.dy;
+    A.dxk[2] = A.rdx[2] = S.dy;                       // inactive
     A.act[0] = true;
-    A.act[1] = two_d;
+    A.act[1] = P.ny > 1;
     A.act[2] = false;
     A.dt = dt;
     A.dt_dev = nullptr;
@@ -77,36 +85,40 @@ __device__ __forceinline__ StageArgs<T> batch_stage_args(const BatchProblem& P, 
     return A;
 }
 
-// Block-wide maximum of a non-negative rate (NaN propagates), as a double.
-template <typename T, int NT>
-__device__ __forceinline__ double block_rate_max(T r, unsigned long long* red) {
+// The warps' largest rates into red[] (NaN propagates); the caller's barrier
+// orders them before the thread that combines them.
+template <typename T>
+__device__ __forceinline__ void warp_rate_max(T r, unsigned long long* red) {
     unsigned long long b = rate_bits(r);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long v = __shfl_xor_sync(0xffffffffu, b, o);
+        const unsigned long long v = __shfl_xor_sync(FULL, b, o);
         b = v > b ? v : b;
     }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    __syncthreads();                    // red[] free from any earlier use
-    if (lane == 0) red[warp] = b;
-    __syncthreads();
-    unsigned long long m = 0;
-#pragma unroll
-    for (int w = 0; w < NT / 32; ++w) m = red[w] > m ? red[w] : m;
-    return __longlong_as_double((long long)m);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = b;
 }
 
-// TX1: tile width of 1D problems; TX2 x TY2: tile of 2D problems.  Both use
-// the same block of TX1 == TX2 * TY2 threads.
-template <typename T, int TX1, int TX2, int TY2>
-__global__ void __launch_bounds__(TX1) batched_kernel(const BatchArgs<T> B) {
-    static_assert(TX1 == TX2 * TY2, "1D and 2D tiles share one block size");
-    constexpr int NT = TX1;
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ unsigned long long red[NT / 32];
-    __shared__ int s_next;
-    const int tid = threadIdx.x;
+// NW warps per block.
+template <typename T, int NW>
+__global__ void __launch_bounds__(32 * NW) batched_kernel(const BatchArgs<T> B) {
+    constexpr int NT = 32 * NW;
+    __shared__ unsigned long long red[NW];
+    __shared__ BatchScalars<T> s_sc;
+    __shared__ double s_dt, s_t;
+    __shared__ int s_next, s_chunks;
+    const int tid = threadIdx.x, warp = tid >> 5;
     bool bad = false;
+
+    // dt of the next step from the rates in red[], by one thread; every step
+    // but the last advances t
+    auto next_dt = [&]() {
+        unsigned long long m = 0;
+        for (int w = 0; w < NW; ++w) m = red[w] > m ? red[w] : m;
+        const double rate = __longlong_as_double((long long)m);
+        const bool ok = rate > 0.0 && !isinf(rate);
+        s_dt = ok ? B.cfl / rate : 0.0;
+        return ok;
+    };
 
     for (;;) {
         __syncthreads();
@@ -119,58 +131,82 @@ __global__ void __launch_bounds__(TX1) batched_kernel(const BatchArgs<T> B) {
         T* W = B.W + P.off;
         const bool two_d = P.ny > 1;
         const long long N = (long long)P.nx * P.ny;
+        const int strips = (P.nx + STRIP - 1) / STRIP;
+        if (tid == 0) {
+            s_sc.gamma = (T)P.gamma;
+            s_sc.gm1 = (T)(P.gamma - 1.0);
+            s_sc.igm1 = (T)(1.0 / (P.gamma - 1.0));
+            s_sc.dx = make_width<T>(1.0 / P.nx);
+            s_sc.dy = make_width<T>(1.0 / P.ny);
+            s_t = B.t[B.order[qi]];
+        }
+        if (warp == NW - 1) {
+            // row chunks per strip: of 1 .. 32, the one whose rounds over the
+            // block's warps take the fewest rows (a chunk pays about three
+            // rows for its warm-up and look-ahead)
+            const int k = (tid & 31) + 1;
+            const long long cost = (((long long)strips * k + NW - 1) / NW) * ((P.ny + k - 1) / k + 3);
+            const unsigned key = ((unsigned)min(cost, (1ll << 25) - 1) << 6) | (unsigned)k;
+            const unsigned best = __reduce_min_sync(FULL, key);
+            if ((tid & 31) == 0) s_chunks = two_d ? (int)(best & 63u) : 1;
+        }
+        __syncthreads();
+        const BatchScalars<T> sc = s_sc;
+        const int chunk = (P.ny + s_chunks - 1) / s_chunks;
+        const long long items = (long long)strips * s_chunks;    // below 2^32: at most 32 chunks
 
         // signal rate of the initial state
-        StageArgs<T> A1 = batch_stage_args<T>(P, U, W, 1, 0.0);
-        T r0 = T(0);
-        for (long long c = tid; c < N; c += NT) {
-            T Uc[NF], Wp[NF];
+        {
+            const StageArgs<T> A = batch_stage_args<T>(P, sc, U, W, 1, 0.0);
+            T r0 = T(0);
+            for (long long c = tid; c < N; c += NT) {
+                T Uc[NF], Wp[NF];
 #pragma unroll
-            for (int f = 0; f < NF; ++f) Uc[f] = U[f * N + c];
-            cons_to_prim(Uc, A1.gm1, Wp);
-            bad |= nonphys(Wp);
-            const T r = cell_rate(Wp, A1.gamma, A1.act, A1.rdx);
-            r0 = (r > r0 || r != r) ? r : r0;
-        }
-        double rate = block_rate_max<T, NT>(r0, red);
-        double t = B.t[B.order[qi]];
-
-        for (int step = 0; step < B.nsteps; ++step) {
-            double dt;
-            if (!(rate > 0.0) || isinf(rate)) {
-                dt = 0.0;
-                bad = true;
-            } else {
-                dt = B.cfl / rate;
+                for (int f = 0; f < NF; ++f) Uc[f] = U[f * N + c];
+                cons_to_prim(Uc, A.gm1, Wp);
+                bad |= nonphys(Wp);
+                const T r = cell_rate(Wp, A.gamma, A.act, A.rdx);
+                r0 = (r > r0 || r != r) ? r : r0;
             }
+            warp_rate_max(r0, red);
+        }
+        __syncthreads();
+        for (int step = 0; step < B.nsteps; ++step) {
+            if (tid == 0) {
+                if (!next_dt()) bad = true;
+                s_t += s_dt;
+            }
+            __syncthreads();
+            const double dt = s_dt;
             TileAcc<T> acc;
             acc.rate_max = T(0);
             acc.bad = false;
 #pragma unroll
             for (int f = 0; f < NF; ++f) acc.tot[f] = T(0);
-            int tile = 0;                   // tile count: the parity of stage_tile's plane
+#pragma unroll 1
             for (int stage = 1; stage <= 2; ++stage) {
-                StageArgs<T> A = batch_stage_args<T>(P, U, W, stage, dt);
-                // non-null: stage_tile folds the signal rate of the new state
+                StageArgs<T> A = batch_stage_args<T>(P, sc, U, W, stage, dt);
+                // non-null: strip_rows folds the signal rate of the new state
                 // into acc (it never writes through the pointer)
                 A.rate_slot = stage == 2 ? red : nullptr;
                 if (two_d) {
-                    for (int y0 = 0; y0 < P.ny; y0 += TY2)
-                        for (int x0 = 0; x0 < P.nx; x0 += TX2)
-                            stage_tile<T, TX2, TY2, 2, 0, 1, false>(A, smem_raw, x0, y0, 0, 1, acc,
-                                                                    tile++);
+                    for (unsigned it = warp; it < (unsigned)items; it += NW) {
+                        const unsigned c = it / (unsigned)strips;
+                        const int y0 = (int)c * chunk;
+                        if (y0 < P.ny)
+                            strip_rows<T, 2, 0, 1, false, 0>(A, (int)(it - c * strips) * STRIP, y0,
+                                                             min(y0 + chunk, P.ny), acc);
+                    }
                 } else {
-                    for (int x0 = 0; x0 < P.nx; x0 += TX1)
-                        stage_tile<T, TX1, 1, 1, 0, 0, false>(A, smem_raw, x0, 0, 0, 1, acc,
-                                                              tile++);
+                    for (int it = warp; it < strips; it += NW)
+                        strip_rows<T, 1, 0, 0, false, 1>(A, it * STRIP, 0, 1, acc);
                 }
+                if (stage == 2) warp_rate_max(acc.rate_max, red);
                 __syncthreads();            // every cell of this stage written
             }
             bad |= acc.bad;
-            rate = block_rate_max<T, NT>(acc.rate_max, red);
-            t = t + dt;
         }
-        if (tid == 0) B.t[B.order[qi]] = t;
+        if (tid == 0) B.t[B.order[qi]] = s_t;
     }
     if (__syncthreads_or(bad) && tid == 0) atomicOr(B.status, 1);
 }

@@ -200,8 +200,6 @@ double* tot_slot(hard_hydro_s* h) { return reinterpret_cast<double*>(h->slots + 
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-int tile_of(const hard_hydro_s* h) { return h->tile < 0 ? 0 : h->tile; }
-
 bool weno(const hard_hydro_s* h) { return h->scheme == HARD_SCHEME_WENO5Z_HLL && h->mesh.dim > 0; }
 
 bool has_halo(const hard_hydro_s* h) {
@@ -218,7 +216,7 @@ bool halo_ready(const hard_hydro_s* h) {
 // blocks of one stage launch (rows of the totals partial array)
 long long launch_blocks(const hard_hydro_s* h) {
     if (weno(h)) return hh::weno_stage_blocks(h->mesh, h->mesh.dim == 3);
-    return hh::stage_blocks(h->mesh, tile_of(h));
+    return hh::stage_blocks(h->mesh, h->tile, h->dtype == HARD_F64);
 }
 
 cudaError_t stage_launch(hard_hydro_s* h, const StageCall& call, cudaStream_t s) {
@@ -231,8 +229,8 @@ cudaError_t stage_launch(hard_hydro_s* h, const StageCall& call, cudaStream_t s)
         return h->dtype == HARD_F64 ? hh::launch_weno_stage_f64(h->mesh, c, s)
                                     : hh::launch_weno_stage_f32(h->mesh, c, s);
     }
-    if (h->dtype == HARD_F64) return hh::launch_stage_f64(h->mesh, h->kernel, tile_of(h), c, s);
-    return hh::launch_stage_f32(h->mesh, h->kernel, tile_of(h), c, s);
+    if (h->dtype == HARD_F64) return hh::launch_stage_f64(h->mesh, h->kernel, h->tile, c, s);
+    return hh::launch_stage_f32(h->mesh, h->kernel, h->tile, c, s);
 }
 
 // Both stages of one step, each over the whole mesh.
@@ -439,7 +437,7 @@ int hard_hydro_tile_info(hard_hydro_t h, int tile, int out4[4]) {
     out4[0] = t.tx;
     out4[1] = t.ty;
     out4[2] = t.zc;
-    out4[3] = t.tx * t.ty;
+    out4[3] = hh::tile_threads(h->mesh.dim, tile);
     return HARD_OK;
 }
 
@@ -935,7 +933,7 @@ bool handle_view(hard_hydro_t h, const MeshDesc** mesh, int* dtype, int* kernel,
     *mesh = &h->mesh;
     *dtype = h->dtype;
     *kernel = h->kernel;
-    *tile = tile_of(h);
+    *tile = h->tile;
     return true;
 }
 

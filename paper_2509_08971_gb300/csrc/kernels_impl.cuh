@@ -12,6 +12,7 @@
 #include "launch.h"
 #include "stage_kernel.cuh"
 #include "stage_tma.cuh"
+#include "strip.cuh"
 #ifdef HH_WS
 #include "stage_ws.cuh"
 #endif
@@ -57,17 +58,29 @@ StageArgs<T> make_args(const MeshDesc& m, const TileDesc& td, const StageCall& c
     return A;
 }
 
-template <int TX, int TY, int DIM, int PX, int PY>
+template <int TX, int TY>
 cudaError_t run_stage(const MeshDesc& m, const TileDesc& td, const StageCall& c, cudaStream_t s) {
     StageArgs<T> A = make_args(m, td, c);
-    dim3 grid(cdiv(m.n[0], TX), DIM >= 2 ? cdiv(m.n[1], TY) : 1,
-              DIM == 3 ? cdiv(A.zhi - A.zlo, A.zchunk) : 1);
-    const size_t smem = StageSmem<T, TX, TY, DIM>::bytes;
-    auto kern = stage_kernel<T, TX, TY, DIM, PX, PY, false>;
+    dim3 grid(cdiv(m.n[0], TX), cdiv(m.n[1], TY), cdiv(A.zhi - A.zlo, A.zchunk));
+    const size_t smem = StageSmem<T, TX, TY>::bytes;
+    auto kern = stage_kernel<T, TX, TY, 0, 1>;
     static std::atomic<unsigned long long> attr{0};
     cudaError_t e = smem_attr_once(kern, smem, attr);
     if (e != cudaSuccess) return e;
     kern<<<grid, TX * TY, smem, s>>>(A);
+    return cudaGetLastError();
+}
+
+// 1D and 2D meshes: one warp per strip and td.ty rows (strip.cuh).
+template <int DIM, int PX, int PY, int RR, int NWARP>
+cudaError_t run_strip(const MeshDesc& m, const TileDesc& td, const StageCall& c, cudaStream_t s) {
+    static_assert(STRIP == STRIP_CELLS, "the launch rule counts the kernel's strips");
+    StageArgs<T> A = make_args(m, td, c);
+    A.zchunk = td.ty;                                   // rows per warp
+    const long long strips = cdiv(m.n[0], STRIP), warps = strips * cdiv(m.n[1], td.ty);
+    const long long blocks = cdiv<long long>(warps, NWARP);
+    if (blocks >= (1ll << 31)) return cudaErrorInvalidValue;
+    strip_kernel<T, DIM, PX, PY, RR, NWARP><<<(unsigned)blocks, 32 * NWARP, 0, s>>>(A);
     return cudaGetLastError();
 }
 
@@ -333,8 +346,9 @@ __global__ void totals_kernel(const T* __restrict__ U, long long N, double* part
 template <int DIM, int PX, int PY>
 cudaError_t dispatch_tile(const MeshDesc& m, int kernel, int tile, const StageCall& c,
                           cudaStream_t s) {
-    const TileDesc td = tile_desc(DIM, tile);
+    const TileDesc td = launch_tile(m, tile, sizeof(T) == 8);
     if constexpr (DIM == 3) {
+        if (tile < 0) tile = 0;
         // the TMA kernel carries the rate / totals epilogue for stage 2 only
         const bool epi_ok = c.stage == 2 || (!c.rate_slot && !c.tot_partial);
         if (kernel == 0 && epi_ok && tma_eligible(m, c.Uc)) {
@@ -358,48 +372,35 @@ cudaError_t dispatch_tile(const MeshDesc& m, int kernel, int tile, const StageCa
             if (used || e != cudaSuccess) return e;
         }
         switch (tile) {
-            case 0: case 1: return run_stage<32, 8, 3, 0, 1>(m, td, c, s);
-            case 2: case 5: return run_stage<32, 16, 3, 0, 1>(m, td, c, s);
-            case 3: return run_stage<64, 8, 3, 0, 1>(m, td, c, s);
-            default: return run_stage<32, 4, 3, 0, 1>(m, td, c, s);
+            case 0: case 1: return run_stage<32, 8>(m, td, c, s);
+            case 2: case 5: return run_stage<32, 16>(m, td, c, s);
+            case 3: return run_stage<64, 8>(m, td, c, s);
+            default: return run_stage<32, 4>(m, td, c, s);
         }
     } else if constexpr (DIM == 2) {
-        if constexpr (PX != 0 || PY != 1) {
-            return run_stage<32, 8, 2, PX, PY>(m, tile_desc(2, 0), c, s);
-        } else {
-            switch (tile) {
-                case 0: return run_stage<32, 8, 2, 0, 1>(m, td, c, s);
-                case 1: return run_stage<32, 16, 2, 0, 1>(m, td, c, s);
-                default: return run_stage<64, 8, 2, 0, 1>(m, td, c, s);
-            }
+        switch (td.ty) {
+            case 2: return run_strip<2, PX, PY, 2, 2>(m, td, c, s);
+            case 4: return run_strip<2, PX, PY, 4, 2>(m, td, c, s);
+            default: return run_strip<2, PX, PY, 0, 2>(m, td, c, s);
         }
     } else {
-        if constexpr (PX != 0) {
-            return run_stage<128, 1, 1, PX, 0>(m, tile_desc(1, 0), c, s);
-        } else {
-            if (tile == 0) return run_stage<128, 1, 1, 0, 0>(m, td, c, s);
-            return run_stage<256, 1, 1, 0, 0>(m, td, c, s);
-        }
+        if (td.tx == STRIP) return run_strip<1, PX, 0, 1, 1>(m, td, c, s);
+        return run_strip<1, PX, 0, 1, 4>(m, td, c, s);
     }
 }
 
-template <int TX1, int TX2, int TY2>
+template <int NW>
 cudaError_t run_batched(const BatchCall& c, cudaStream_t s) {
-    constexpr size_t s1 = StageSmem<T, TX1, 1, 1>::bytes, s2 = StageSmem<T, TX2, TY2, 2>::bytes;
-    constexpr size_t smem = s1 > s2 ? s1 : s2;
-    auto kern = batched_kernel<T, TX1, TX2, TY2>;
+    auto kern = batched_kernel<T, NW>;
     static PerDeviceInt grids;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     int grid = grids.get(dev);
     if (grid == 0) {
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
         int sms = 0, per_sm = 0;
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, TX1, smem);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * NW, 0);
         if (e != cudaSuccess) return e;
         grid = sms * (per_sm > 0 ? per_sm : 1);
         grids.set(dev, grid);
@@ -416,7 +417,7 @@ cudaError_t run_batched(const BatchCall& c, cudaStream_t s) {
     B.counter = c.counter;
     B.status = c.status;
     const int blocks = grid < c.nprob ? grid : c.nprob;
-    kern<<<blocks, TX1, smem, s>>>(B);
+    kern<<<blocks, 32 * NW, 0, s>>>(B);
     return cudaGetLastError();
 }
 
@@ -505,9 +506,9 @@ cudaError_t HH_CAT(launch_totals_, HH_SUFFIX)(const MeshDesc& m, const void* U, 
 namespace hh {
 cudaError_t HH_CAT(launch_batched_, HH_SUFFIX)(const BatchCall& c, int tile, cudaStream_t s) {
     switch (tile) {
-        case 1: return run_batched<128, 32, 4>(c, s);
-        case 2: return run_batched<512, 64, 8>(c, s);
-        default: return run_batched<256, 32, 8>(c, s);
+        case 1: return run_batched<BATCH_WARPS[1]>(c, s);
+        case 2: return run_batched<BATCH_WARPS[2]>(c, s);
+        default: return run_batched<BATCH_WARPS[0]>(c, s);
     }
 }
 }  // namespace hh

@@ -2,7 +2,7 @@
 // states -> HLLC -> flux difference -> RK stage combine, one launch per stage,
 // with the signal-rate max and the conserved totals fused into the epilogue.
 //
-// Tiling (2.5D z-march).  A CTA owns a TX x TY column of the mesh and marches
+// 3D meshes (1D and 2D meshes: strip.cuh).  Tiling (2.5D z-march).  A CTA owns a TX x TY column of the mesh and marches
 // its z-chunk plane by plane.  For each plane it stages the haloed
 // (TX+4) x (TY+4) primitive plane in shared memory, evaluates every x and y
 // face flux once into shared memory and forms the x/y part of the flux
@@ -73,52 +73,45 @@ __device__ __forceinline__ int bc_map(int m, int n, int lo, int hi, bool& flip) 
     return s < 0 ? 0 : (s >= n ? n - 1 : s);
 }
 
-template <typename T, int TX, int TY, int DIM>
+template <typename T, int TX, int TY>
 struct StageSmem {
-    static constexpr int HX = TX + 4;
-    static constexpr int HY = DIM >= 2 ? TY + 4 : 1;
-    static constexpr int NP = NF * HX * HY;                       // primitive plane
-    static constexpr int NFX = NF * TY * (TX + 1);                // x-face fluxes
-    static constexpr int NFY = DIM >= 2 ? NF * (TY + 1) * TX : 0; // y-face fluxes
-    // two primitive planes (by plane parity, or by tile parity when a block
-    // evaluates one tile after another), one plane of x and y face fluxes
+    static constexpr int HX = TX + 4, HY = TY + 4;
+    static constexpr int NP = NF * HX * HY;               // primitive plane
+    static constexpr int NFX = NF * TY * (TX + 1);        // x-face fluxes
+    static constexpr int NFY = NF * (TY + 1) * TX;        // y-face fluxes
+    // two primitive planes (by plane parity), one plane of x and y face fluxes
     static constexpr size_t bytes = sizeof(T) * (2 * NP + NFX + NFY);
 };
 
 // Load the conserved values of kernel cell (gx, gy, gz) with the boundary map
 // applied along the active kernel axes, as primitives.
-// NC: the state is not written during this launch, so the read-only
-// (non-coherent) cache path may serve it.  A kernel that rewrites its input
-// within the launch (the batched time loop) must read with NC = false.
-template <typename T, int DIM, int PX, int PY, bool NC>
+template <typename T, int PX, int PY>
 __device__ __forceinline__ void load_prim(const StageArgs<T>& A, int gx, int gy, int gz, T W[NF],
                                           bool& bad) {
-    bool fx, fy = false, fz = false;
-    int sx = bc_map(gx, A.n[0], A.bc_lo[0], A.bc_hi[0], fx);
-    int sy = 0, sz = 0;
-    if (DIM >= 2) sy = bc_map(gy, A.n[1], A.bc_lo[1], A.bc_hi[1], fy);
+    bool fx, fy, fz = false;
+    const int sx = bc_map(gx, A.n[0], A.bc_lo[0], A.bc_hi[0], fx);
+    const int sy = bc_map(gy, A.n[1], A.bc_lo[1], A.bc_hi[1], fy);
+    int sz;
     const T* src = A.Uc;
     long long fstride = A.N;
-    if (DIM >= 3) {
-        const bool hlo = gz < 0 && A.bc_lo[2] == BC_HALO;
-        const bool hhi = gz >= A.n[2] && A.bc_hi[2] == BC_HALO;
-        if (hlo || hhi) {
-            // ghost plane from the neighbouring slab (planes -2, -1 / nz, nz+1)
-            const int k = hlo ? gz + 2 : gz - A.n[2];
-            sz = k < 0 ? 0 : (k > 1 ? 1 : k);
-            src = A.zg[hlo ? 0 : 1];
-            fstride = 2ll * A.n[1] * A.n[0];
-        } else {
-            sz = bc_map(gz, A.n[2], A.bc_lo[2], A.bc_hi[2], fz);
-        }
+    const bool hlo = gz < 0 && A.bc_lo[2] == BC_HALO;
+    const bool hhi = gz >= A.n[2] && A.bc_hi[2] == BC_HALO;
+    if (hlo || hhi) {
+        // ghost plane from the neighbouring slab (planes -2, -1 / nz, nz+1)
+        const int k = hlo ? gz + 2 : gz - A.n[2];
+        sz = k < 0 ? 0 : (k > 1 ? 1 : k);
+        src = A.zg[hlo ? 0 : 1];
+        fstride = 2ll * A.n[1] * A.n[0];
+    } else {
+        sz = bc_map(gz, A.n[2], A.bc_lo[2], A.bc_hi[2], fz);
     }
-    long long c = ((long long)sz * A.n[1] + sy) * A.n[0] + sx;
+    const long long c = ((long long)sz * A.n[1] + sy) * A.n[0] + sx;
     T U[NF];
 #pragma unroll
-    for (int f = 0; f < NF; ++f) U[f] = NC ? __ldg(src + f * fstride + c) : src[f * fstride + c];
+    for (int f = 0; f < NF; ++f) U[f] = __ldg(src + f * fstride + c);
     if (fx) U[1 + PX] = -U[1 + PX];
-    if (DIM >= 2 && fy) U[1 + PY] = -U[1 + PY];
-    if (DIM >= 3 && fz) U[3] = -U[3];
+    if (fy) U[1 + PY] = -U[1 + PY];
+    if (fz) U[3] = -U[3];
     cons_to_prim(U, A.gm1, W);
     bad |= nonphys(W);
 }
@@ -184,18 +177,12 @@ __device__ __forceinline__ bool sum5_writer(int lane) {
     return lane == 0 || lane == 4 || lane == 8 || lane == 16 || lane == 24;
 }
 
-// One tile of one stage: the TX x TY column at (x0, y0), z-planes [z0, z1)
-// (DIM == 3; a single plane otherwise).  Writes the completed cells of the
-// tile to A.Uo and folds them into `acc`.  All threads of the block call it.
-// A block that evaluates tiles one after another numbers them in `tile`: the
-// primitive plane alternates by that parity (by plane parity along z), so a
-// tile's loads never overwrite the plane that the previous tile's cells are
-// still reading, and no barrier is needed before them.
-template <typename T, int TX, int TY, int DIM, int PX, int PY, bool NC>
+// The TX x TY column at (x0, y0), z planes [z0, z1): writes the completed
+// cells to A.Uo and folds them into `acc`.  All threads of the block call it.
+template <typename T, int TX, int TY, int PX, int PY>
 __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, unsigned char* smem_raw, int x0,
-                                           int y0, int z0, int z1, TileAcc<T>& acc,
-                                           int tile = 0) {
-    using S = StageSmem<T, TX, TY, DIM>;
+                                           int y0, int z0, int z1, TileAcc<T>& acc) {
+    using S = StageSmem<T, TX, TY>;
     constexpr int NT = TX * TY;
     constexpr int HX = S::HX, HY = S::HY;
     T* Ps2 = reinterpret_cast<T*>(smem_raw);         // 2 x [NF][HY][HX]
@@ -205,7 +192,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, unsigned char*
     const int tid = threadIdx.x;
     const int tx = tid % TX, ty = tid / TX;
     const int x = x0 + tx, y = y0 + ty;
-    const bool own = x < A.n[0] && (DIM < 2 || y < A.n[1]);
+    const bool own = x < A.n[0] && y < A.n[1];
     const T dt = (T)(A.dt_dev ? *A.dt_dev : A.dt);
     const T gamma = A.gamma, gm1 = A.gm1, igm1 = A.igm1;
     bool bad = false;
@@ -218,21 +205,20 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, unsigned char*
         qm1[f] = dprev[f] = qLp[f] = Fzp[f] = Da[f] = Db[f] = T(0);
     }
 
-    const int jbeg = DIM == 3 ? z0 - 2 : 0;
-    const int jend = DIM == 3 ? z1 + 2 : 1;
-    for (int j = jbeg; j < jend; ++j) {
-        const bool xy = DIM < 3 || (j >= z0 && j < z1);
+    const int jbeg = z0 - 2;
+    for (int j = jbeg; j < z1 + 2; ++j) {
+        const bool xy = j >= z0 && j < z1;
         T qj[NF];
         T Dj[NF];
-        T* Ps = Ps2 + (((DIM == 3 ? j : tile) & 1) * S::NP);
+        T* Ps = Ps2 + (j & 1) * S::NP;
         if (xy) {
-            // Ps of the previous plane (tile) stays untouched; the fluxes are
+            // Ps of the previous plane stays untouched; the fluxes are
             // written after the next barrier, which no thread passes before
             // every thread has finished reading the previous ones
             for (int e = tid; e < HX * HY; e += NT) {
                 int hx = e % HX, hy = e / HX;
                 T W[NF];
-                load_prim<T, DIM, PX, PY, NC>(A, x0 - 2 + hx, y0 - 2 + hy, j, W, bad);
+                load_prim<T, PX, PY>(A, x0 - 2 + hx, y0 - 2 + hy, j, W, bad);
 #pragma unroll
                 for (int f = 0; f < NF; ++f) Ps[(f * HY + hy) * HX + hx] = W[f];
             }
@@ -240,88 +226,72 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, unsigned char*
             // x faces: (TX+1) per row; face fx sits left of tile cell fx
             for (int e = tid; e < (TX + 1) * TY; e += NT) {
                 int fx = e % (TX + 1), row = e / (TX + 1);
-                int hy = DIM >= 2 ? row + 2 : 0;
                 T q[4][NF];
 #pragma unroll
                 for (int s = 0; s < 4; ++s)
 #pragma unroll
-                    for (int f = 0; f < NF; ++f) q[s][f] = Ps[(f * HY + hy) * HX + fx + s];
+                    for (int f = 0; f < NF; ++f) q[s][f] = Ps[(f * HY + row + 2) * HX + fx + s];
                 T F[NF];
                 face_flux4<PX>(q[0], q[1], q[2], q[3], gamma, gm1, igm1, F);
 #pragma unroll
                 for (int f = 0; f < NF; ++f) Fx[(f * TY + row) * (TX + 1) + fx] = F[f];
             }
-            if (DIM >= 2) {
-                for (int e = tid; e < TX * (TY + 1); e += NT) {
-                    int col = e % TX, fy = e / TX;
-                    T q[4][NF];
+            for (int e = tid; e < TX * (TY + 1); e += NT) {
+                int col = e % TX, fy = e / TX;
+                T q[4][NF];
 #pragma unroll
-                    for (int s = 0; s < 4; ++s)
+                for (int s = 0; s < 4; ++s)
 #pragma unroll
-                        for (int f = 0; f < NF; ++f) q[s][f] = Ps[(f * HY + fy + s) * HX + col + 2];
-                    T F[NF];
-                    face_flux4<PY>(q[0], q[1], q[2], q[3], gamma, gm1, igm1, F);
+                    for (int f = 0; f < NF; ++f) q[s][f] = Ps[(f * HY + fy + s) * HX + col + 2];
+                T F[NF];
+                face_flux4<PY>(q[0], q[1], q[2], q[3], gamma, gm1, igm1, F);
 #pragma unroll
-                    for (int f = 0; f < NF; ++f) Fy[(f * (TY + 1) + fy) * TX + col] = F[f];
-                }
+                for (int f = 0; f < NF; ++f) Fy[(f * (TY + 1) + fy) * TX + col] = F[f];
             }
             __syncthreads();
-            const int hyc = DIM >= 2 ? ty + 2 : 0;
 #pragma unroll
             for (int f = 0; f < NF; ++f) {
-                qj[f] = Ps[(f * HY + hyc) * HX + tx + 2];
+                qj[f] = Ps[(f * HY + ty + 2) * HX + tx + 2];
                 T a = Fx[(f * TY + ty) * (TX + 1) + tx + 1] - Fx[(f * TY + ty) * (TX + 1) + tx];
                 Dj[f] = sub_over_dx(T(0), a, A.dxk[0]);
-                if (DIM >= 2) {
-                    T b = Fy[(f * (TY + 1) + ty + 1) * TX + tx] - Fy[(f * (TY + 1) + ty) * TX + tx];
-                    Dj[f] = sub_over_dx(Dj[f], b, A.dxk[1]);
-                }
+                T b = Fy[(f * (TY + 1) + ty + 1) * TX + tx] - Fy[(f * (TY + 1) + ty) * TX + tx];
+                Dj[f] = sub_over_dx(Dj[f], b, A.dxk[1]);
             }
         } else {
             // warm-up / look-ahead plane: only this column's primitives
-            load_prim<T, DIM, PX, PY, NC>(A, min(x, A.n[0] - 1), min(y, A.n[1] - 1), j, qj, bad);
+            load_prim<T, PX, PY>(A, min(x, A.n[0] - 1), min(y, A.n[1] - 1), j, qj, bad);
 #pragma unroll
             for (int f = 0; f < NF; ++f) Dj[f] = T(0);
         }
 
-        int k;                 // cell completed in this iteration (-1: none)
-        T L[NF];
-        if (DIM == 3) {
-            const int cnt = j - jbeg;
-            T dcur[NF], Fz[NF];
-            if (cnt >= 2) {
-                T qL[NF], qR[NF];
+        const int cnt = j - jbeg;
+        T dcur[NF], Fz[NF], L[NF];
 #pragma unroll
-                for (int f = 0; f < NF; ++f) {
-                    dcur[f] = qj[f] - qm1[f];
-                    T d = minmod(dprev[f], dcur[f]);
-                    qR[f] = sub_half(qm1[f], d);
-                    qL[f] = add_half(qm1[f], d);
-                }
-                if (cnt >= 3) hllc_axis<2>(qLp, qR, gamma, gm1, igm1, Fz);   // face j-3/2
-#pragma unroll
-                for (int f = 0; f < NF; ++f) qLp[f] = qL[f];
-            } else {
-#pragma unroll
-                for (int f = 0; f < NF; ++f) dcur[f] = qj[f] - qm1[f];
-            }
-            k = cnt >= 4 ? j - 2 : -1;
-            if (k >= 0) {
-#pragma unroll
-                for (int f = 0; f < NF; ++f) L[f] = sub_over_dx(Da[f], Fz[f] - Fzp[f], A.dxk[2]);
-            }
+        for (int f = 0; f < NF; ++f) dcur[f] = qj[f] - qm1[f];
+        if (cnt >= 2) {
+            T qL[NF], qR[NF];
 #pragma unroll
             for (int f = 0; f < NF; ++f) {
-                if (cnt >= 3) Fzp[f] = Fz[f];
-                dprev[f] = dcur[f];
-                qm1[f] = qj[f];
-                Da[f] = Db[f];
-                Db[f] = Dj[f];
+                T d = minmod(dprev[f], dcur[f]);
+                qR[f] = sub_half(qm1[f], d);
+                qL[f] = add_half(qm1[f], d);
             }
-        } else {
-            k = 0;
+            if (cnt >= 3) hllc_axis<2>(qLp, qR, gamma, gm1, igm1, Fz);   // face j-3/2
 #pragma unroll
-            for (int f = 0; f < NF; ++f) L[f] = Dj[f];
+            for (int f = 0; f < NF; ++f) qLp[f] = qL[f];
+        }
+        const int k = cnt >= 4 ? j - 2 : -1;                             // the cell completed
+        if (k >= 0) {
+#pragma unroll
+            for (int f = 0; f < NF; ++f) L[f] = sub_over_dx(Da[f], Fz[f] - Fzp[f], A.dxk[2]);
+        }
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+            if (cnt >= 3) Fzp[f] = Fz[f];
+            dprev[f] = dcur[f];
+            qm1[f] = qj[f];
+            Da[f] = Db[f];
+            Db[f] = Dj[f];
         }
 
         if (k >= 0 && own) {
@@ -355,7 +325,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, unsigned char*
     acc.bad |= bad;
 }
 
-template <typename T, int TX, int TY, int DIM, int PX, int PY, bool TMA>
+template <typename T, int TX, int TY, int PX, int PY>
 __global__ void __launch_bounds__(TX * TY)
 stage_kernel(const StageArgs<T> A) {
     constexpr int NT = TX * TY;
@@ -364,15 +334,15 @@ stage_kernel(const StageArgs<T> A) {
     __shared__ unsigned long long red_rate[NT / 32];
     const int tid = threadIdx.x;
     const int x0 = blockIdx.x * TX;
-    const int y0 = DIM >= 2 ? blockIdx.y * TY : 0;
-    const int z0 = DIM == 3 ? A.zlo + blockIdx.z * A.zchunk : 0;
-    const int z1 = DIM == 3 ? min(z0 + A.zchunk, A.zhi) : 1;
+    const int y0 = blockIdx.y * TY;
+    const int z0 = A.zlo + blockIdx.z * A.zchunk;
+    const int z1 = min(z0 + A.zchunk, A.zhi);
     TileAcc<T> acc;
     acc.rate_max = T(0);
     acc.bad = false;
 #pragma unroll
     for (int f = 0; f < NF; ++f) acc.tot[f] = T(0);
-    stage_tile<T, TX, TY, DIM, PX, PY, true>(A, smem_raw, x0, y0, z0, z1, acc);
+    stage_tile<T, TX, TY, PX, PY>(A, smem_raw, x0, y0, z0, z1, acc);
     const T rate_max = acc.rate_max;
     const bool bad = acc.bad;
     T tot[NF];
@@ -407,7 +377,7 @@ stage_kernel(const StageArgs<T> A) {
         }
     }
     if (A.tot_partial && tid < NF) {
-        const long long bz = DIM == 3 ? A.zlo / A.zchunk + blockIdx.z : blockIdx.z;
+        const long long bz = A.zlo / A.zchunk + blockIdx.z;
         const long long blk = (bz * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
         double s = 0.0;
         for (int w = 0; w < NT / 32; ++w) s += red_tot[w][tid];

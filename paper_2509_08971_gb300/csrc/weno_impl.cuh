@@ -48,9 +48,8 @@ StageArgs<T> weno_args(const MeshDesc& m, int zchunk, const StageCall& c) {
 
 template <int TX, int TY, int DIM, int PX, int PY>
 cudaError_t run_weno(const MeshDesc& m, const StageCall& c, cudaStream_t s) {
-    const TileDesc td = tile_desc(DIM, 0);
     static_assert(DIM < 2 || TY > 1, "2D/3D tiles have rows");
-    const StageArgs<T> A = weno_args(m, td.zc, c);
+    const StageArgs<T> A = weno_args(m, WENO_ZC, c);
     const dim3 grid(wcdiv(m.n[0], TX), DIM >= 2 ? wcdiv(m.n[1], TY) : 1,
                     DIM == 3 ? wcdiv(m.n[2], A.zchunk) : 1);
     constexpr size_t smem = WenoSmem<T, TX, TY, DIM>::bytes;
@@ -130,43 +129,39 @@ cudaError_t HH_WCAT(launch_advect_E_stage_, HH_SUFFIX)(const MeshDesc& m, int st
     }
     A.dt = dt;
     A.stage = stage;
-    A.zchunk = tile_desc(3, 0).zc;
+    A.zchunk = WENO_ZC;
     if (m.dim == 3 && scratch) {
         A.zchunk = WENO_SWEEP_CHUNK;
         return run_advect_sweeps(m, A, static_cast<T*>(scratch), s);
     }
-    if (m.dim == 3) return run_advect<32, 8, 3, 0, 1>(m, A, s);
+    if (m.dim == 3) return run_advect<WENO_TX2, WENO_TY2, 3, 0, 1>(m, A, s);
     if (m.dim == 2) {
-        if (m.px == 0 && m.py == 1) return run_advect<32, 8, 2, 0, 1>(m, A, s);
-        if (m.px == 0 && m.py == 2) return run_advect<32, 8, 2, 0, 2>(m, A, s);
-        return run_advect<32, 8, 2, 1, 2>(m, A, s);
+        if (m.px == 0 && m.py == 1) return run_advect<WENO_TX2, WENO_TY2, 2, 0, 1>(m, A, s);
+        if (m.px == 0 && m.py == 2) return run_advect<WENO_TX2, WENO_TY2, 2, 0, 2>(m, A, s);
+        return run_advect<WENO_TX2, WENO_TY2, 2, 1, 2>(m, A, s);
     }
     if (m.dim == 1) {
-        if (m.px == 0) return run_advect<128, 1, 1, 0, 0>(m, A, s);
-        if (m.px == 1) return run_advect<128, 1, 1, 1, 0>(m, A, s);
-        return run_advect<128, 1, 1, 2, 0>(m, A, s);
+        if (m.px == 0) return run_advect<WENO_TX1, 1, 1, 0, 0>(m, A, s);
+        if (m.px == 1) return run_advect<WENO_TX1, 1, 1, 1, 0>(m, A, s);
+        return run_advect<WENO_TX1, 1, 1, 2, 0>(m, A, s);
     }
     return cudaErrorInvalidValue;
 }
 
 cudaError_t HH_WCAT(launch_weno_stage_, HH_SUFFIX)(const MeshDesc& m, const StageCall& c,
                                                    cudaStream_t s) {
-    // the tile of each dimension is entry 0 of its table: 32 x 8 (z-chunk 32), 32 x 8, 128 x 1
-    static_assert(TILES3[0].tx == 32 && TILES3[0].ty == 8 && TILES2[0].tx == 32 &&
-                      TILES2[0].ty == 8 && TILES1[0].tx == 128,
-                  "the WENO launcher runs tile 0 of each table");
     for (int a = 0; a < 3; ++a)
         if (m.n[a] > 1 && m.n[a] < WENO_G) return cudaErrorInvalidValue;
-    if (m.dim == 3) return c.scratch ? run_weno_sweeps(m, c, s) : run_weno<32, 8, 3, 0, 1>(m, c, s);
+    if (m.dim == 3) return c.scratch ? run_weno_sweeps(m, c, s) : run_weno<WENO_TX2, WENO_TY2, 3, 0, 1>(m, c, s);
     if (m.dim == 2) {
-        if (m.px == 0 && m.py == 1) return run_weno<32, 8, 2, 0, 1>(m, c, s);
-        if (m.px == 0 && m.py == 2) return run_weno<32, 8, 2, 0, 2>(m, c, s);
-        return run_weno<32, 8, 2, 1, 2>(m, c, s);
+        if (m.px == 0 && m.py == 1) return run_weno<WENO_TX2, WENO_TY2, 2, 0, 1>(m, c, s);
+        if (m.px == 0 && m.py == 2) return run_weno<WENO_TX2, WENO_TY2, 2, 0, 2>(m, c, s);
+        return run_weno<WENO_TX2, WENO_TY2, 2, 1, 2>(m, c, s);
     }
     if (m.dim == 1) {
-        if (m.px == 0) return run_weno<128, 1, 1, 0, 0>(m, c, s);
-        if (m.px == 1) return run_weno<128, 1, 1, 1, 0>(m, c, s);
-        return run_weno<128, 1, 1, 2, 0>(m, c, s);
+        if (m.px == 0) return run_weno<WENO_TX1, 1, 1, 0, 0>(m, c, s);
+        if (m.px == 1) return run_weno<WENO_TX1, 1, 1, 1, 0>(m, c, s);
+        return run_weno<WENO_TX1, 1, 1, 2, 0>(m, c, s);
     }
     return cudaErrorInvalidValue;               // no active axis: the PLM launcher handles it
 }

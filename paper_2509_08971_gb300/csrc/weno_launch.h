@@ -11,6 +11,9 @@ namespace hh {
 #ifndef HH_WENO_CHUNK
 #define HH_WENO_CHUNK 64
 #endif
+// Tiles of the fused kernel: 128 cells in 1D, 32 x 8 in 2D and 3D, 32-plane
+// z chunks.
+inline constexpr int WENO_TX1 = 128, WENO_TX2 = 32, WENO_TY2 = 8, WENO_ZC = 32;
 inline constexpr int WENO_SWEEP_THREADS = 128;
 inline constexpr int WENO_SWEEP_CHUNK = HH_WENO_CHUNK;
 
@@ -23,7 +26,9 @@ inline long long weno_stage_blocks(const MeshDesc& m, bool sweeps) {
         const long long bz = (m.n[2] + WENO_SWEEP_CHUNK - 1) / WENO_SWEEP_CHUNK;
         return bx * m.n[1] * bz;
     }
-    return stage_blocks(m, 0);
+    return (long long)((m.n[0] + (m.dim == 1 ? WENO_TX1 : WENO_TX2) - 1) / (m.dim == 1 ? WENO_TX1 : WENO_TX2)) *
+           (m.dim >= 2 ? (m.n[1] + WENO_TY2 - 1) / WENO_TY2 : 1) *
+           (m.dim == 3 ? (m.n[2] + WENO_ZC - 1) / WENO_ZC : 1);
 }
 
 // One stage of the second scheme on the mesh: on a 3D mesh with c.scratch
