@@ -437,7 +437,7 @@ int hard_hydro_tile_info(hard_hydro_t h, int tile, int out4[4]) {
     out4[0] = t.tx;
     out4[1] = t.ty;
     out4[2] = t.zc;
-    out4[3] = hh::tile_threads(h->mesh.dim, tile);
+    out4[3] = t.tx * t.ty;
     return HARD_OK;
 }
 

@@ -71,13 +71,12 @@ cudaError_t run_stage(const MeshDesc& m, const TileDesc& td, const StageCall& c,
     return cudaGetLastError();
 }
 
-// 1D and 2D meshes: one warp per strip and td.ty rows (strip.cuh).
+// 1D and 2D meshes: one warp per strip and td.zc rows (strip.cuh).
 template <int DIM, int PX, int PY, int RR, int NWARP>
 cudaError_t run_strip(const MeshDesc& m, const TileDesc& td, const StageCall& c, cudaStream_t s) {
     static_assert(STRIP == STRIP_CELLS, "the launch rule counts the kernel's strips");
-    StageArgs<T> A = make_args(m, td, c);
-    A.zchunk = td.ty;                                   // rows per warp
-    const long long strips = cdiv(m.n[0], STRIP), warps = strips * cdiv(m.n[1], td.ty);
+    const StageArgs<T> A = make_args(m, td, c);         // A.zchunk: rows per warp
+    const long long strips = cdiv(m.n[0], STRIP), warps = strips * cdiv(m.n[1], td.zc);
     const long long blocks = cdiv<long long>(warps, NWARP);
     if (blocks >= (1ll << 31)) return cudaErrorInvalidValue;
     strip_kernel<T, DIM, PX, PY, RR, NWARP><<<(unsigned)blocks, 32 * NWARP, 0, s>>>(A);
@@ -378,13 +377,13 @@ cudaError_t dispatch_tile(const MeshDesc& m, int kernel, int tile, const StageCa
             default: return run_stage<32, 4>(m, td, c, s);
         }
     } else if constexpr (DIM == 2) {
-        switch (td.ty) {
+        switch (td.zc) {
             case 2: return run_strip<2, PX, PY, 2, 2>(m, td, c, s);
             case 4: return run_strip<2, PX, PY, 4, 2>(m, td, c, s);
             default: return run_strip<2, PX, PY, 0, 2>(m, td, c, s);
         }
     } else {
-        if (td.tx == STRIP) return run_strip<1, PX, 0, 1, 1>(m, td, c, s);
+        if (td.ty == 1) return run_strip<1, PX, 0, 1, 1>(m, td, c, s);
         return run_strip<1, PX, 0, 1, 4>(m, td, c, s);
     }
 }

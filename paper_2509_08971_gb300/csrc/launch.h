@@ -45,10 +45,10 @@ struct StageCall {
 // Tile configurations per number of active axes (the autotuner's space).
 inline constexpr TileDesc TILES3[] = {{32, 8, 32}, {32, 8, 64}, {32, 16, 64}, {64, 8, 64},
                                       {32, 4, 64}, {32, 16, 32}};
-// 1D and 2D meshes run one warp per strip (strip.cuh): ty rows per warp, tx / 28
-// warps per block.
-inline constexpr TileDesc TILES2[] = {{56, 2, 0}, {56, 4, 0}, {56, 16, 0}};
-inline constexpr TileDesc TILES1[] = {{28, 1, 0}, {112, 1, 0}};
+// 1D and 2D meshes run one warp per strip of 28 cells (strip.cuh): 32 lanes, ty
+// warps per block, zc rows per warp.
+inline constexpr TileDesc TILES2[] = {{32, 2, 2}, {32, 2, 4}, {32, 2, 16}};
+inline constexpr TileDesc TILES1[] = {{32, 1, 1}, {32, 4, 1}};
 inline constexpr int STRIP_CELLS = 28;
 
 inline int tile_count(int dim) {
@@ -59,10 +59,6 @@ inline TileDesc tile_desc(int dim, int tile) {
     if (dim == 2) return TILES2[tile];
     if (dim == 1) return TILES1[tile];
     return TileDesc{256, 1, 0};
-}
-inline int tile_threads(int dim, int tile) {
-    const TileDesc t = tile_desc(dim, tile);
-    return dim == 1 || dim == 2 ? t.tx / STRIP_CELLS * 32 : t.tx * t.ty;
 }
 // The tile a launch uses: the table's entry, or for tile < 0 the library's
 // choice.  2D: rows per warp.  A warp of two rows pays ~1.3x (FP32) / 1.4x
@@ -84,9 +80,8 @@ inline long long stage_blocks(const MeshDesc& m, int tile, bool f64) {
     const TileDesc t = launch_tile(m, tile, f64);
     if (m.dim < 3) {
         const long long strips = (m.n[0] + STRIP_CELLS - 1) / STRIP_CELLS;
-        const long long warps = strips * ((m.n[1] + t.ty - 1) / t.ty);
-        const int per = t.tx / STRIP_CELLS;
-        return (warps + per - 1) / per;
+        const long long warps = strips * ((m.n[1] + t.zc - 1) / t.zc);
+        return (warps + t.ty - 1) / t.ty;
     }
     const long long gx = (m.n[0] + t.tx - 1) / t.tx;
     const long long gy = (m.n[1] + t.ty - 1) / t.ty;
