@@ -225,47 +225,61 @@ template <int TY> struct WsConf {
     static constexpr int RPW = TY == 8 ? HH_WS_RPW8 : 1;
 };
 
-template <int TY>
+template <int TY, bool TMA>
 cudaError_t run_stage_ws(const MeshDesc& m, const TileDesc& td, const StageCall& c,
                          cudaStream_t s, bool& used) {
     constexpr int NCW = WsConf<TY>::NCW, RPW = WsConf<TY>::RPW;
-    using L1 = WsLayout<32, TY, NCW, 1, RPW>;
-    using L2 = WsLayout<32, TY, NCW, 2, RPW>;
+    using L1 = WsLayout<32, TY, NCW, 1, RPW, TMA>;
+    using L2 = WsLayout<32, TY, NCW, 2, RPW, TMA>;
     used = false;
     if constexpr (L2::bytes > SMEM_LIMIT) {
         return cudaSuccess;
     } else {
-        if ((reinterpret_cast<uintptr_t>(c.Uo) & 15u) != 0 ||
-            (c.stage == 2 && (reinterpret_cast<uintptr_t>(c.U0) & 15u) != 0))
-            return cudaSuccess;
         WsMaps maps;
-        if (!encode_state_map(&maps.main, c.Uc, m, L1::HXC, L1::HYC) ||
-            !encode_state_map(&maps.xstrip, c.Uc, m, 4, L1::HYC) ||
-            !encode_state_map(&maps.ystrip, c.Uc, m, L1::HXC, 2) ||
-            !encode_state_map(&maps.u0, c.stage == 2 ? c.U0 : c.Uc, m, 32, TY) ||
-            !encode_state_map(&maps.out, c.Uo, m, 32, TY) ||
-            !encode_ghost_maps(maps, m, c, L1::HXC, L1::HYC))
-            return cudaSuccess;
+        if constexpr (TMA) {
+            if ((reinterpret_cast<uintptr_t>(c.Uo) & 15u) != 0 ||
+                (c.stage == 2 && (reinterpret_cast<uintptr_t>(c.U0) & 15u) != 0))
+                return cudaSuccess;
+            if (!encode_state_map(&maps.main, c.Uc, m, L1::HXC, L1::HYC) ||
+                !encode_state_map(&maps.xstrip, c.Uc, m, 4, L1::HYC) ||
+                !encode_state_map(&maps.ystrip, c.Uc, m, L1::HXC, 2) ||
+                !encode_state_map(&maps.u0, c.stage == 2 ? c.U0 : c.Uc, m, 32, TY) ||
+                !encode_state_map(&maps.out, c.Uo, m, 32, TY) ||
+                !encode_ghost_maps(maps, m, c, L1::HXC, L1::HYC))
+                return cudaSuccess;
+        } else {
+            std::memset(&maps, 0, sizeof(maps));
+        }
         StageArgs<T> A = make_args(m, td, c);
         // failure-path test: HARD_HYDRO_STARVE_TMA=1 makes the ring's waits
         // run out (the stage then reports HARD_ETIMEOUT and leaves Uout unset)
         const char* starve = std::getenv("HARD_HYDRO_STARVE_TMA");
-        A.starve_tma = starve && starve[0] == '1';
+        A.starve_tma = TMA && starve && starve[0] == '1';
         dim3 grid(cdiv(m.n[0], 32), cdiv(m.n[1], TY), cdiv(A.zhi - A.zlo, A.zchunk));
         static std::atomic<unsigned long long> attr1{0}, attr2{0};
         cudaError_t e;
         if (c.stage == 1) {
-            e = smem_attr_once(stage_ws_kernel<32, TY, NCW, 1, RPW>, L1::bytes, attr1);
+            e = smem_attr_once(stage_ws_kernel<32, TY, NCW, 1, RPW, TMA>, L1::bytes, attr1);
             if (e != cudaSuccess) return e;
-            stage_ws_kernel<32, TY, NCW, 1, RPW><<<grid, L1::NT, L1::bytes, s>>>(A, maps);
+            stage_ws_kernel<32, TY, NCW, 1, RPW, TMA><<<grid, L1::NT, L1::bytes, s>>>(A, maps);
         } else {
-            e = smem_attr_once(stage_ws_kernel<32, TY, NCW, 2, RPW>, L2::bytes, attr2);
+            e = smem_attr_once(stage_ws_kernel<32, TY, NCW, 2, RPW, TMA>, L2::bytes, attr2);
             if (e != cudaSuccess) return e;
-            stage_ws_kernel<32, TY, NCW, 2, RPW><<<grid, L2::NT, L2::bytes, s>>>(A, maps);
+            stage_ws_kernel<32, TY, NCW, 2, RPW, TMA><<<grid, L2::NT, L2::bytes, s>>>(A, maps);
         }
         used = true;
         return cudaGetLastError();
     }
+}
+// TMA where the mesh allows it; other meshes whose planes have 32-bit offsets
+// take 4-byte copies into the same ring.
+template <int TY>
+cudaError_t run_ws_loads(const MeshDesc& m, const TileDesc& td, const StageCall& c, cudaStream_t s,
+                         bool tma, bool& used) {
+    cudaError_t e = tma ? run_stage_ws<TY, true>(m, td, c, s, used) : cudaSuccess;
+    if (e == cudaSuccess && !used && (long long)m.n[0] * m.n[1] < (1ll << 31))
+        e = run_stage_ws<TY, false>(m, td, c, s, used);
+    return e;
 }
 #endif
 
@@ -347,35 +361,32 @@ cudaError_t dispatch_tile(const MeshDesc& m, int kernel, int tile, const StageCa
                           cudaStream_t s) {
     const TileDesc td = launch_tile(m, tile, sizeof(T) == 8);
     if constexpr (DIM == 3) {
-        if (tile < 0) tile = 0;
         // the TMA kernel carries the rate / totals epilogue for stage 2 only
         const bool epi_ok = c.stage == 2 || (!c.rate_slot && !c.tot_partial);
-        if (kernel == 0 && epi_ok && tma_eligible(m, c.Uc)) {
+        if (kernel == 0 && epi_ok) {
             bool used = false;
-            cudaError_t e;
+            cudaError_t e = cudaSuccess;
+            const bool tma = tma_eligible(m, c.Uc);
 #ifdef HH_WS
-            switch (tile) {
-                case 0: case 1: e = run_stage_ws<8>(m, td, c, s, used); break;
-                case 2: case 5: e = run_stage_ws<16>(m, td, c, s, used); break;
-                case 3: e = cudaSuccess; break;            // 64-wide tiles: no warp-per-row form
-                default: e = run_stage_ws<4>(m, td, c, s, used); break;
+            if (td.tx == 32) {                 // 64-wide tiles have no warp-per-row form
+                if (td.ty == 16) e = run_ws_loads<16>(m, td, c, s, tma, used);
+                else if (td.ty == 8) e = run_ws_loads<8>(m, td, c, s, tma, used);
+                else e = run_ws_loads<4>(m, td, c, s, tma, used);
             }
 #else
-            switch (tile) {
-                case 0: case 1: e = run_stage_tma<32, 8>(m, td, c, s, used); break;
-                case 2: case 5: e = run_stage_tma<32, 16>(m, td, c, s, used); break;
-                case 3: e = run_stage_tma<64, 8>(m, td, c, s, used); break;
-                default: e = run_stage_tma<32, 4>(m, td, c, s, used); break;
+            if (tma) {
+                if (td.tx == 64) e = run_stage_tma<64, 8>(m, td, c, s, used);
+                else if (td.ty == 16) e = run_stage_tma<32, 16>(m, td, c, s, used);
+                else if (td.ty == 8) e = run_stage_tma<32, 8>(m, td, c, s, used);
+                else e = run_stage_tma<32, 4>(m, td, c, s, used);
             }
 #endif
             if (used || e != cudaSuccess) return e;
         }
-        switch (tile) {
-            case 0: case 1: return run_stage<32, 8>(m, td, c, s);
-            case 2: case 5: return run_stage<32, 16>(m, td, c, s);
-            case 3: return run_stage<64, 8>(m, td, c, s);
-            default: return run_stage<32, 4>(m, td, c, s);
-        }
+        if (td.tx == 64) return run_stage<64, 8>(m, td, c, s);
+        if (td.ty == 16) return run_stage<32, 16>(m, td, c, s);
+        if (td.ty == 8) return run_stage<32, 8>(m, td, c, s);
+        return run_stage<32, 4>(m, td, c, s);
     } else if constexpr (DIM == 2) {
         switch (td.zc) {
             case 2: return run_strip<2, PX, PY, 2, 2>(m, td, c, s);

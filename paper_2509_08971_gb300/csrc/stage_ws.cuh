@@ -29,6 +29,15 @@
 // x/y ghosts of boundary tiles come as narrow strip boxes on the same
 // mbarrier.  The conserved value of a cell, needed by the RK combine, is read
 // back from the ring; stage 2's U^n plane arrives by TMA on the same barrier.
+//
+// TMA = false: meshes that bulk tensor loads cannot address (rows that are no
+// multiple of 16 bytes).  Each thread copies its cells of the plane into the
+// same ring with 4-byte cp.async, every ghost cell already through the
+// boundary map, and arrives on the slot's mbarrier when they have landed;
+// U^n is read into registers at the head of the iteration and results are
+// stored from registers.  150 x 117 x 93, 32 x 8 x 32 tiles: 128 us a stage in
+// the block-synchronous kernel that these meshes took (stage_kernel), 79 us
+// here; 152 cells a row by TMA 66 us (the copies and stores are issue slots).
 #pragma once
 #include "stage_kernel.cuh"
 #include "stage_tma.cuh"
@@ -47,11 +56,12 @@ struct WsMaps {
     CUtensorMap gmain[2], gxstrip[2], gystrip[2];
 };
 
-template <int TX, int TY, int NCW, int STAGE, int RPW>
+template <int TX, int TY, int NCW, int STAGE, int RPW, bool TMA>
 struct WsLayout {
     static_assert(TX == 32, "lane = x in the face warps");
     static_assert(2 * TY <= 32, "one converter lane per x edge face");
     static_assert(TY % RPW == 0, "whole tile rows per face warp");
+    static constexpr bool TMA_LOADS = TMA;
     static constexpr int NFW = TY / RPW;                // face warps, RPW tile rows each
     static constexpr int NW = NFW + NCW;
     static constexpr int NT = 32 * NW;
@@ -64,15 +74,15 @@ struct WsLayout {
     static constexpr int XS = pad32(NF * HYC * 4);      // x strip box
     static constexpr int YS = pad32(NF * 2 * HXC);      // y strip box
     static constexpr int XLO = 0, XHI = XS, YLO = 2 * XS, YHI = 2 * XS + YS;
-    static constexpr int STRIP = 2 * XS + 2 * YS;
+    static constexpr int STRIP = TMA ? 2 * XS + 2 * YS : 0;
     static constexpr int U0S = pad32(NF * TY * TX);
-    static constexpr int NU0 = STAGE == 2 ? 2 : 0;
+    static constexpr int NU0 = TMA && STAGE == 2 ? 2 : 0;
     static constexpr int PQ = pad32(5 * NPC);           // float4 part, then p
     static constexpr int FYR = TY + 1;                  // y-face rows
     static constexpr int FQ = pad32(5 * FYR * TX);      // float4 part, then the energy flux
     static constexpr int FXR = TX + 1;                  // x faces per tile row
     static constexpr int FX = pad32(5 * TY * FXR);      // x-face fluxes: float4 part, then energy
-    static constexpr int OST = pad32(NF * TY * TX);     // output plane staged for the TMA store
+    static constexpr int OST = TMA ? pad32(NF * TY * TX) : 0;   // output plane staged for the TMA store
     // offsets in floats from the end of the barrier block
     static constexpr int O_STRIP = D * MAIN;
     static constexpr int O_U0 = O_STRIP + 2 * STRIP;
@@ -81,7 +91,9 @@ struct WsLayout {
     static constexpr int O_FX = O_FY + 2 * FQ;
     static constexpr int O_OST = O_FX + 2 * FX;
     static constexpr int O_MAP = O_OST + 2 * OST;       // halo conversion map (ints)
-    static constexpr int O_END = O_MAP + pad32(4 * TX + 4 * TY);
+    static constexpr int O_SRC = O_MAP + pad32(4 * TX + 4 * TY);
+    // copies without TMA: source offset of each cell of the halo ring
+    static constexpr int O_END = O_SRC + (TMA ? 0 : pad32(4 * TX + 4 * TY));
     static constexpr size_t BAR_BYTES = 128;            // D mbarriers, abort flags
     static constexpr size_t RED_BYTES = (size_t)NFW * (NF + 1) * 8;
     static constexpr size_t data_bytes = BAR_BYTES + 4 * (size_t)O_END + RED_BYTES;
@@ -117,17 +129,23 @@ __device__ __forceinline__ void halo_cell(int e, int& cx, int& cy) {
 // slot: bits 0-15 the offset of field 0 (0xFFFF: a cell no face reads),
 // bits 16-27 the field stride, bit 28 / bit 29 negate rho*u / rho*v
 // (reflecting walls), bit 30 set: the offset is into the strip block.
-template <int TX, int TY, int HXC, int HYC, int XLO, int XHI, int YLO, int YHI>
+template <class L>
 __device__ __forceinline__ int ws_source(int cx, int cy, int x0, int y0, int nx, int ny,
                                          const int* bc_lo, const int* bc_hi) {
+    constexpr int HXC = L::HXC, HYC = L::HYC;
     const int gx = x0 + cx, gy = y0 + cy;
     const bool gxo = gx < 0 || gx >= nx, gyo = gy < 0 || gy >= ny;
     int src = (cy + 2) * HXC + cx + 4, fs = HYC * HXC, flags = 0;
     if ((gxo && gyo) || gx > nx + 1 || gy > ny + 1) return 0xFFFF;   // corner / beyond a ragged edge
+    if (!L::TMA_LOADS) {                     // each cell was copied to its own place
+        const bool fx = gxo && (gx < 0 ? bc_lo[0] : bc_hi[0]) == 2;
+        const bool fy = gyo && (gy < 0 ? bc_lo[1] : bc_hi[1]) == 2;
+        return src | (fs << 16) | ((fx ? 1 : 0) | (fy ? 2 : 0)) << 28;
+    }
     if (gxo) {
         const int bc = gx < 0 ? bc_lo[0] : bc_hi[0];
         if (bc == 0) {
-            src = (gx < 0 ? XLO : XHI) + (cy + 2) * 4 + (gx < 0 ? gx + 4 : gx - nx);
+            src = (gx < 0 ? L::XLO : L::XHI) + (cy + 2) * 4 + (gx < 0 ? gx + 4 : gx - nx);
             fs = HYC * 4;
             flags = 4;
         } else if (bc == 1) {
@@ -139,7 +157,7 @@ __device__ __forceinline__ int ws_source(int cx, int cy, int x0, int y0, int nx,
     } else if (gyo) {
         const int bc = gy < 0 ? bc_lo[1] : bc_hi[1];
         if (bc == 0) {
-            src = (gy < 0 ? YLO : YHI) + (gy < 0 ? gy + 2 : gy - ny) * HXC + cx + 4;
+            src = (gy < 0 ? L::YLO : L::YHI) + (gy < 0 ? gy + 2 : gy - ny) * HXC + cx + 4;
             fs = 2 * HXC;
             flags = 4;
         } else if (bc == 1) {
@@ -203,10 +221,10 @@ __device__ __forceinline__ float ws_rate(const float U[NF], float gamma, float g
 // consecutive tile rows: with two, the y slope of a row is shared by the two
 // y faces around it and the iteration's control work is spread over two
 // cells per thread.
-template <int TX, int TY, int NCW, int STAGE, int RPW>
+template <int TX, int TY, int NCW, int STAGE, int RPW, bool TMA>
 __global__ void __launch_bounds__(32 * (TY / RPW + NCW), TY >= 16 ? 1 : (TY >= 8 ? 2 : 3))
 stage_ws_kernel(const __grid_constant__ StageArgs<float> A, const __grid_constant__ WsMaps M) {
-    using L = WsLayout<TX, TY, NCW, STAGE, RPW>;
+    using L = WsLayout<TX, TY, NCW, STAGE, RPW, TMA>;
     constexpr int D = L::D, HXC = L::HXC, HYC = L::HYC, HXP = L::HXP, NPC = L::NPC;
     constexpr int FYR = L::FYR, NCT = 32 * NCW, NFW = L::NFW;
     constexpr bool EPI = STAGE == 2;
@@ -228,6 +246,7 @@ stage_ws_kernel(const __grid_constant__ StageArgs<float> A, const __grid_constan
     float* Fxbase = sm + L::O_FX;
     float* Ost = sm + L::O_OST;
     int* hmap = reinterpret_cast<int*>(sm + L::O_MAP);
+    int* smap = reinterpret_cast<int*>(sm + L::O_SRC);
     double (*red_tot)[NF] = reinterpret_cast<double (*)[NF]>(sm + L::O_END);
     unsigned long long* red_rate =
         reinterpret_cast<unsigned long long*>(reinterpret_cast<double*>(red_tot) + L::NFW * NF);
@@ -251,6 +270,30 @@ stage_ws_kernel(const __grid_constant__ StageArgs<float> A, const __grid_constan
                               (py_hi ? L::YS_BYTES : 0);
     const int issuer = 32 * NFW;                        // lane 0 of the first converter warp
 
+    const long long plane = (long long)nx * ny;
+    const int yr0 = warp * RPW;                         // first tile row of a face warp
+    // the face warps' cells: tile row yr0 + r, column lane
+    bool own[RPW];
+#pragma unroll
+    for (int r = 0; r < RPW; ++r) own[r] = facew && x0 + lane < nx && y0 + yr0 + r < ny;
+    const unsigned gown = (unsigned)(y0 + yr0) * (unsigned)nx + (unsigned)(x0 + lane);   // row yr0 in a mesh plane (copies)
+    const int pown0 = (yr0 + 2) * HXP + lane + 2;       // row yr0 in a primitive plane
+    const int rown0 = (yr0 + 2) * HXC + lane + 4;       // row yr0 in a ring slot
+    // In-plane source of tile cell (cx, cy) through the x and y boundary maps
+    // (-1: a cell no face reads); of the own cells in registers.
+    auto plane_source = [&](int cx, int cy) {
+        const int gx = x0 + cx, gy = y0 + cy;
+        const bool gxo = gx < 0 || gx >= nx, gyo = gy < 0 || gy >= ny;
+        if ((gxo && gyo) || gx > nx + 1 || gy > ny + 1) return -1;
+        bool fl;
+        const int sy = bc_map(gy, ny, A.bc_lo[1], A.bc_hi[1], fl);
+        return sy * nx + bc_map(gx, nx, A.bc_lo[0], A.bc_hi[0], fl);
+    };
+    int osrc[TMA ? 1 : RPW];
+    if (!TMA)
+#pragma unroll
+        for (int r = 0; r < RPW; ++r) osrc[TMA ? 0 : r] = plane_source(lane, yr0 + r);
+
     // Ring plane of iteration index q (plane jbeg + q) with its strips; in
     // stage 2 also the U^n plane jbeg + q - 2 that the RK combine of
     // iteration q - 1 needs (it completes on the same barrier).
@@ -258,6 +301,34 @@ stage_ws_kernel(const __grid_constant__ StageArgs<float> A, const __grid_constan
         uint64_t* bar = bars + (q & (D - 1));
         bool fz;
         const int pz = jbeg + q;
+        if constexpr (!TMA) {
+            // every face lane copies its own cells, the converter lanes the
+            // halo ring (smap)
+            const bool lo = pz < 0 && A.bc_lo[2] == BC_HALO, hi = pz >= nz && A.bc_hi[2] == BC_HALO;
+            const long long fs = lo || hi ? 2 * plane : A.N;
+            const float* src = lo ? A.zg[0] + (pz + 2) * plane
+                             : hi ? A.zg[1] + (pz - nz) * plane
+                                  : A.Uc + bc_map(pz, nz, A.bc_lo[2], A.bc_hi[2], fz) * plane;
+            float* slot = ring + (q & (D - 1)) * L::MAIN;
+            auto copy = [&](float* dst, int o) {
+                if (o < 0) return;
+                const float* g = src + o;
+#pragma unroll
+                for (int f = 0; f < NF; ++f) cp_async_4(dst + f * (HYC * HXC), g + f * fs);
+            };
+            if (facew) {
+#pragma unroll
+                for (int r = 0; r < RPW; ++r) copy(slot + rown0 + r * HXC, osrc[r]);
+            } else {
+                for (int e = tid - 32 * NFW; e < L::NHALO; e += NCT) {
+                    int cx, cy;
+                    halo_cell<TX, TY>(e, cx, cy);
+                    copy(slot + (cy + 2) * HXC + cx + 4, smap[e]);
+                }
+            }
+            cp_async_arrive(bar);
+            return;
+        }
         const bool hlo = pz < 0 && A.bc_lo[2] == BC_HALO, hhi = pz >= nz && A.bc_hi[2] == BC_HALO;
         const int side = hlo ? 0 : 1;
         const int jj = hlo ? pz + 2 : (hhi ? pz - nz : bc_map(pz, nz, A.bc_lo[2], A.bc_hi[2], fz));
@@ -283,7 +354,6 @@ stage_ws_kernel(const __grid_constant__ StageArgs<float> A, const __grid_constan
     // conversion maps of edge tiles: the face warps' own cells in registers,
     // the halo ring in shared memory (written by the converter lanes, read
     // after the barrier); interior tiles read the main box at fixed offsets
-    const int yr0 = warp * RPW;                         // first tile row of a face warp
     int cv_own[RPW];
 #pragma unroll
     for (int r = 0; r < RPW; ++r) cv_own[r] = 0;
@@ -291,26 +361,32 @@ stage_ws_kernel(const __grid_constant__ StageArgs<float> A, const __grid_constan
         if (facew) {
 #pragma unroll
             for (int r = 0; r < RPW; ++r)
-                cv_own[r] = ws_source<TX, TY, HXC, HYC, L::XLO, L::XHI, L::YLO, L::YHI>(
-                    lane, yr0 + r, x0, y0, nx, ny, A.bc_lo, A.bc_hi);
+                cv_own[r] = ws_source<L>(lane, yr0 + r, x0, y0, nx, ny, A.bc_lo, A.bc_hi);
         } else {
             for (int e = tid - 32 * NFW; e < L::NHALO; e += NCT) {
                 int cx, cy;
                 halo_cell<TX, TY>(e, cx, cy);
-                hmap[e] = ws_source<TX, TY, HXC, HYC, L::XLO, L::XHI, L::YLO, L::YHI>(
-                    cx, cy, x0, y0, nx, ny, A.bc_lo, A.bc_hi);
+                hmap[e] = ws_source<L>(cx, cy, x0, y0, nx, ny, A.bc_lo, A.bc_hi);
             }
         }
     }
-    int issued = -1;                                    // last iteration index loaded (issuer)
+    if (!TMA && !facew)
+        for (int e = tid - 32 * NFW; e < L::NHALO; e += NCT) {
+            int cx, cy;
+            halo_cell<TX, TY>(e, cx, cy);
+            smap[e] = plane_source(cx, cy);
+        }
+    // who loads: one converter lane by TMA, or every thread by 4-byte copies
+    const bool loads = !TMA || tid == issuer;
+    int issued = -1;                                    // last iteration index loaded (loads)
     if (tid == issuer) {
-        for (int s = 0; s < D; ++s) mbar_init(bars + s, 1);
+        for (int s = 0; s < D; ++s) mbar_init(bars + s, TMA ? 1 : L::NT);
         mbar_fence_init();
         s_abort[0] = s_abort[1] = 0;
-        prefetch_tmap(&M.main);
+        if (TMA) prefetch_tmap(&M.main);
     }
     __syncthreads();
-    if (tid == issuer) {
+    if (loads) {
         issue(0);
         issue(1);                                       // niter >= 4: z1 > z0
         issued = 1;
@@ -319,13 +395,6 @@ stage_ws_kernel(const __grid_constant__ StageArgs<float> A, const __grid_constan
     const float gamma = A.gamma, gm1 = A.gm1, igm1 = A.igm1;
     const float idx = A.dxk[0], idy = A.dxk[1], idz = A.dxk[2];
     const float dt = (float)(A.dt_dev ? *A.dt_dev : A.dt);
-    // the face warps' cells: tile row yr0 + r, column lane
-    bool own[RPW];
-#pragma unroll
-    for (int r = 0; r < RPW; ++r) own[r] = facew && x0 + lane < nx && y0 + yr0 + r < ny;
-    const int pown0 = (yr0 + 2) * HXP + lane + 2;       // row yr0 in a primitive plane
-    const int rown0 = (yr0 + 2) * HXC + lane + 4;       // row yr0 in a ring slot
-
     // conserved -> primitive of the own cells of the plane of iteration index q
     auto convert_own = [&](int q, float (&W)[RPW][NF]) {
         const float* slot = ring + (q & (D - 1)) * L::MAIN;
@@ -365,7 +434,23 @@ stage_ws_kernel(const __grid_constant__ StageArgs<float> A, const __grid_constan
         const int cb = it & 1, pb = cb ^ 1;              // buffers of plane p and of plane p+-1
         const uint32_t wpar = (uint32_t)((it + 1) >> 2) & 1u;      // D = 4
         uint64_t* wbar = bars + ((it + 1) & (D - 1));
+        if (!TMA && it + 2 <= niter) {
+            issue(it + 2);
+            issued = it + 2;
+        }
         if (facew) {
+            // without TMA: U^n of the cells this iteration completes, in
+            // flight during its faces
+            float u0r[TMA || STAGE == 1 ? 1 : RPW][NF];
+            if constexpr (!TMA && STAGE == 2) {
+                if (FIN) {
+#pragma unroll
+                    for (int r = 0; r < RPW; ++r)
+#pragma unroll
+                        for (int f = 0; f < NF; ++f)
+                            u0r[r][f] = own[r] ? (A.U0 + f * A.N + (p - 1) * plane)[gown + r * nx] : 0.f;
+                }
+            }
             if (XY) {
                 const float4* P4 = reinterpret_cast<const float4*>(Pbase + cb * L::PQ);
                 const float* Pp = Pbase + cb * L::PQ + 4 * NPC;
@@ -484,9 +569,11 @@ stage_ws_kernel(const __grid_constant__ StageArgs<float> A, const __grid_constan
                                 if constexpr (STAGE == 1) {
                                     Uo[f] = fmaf(dt, Lf, uc);
                                 } else {
-                                    Uo[f] = fmaf(0.5f, U0k[f * (TY * TX)], 0.5f * fmaf(dt, Lf, uc));
+                                    const float u0 = TMA ? U0k[f * (TY * TX)] : u0r[TMA ? 0 : r][f];
+                                    Uo[f] = fmaf(0.5f, u0, 0.5f * fmaf(dt, Lf, uc));
                                 }
-                                Ok[f * (TY * TX)] = Uo[f];
+                                if (TMA) Ok[f * (TY * TX)] = Uo[f];
+                                else if (own[r]) (A.Uo + f * A.N + (p - 1) * plane)[gown + r * nx] = Uo[f];
                                 yb[f] = yt[f];
                             }
                             if (EPI && A.rate_slot) {
@@ -505,7 +592,7 @@ stage_ws_kernel(const __grid_constant__ StageArgs<float> A, const __grid_constan
 #pragma unroll
                     for (int f = 0; f < NF; ++f) qLz[r][f] = qLn[f];
                 }
-                if (FIN && it >= 2) fence_proxy_async_smem();   // the staged plane is read by TMA
+                if (TMA && FIN && it >= 2) fence_proxy_async_smem();   // the staged plane is read by TMA
             } else {
 #pragma unroll
                 for (int r = 0; r < RPW; ++r)
@@ -518,7 +605,7 @@ stage_ws_kernel(const __grid_constant__ StageArgs<float> A, const __grid_constan
                 for (int f = 0; f < NF; ++f) qn[r][f] = q1[r][f];
         } else {
             // ---- converter warps ----
-            if (tid == issuer) {
+            if (TMA && tid == issuer) {
                 // the plane the face warps staged in the last iteration
                 if (p - 2 >= z0 && p - 2 < z1) {
                     tma_store_4d(&M.out, Ost + pb * L::OST, x0, y0, p - 2, 0);
@@ -589,7 +676,7 @@ stage_ws_kernel(const __grid_constant__ StageArgs<float> A, const __grid_constan
             }
             // the store issued above has read its buffer before the face
             // warps stage the next plane but one into it
-            if (tid == issuer) bulk_wait_read_all();
+            if (TMA && tid == issuer) bulk_wait_read_all();
         }
         __syncthreads();
         return s_abort[cb] != 0;
@@ -620,15 +707,16 @@ stage_ws_kernel(const __grid_constant__ StageArgs<float> A, const __grid_constan
         // flight, so that none lands after this block has left, then return.
         // The failed wait was that of iteration index 0 (prologue) or it + 1;
         // loads were issued up to `issued`.
-        if (tid == issuer) {
+        if (loads) {
             const int first = prologue_failed ? 0 : it + 1;
             for (int r = first; r <= issued; ++r) mbar_wait(bars + (r % D), (uint32_t)((r / D) & 1));
-            bulk_wait_all();
+            if (TMA) bulk_wait_all();
+            else cp_async_wait_all();
         }
         __syncthreads();
         return;
     }
-    if (tid == issuer) {
+    if (TMA && tid == issuer) {
         // the last plane: cell z1 - 1, staged in iteration niter - 1
         tma_store_4d(&M.out, Ost + ((niter - 1) & 1) * L::OST, x0, y0, z1 - 1, 0);
         bulk_commit();
