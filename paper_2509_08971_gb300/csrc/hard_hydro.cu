@@ -105,6 +105,8 @@ void build_mesh(hard_hydro_s* h) {
     m.dim = a;
     m.gamma = h->gamma;
     m.N = (long long)h->n[0] * h->n[1] * h->n[2];
+    if (a == 3)
+        for (int f64 = 0; f64 < 2; ++f64) m.auto3[f64] = hh::choose_tile3(m.n, f64);
 }
 
 void free_scratch(hard_hydro_s* h) {
@@ -215,7 +217,7 @@ bool halo_ready(const hard_hydro_s* h) {
 
 // blocks of one stage launch (rows of the totals partial array)
 long long launch_blocks(const hard_hydro_s* h) {
-    if (weno(h)) return hh::weno_stage_blocks(h->mesh, h->mesh.dim == 3);
+    if (weno(h)) return hh::weno_stage_blocks(h->mesh, h->mesh.dim == 3, h->dtype == HARD_F64);
     return hh::stage_blocks(h->mesh, h->tile, h->dtype == HARD_F64);
 }
 

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 namespace hh {
 
 struct TileDesc {
@@ -22,7 +24,87 @@ struct MeshDesc {
     bool act[3];           // physical axis active
     double gamma;
     long long N;           // total cells
+    TileDesc auto3[2] = {{32, 8, 32}, {32, 8, 32}};   // 3D: choose_tile3 of FP32, FP64
 };
+
+// ---- chunk lengths by a schedule model ----
+// A kernel that marches an axis of n cells in chunks of z has one block per
+// tile column and chunk; a block takes (z + over) steps, over standing for its
+// warm-up cells, first loads and reductions.  span_steps is the time, in
+// steps, until `slots` resident blocks have worked off the whole chunks and
+// then the columns' shorter last ones, in launch order.
+inline constexpr int SMS = 152;
+inline double span_steps(long long cols, int n, int z, double over, long long slots) {
+    const long long full = cols * (n / z), q = full / slots, r = full % slots;
+    const int rem = n % z;
+    const double a = z + over, b = rem + over;
+    const double t0 = q * a, t1 = t0 + a;              // slots - r are free at t0, r at t1
+    double t = r ? t1 : t0;
+    if (!rem) return t;
+    if (cols > 64 * slots) return (full * a + cols * b) / slots + 0.5 * a;
+    for (int k = 1;; ++k) {                            // the short chunks fill up behind
+        const double e0 = t0 + k * b, e1 = t1 + k * b;
+        const auto done = [&](double e) {
+            long long d = 0;
+            if (e >= t0) d += (slots - r) * (long long)((e - t0) / b + 1e-9);
+            if (e >= t1) d += r * (long long)((e - t1) / b + 1e-9);
+            return d;
+        };
+        if (done(e0) >= cols) return e0 > t ? e0 : t;
+        if (r && done(e1) >= cols && done(t0 + (k + 1) * b) >= cols)
+            return e1 < t0 + (k + 1) * b ? e1 : t0 + (k + 1) * b;
+    }
+}
+// The chunk length of the least time(z, blocks).  Lengths that cut n evenly, at
+// most 72 (neighbouring columns drift apart in longer ones and lose halo planes
+// in L2: 512^3, 2.94 ms a stage with 64 planes, 2.97 with 128) but 512 chunks
+// at most; *best (if given) its time.
+template <class Time>
+inline int choose_chunk(long long cols, int n, const Time& time, double* best = nullptr) {
+    double tb = 1e300;
+    int zb = n, last = 0;
+    for (int c = std::min((n + 71) / 72, 512); c <= n && c <= 512; ++c) {
+        const int z = (n + c - 1) / c;
+        if (z == last) continue;
+        last = z;
+        const double t = time(z, cols * ((n + z - 1) / z));
+        if (t < tb) {
+            tb = t;
+            zb = z;
+        }
+    }
+    if (best) *best = tb;
+    return zb;
+}
+// Tile and z chunk of the 3D stage kernels.  Steps measured on 32-wide tiles:
+// FP32 (warp-specialised, bound by issue) 1.53 us a plane of 32 x 8 alone on its
+// SM, 1.85 us with a second block, 1.67 us of 32 x 16 (one block per SM), a
+// block's fixed cost ~3 planes; FP64 (bound by its pipe, whatever is
+// resident) 54.6 us of 32 x 8 and 35.1 us of 32 x 4 (58 us as one of two),
+// fixed cost ~1 plane.  One fixed 32 x 8 x 32 tile leaves most of the chip
+// idle on small meshes and most of the last wave on others.
+inline TileDesc choose_tile3(const int n[3], bool f64) {
+    struct Form { int ty, kmax; double over, step[2]; };
+    static constexpr Form F32[] = {{16, 1, 3.2, {1.67, 0}}, {8, 2, 3.0, {1.53, 1.85}}};
+    static constexpr Form F64[] = {{8, 1, 1.0, {54.6, 0}}, {4, 2, 1.2, {35.1, 58.0}}};
+    TileDesc td{32, 8, 32};
+    double tb = 1e300;
+    for (const Form& f : f64 ? F64 : F32) {
+        const long long gy = (n[1] + f.ty - 1) / f.ty;
+        if (n[1] > 8 * 65535 || gy > 65535) continue;  // gridDim.y
+        const long long cols = (n[0] + 31) / 32 * gy;
+        double t;
+        const int z = choose_chunk(cols, n[2], [&](int zc, long long blocks) {
+            const int k = blocks > SMS ? f.kmax : 1;   // blocks on an SM
+            return span_steps(cols, n[2], zc, f.over, (long long)SMS * k) * f.step[k - 1];
+        }, &t);
+        if (t < tb) {
+            tb = t;
+            td = TileDesc{32, f.ty, z};
+        }
+    }
+    return td;
+}
 
 struct StageCall {
     int stage;                     // 1 or 2
@@ -72,7 +154,7 @@ inline TileDesc launch_tile(const MeshDesc& m, int tile, bool f64) {
         const long long want = 152ll * (f64 ? 4 : 8);
         return TILES2[rows >= 16 * want ? 2 : rows >= 4 * want ? 1 : 0];
     }
-    return tile_desc(m.dim, 0);
+    return m.dim == 3 ? m.auto3[f64] : tile_desc(m.dim, 0);
 }
 // Blocks the stage kernel launches (rows of the totals partial array).
 inline long long stage_blocks(const MeshDesc& m, int tile, bool f64) {

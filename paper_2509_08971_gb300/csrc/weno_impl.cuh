@@ -61,20 +61,27 @@ cudaError_t run_weno(const MeshDesc& m, const StageCall& c, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+// Grid of a march along kernel axis ax, whose chunk it sets.
+dim3 march_grid(const MeshDesc& m, int ax, int& chunk) {
+    const long long columns = (long long)m.n[0] * m.n[ax == 1 ? 2 : 1];
+    chunk = march_chunk(columns, m.n[ax], sizeof(T) == 8);
+    return dim3((unsigned)march_blocks(columns), wcdiv(m.n[ax], chunk));
+}
+
 // The three sweeps of one stage on a 3D mesh (weno_sweep.cuh).
 cudaError_t run_weno_sweeps(const MeshDesc& m, const StageCall& c, cudaStream_t s) {
-    const StageArgs<T> A = weno_args(m, WENO_SWEEP_CHUNK, c);
+    StageArgs<T> A = weno_args(m, 1, c);
     T* L = static_cast<T*>(c.scratch);
     if (m.n[1] > 65535 || m.n[2] > 65535) return cudaErrorInvalidValue;
     const dim3 gx(wcdiv(m.n[0], WX_SEG), wcdiv(m.n[1], SWEEP_THREADS / 32), m.n[2]);
     weno_x_kernel<T, 0><<<gx, SWEEP_THREADS, 0, s>>>(A, L);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const dim3 gy(wcdiv(m.n[0], SWEEP_THREADS), m.n[2], wcdiv(m.n[1], WENO_SWEEP_CHUNK));
+    const dim3 gy = march_grid(m, 1, A.zchunk);
     weno_march_kernel<T, 1, 1, false><<<gy, SWEEP_THREADS, 0, s>>>(A, L);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const dim3 gz(wcdiv(m.n[0], SWEEP_THREADS), m.n[1], wcdiv(m.n[2], WENO_SWEEP_CHUNK));
+    const dim3 gz = march_grid(m, 2, A.zchunk);
     weno_march_kernel<T, 2, 2, true><<<gz, SWEEP_THREADS, 0, s>>>(A, L);
     return cudaGetLastError();
 }
@@ -93,17 +100,17 @@ cudaError_t run_advect(const MeshDesc& m, const AdvectArgs<T>& A, cudaStream_t s
 }
 
 // The three sweeps of one advection stage on a 3D mesh (weno_sweep.cuh).
-cudaError_t run_advect_sweeps(const MeshDesc& m, const AdvectArgs<T>& A, T* L, cudaStream_t s) {
+cudaError_t run_advect_sweeps(const MeshDesc& m, AdvectArgs<T> A, T* L, cudaStream_t s) {
     if (m.n[1] > 65535 || m.n[2] > 65535) return cudaErrorInvalidValue;
     const dim3 gx(wcdiv(m.n[0], WX_SEG), wcdiv(m.n[1], SWEEP_THREADS / 32), m.n[2]);
     advect_x_kernel<T, 0><<<gx, SWEEP_THREADS, 0, s>>>(A, L);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const dim3 gy(wcdiv(m.n[0], SWEEP_THREADS), m.n[2], wcdiv(m.n[1], WENO_SWEEP_CHUNK));
+    const dim3 gy = march_grid(m, 1, A.zchunk);
     advect_march_kernel<T, 1, 1, false><<<gy, SWEEP_THREADS, 0, s>>>(A, L);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const dim3 gz(wcdiv(m.n[0], SWEEP_THREADS), m.n[1], wcdiv(m.n[2], WENO_SWEEP_CHUNK));
+    const dim3 gz = march_grid(m, 2, A.zchunk);
     advect_march_kernel<T, 2, 2, true><<<gz, SWEEP_THREADS, 0, s>>>(A, L);
     return cudaGetLastError();
 }
@@ -130,10 +137,7 @@ cudaError_t HH_WCAT(launch_advect_E_stage_, HH_SUFFIX)(const MeshDesc& m, int st
     A.dt = dt;
     A.stage = stage;
     A.zchunk = WENO_ZC;
-    if (m.dim == 3 && scratch) {
-        A.zchunk = WENO_SWEEP_CHUNK;
-        return run_advect_sweeps(m, A, static_cast<T*>(scratch), s);
-    }
+    if (m.dim == 3 && scratch) return run_advect_sweeps(m, A, static_cast<T*>(scratch), s);
     if (m.dim == 3) return run_advect<WENO_TX2, WENO_TY2, 3, 0, 1>(m, A, s);
     if (m.dim == 2) {
         if (m.px == 0 && m.py == 1) return run_advect<WENO_TX2, WENO_TY2, 2, 0, 1>(m, A, s);

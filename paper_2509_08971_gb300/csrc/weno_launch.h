@@ -5,26 +5,35 @@
 
 namespace hh {
 
-// The directional sweeps of the scheme on 3D meshes (weno_sweep.cuh): blocks
-// of WENO_SWEEP_THREADS columns along x', chunks of WENO_SWEEP_CHUNK cells
-// along the march axis.
-#ifndef HH_WENO_CHUNK
-#define HH_WENO_CHUNK 64
-#endif
+// The marches of the scheme's directional sweeps on 3D meshes (weno_sweep.cuh):
+// blocks of WENO_SWEEP_THREADS columns, a chunk of cells of the march axis each.
+inline constexpr int WENO_SWEEP_THREADS = 128;
+inline long long march_blocks(long long columns) {
+    return (columns + WENO_SWEEP_THREADS - 1) / WENO_SWEEP_THREADS;
+}
+// Cells per chunk of a march over n cells.  The six warm-up cells, of which four
+// only enter the window, cost about four.  Blocks of one SM share its issue
+// slots (FP32, from the second on) or its FP64 pipe, so an SM takes the time
+// of its blocks one after the other, and one block alone twice its share
+// (FP32) or 1.2 times (FP64).
+inline int march_chunk(long long columns, int n, bool f64) {
+    const long long cols = march_blocks(columns);
+    return choose_chunk(cols, n, [&](int z, long long) {
+        return std::max(span_steps(cols, n, z, 4.0, SMS), (f64 ? 1.2 : 2.0) * (z + 4.0));
+    });
+}
 // Tiles of the fused kernel: 128 cells in 1D, 32 x 8 in 2D and 3D, 32-plane
 // z chunks.
 inline constexpr int WENO_TX1 = 128, WENO_TX2 = 32, WENO_TY2 = 8, WENO_ZC = 32;
-inline constexpr int WENO_SWEEP_THREADS = 128;
-inline constexpr int WENO_SWEEP_CHUNK = HH_WENO_CHUNK;
 
 // Blocks of the launch that carries a WENO stage's epilogue (rows of the
 // totals partial array): the combining z' march of the sweeps, or the fused
 // kernel's grid (the first tile of the mesh's tile table).
-inline long long weno_stage_blocks(const MeshDesc& m, bool sweeps) {
+inline long long weno_stage_blocks(const MeshDesc& m, bool sweeps, bool f64) {
     if (m.dim == 3 && sweeps) {
-        const long long bx = (m.n[0] + WENO_SWEEP_THREADS - 1) / WENO_SWEEP_THREADS;
-        const long long bz = (m.n[2] + WENO_SWEEP_CHUNK - 1) / WENO_SWEEP_CHUNK;
-        return bx * m.n[1] * bz;
+        const long long columns = (long long)m.n[0] * m.n[1];
+        const int z = march_chunk(columns, m.n[2], f64);
+        return march_blocks(columns) * ((m.n[2] + z - 1) / z);
     }
     return (long long)((m.n[0] + (m.dim == 1 ? WENO_TX1 : WENO_TX2) - 1) / (m.dim == 1 ? WENO_TX1 : WENO_TX2)) *
            (m.dim >= 2 ? (m.n[1] + WENO_TY2 - 1) / WENO_TY2 : 1) *

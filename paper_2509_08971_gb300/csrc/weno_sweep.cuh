@@ -156,9 +156,16 @@ weno_x_kernel(const StageArgs<T> A, T* __restrict__ L) {
     }
 }
 
-// March along kernel axis AX (1: y', 2: z'): lane = x', one block row of
-// SWEEP_THREADS columns, the other transverse coordinate blockIdx.y, a chunk
-// of A.zchunk cells of the march axis per blockIdx.z.  Adds this axis' flux
+// First cell of column q of the (x', z') plane, x' fastest.
+__device__ __forceinline__ long long column_base(long long q, int n0, int n1) {
+    const long long o = q >> 32 ? q / n0 : (long long)((unsigned)q / (unsigned)n0);
+    return o * n1 * n0 + (q - o * n0);
+}
+
+// March along kernel axis AX (1: y', 2: z'): SWEEP_THREADS columns of the
+// plane across it per block (rows of x' one after the other, so a row of any
+// length fills its lanes), a chunk of A.zchunk cells of the march axis per
+// blockIdx.y.  Adds this axis' flux
 // difference to L; LAST: then the combine.  Every global load is issued one
 // step before its value is used (the next cell's state; the flux difference,
 // state and U^n of the cell that completes at the next step), so a step's
@@ -174,14 +181,15 @@ weno_march_kernel(const StageArgs<T> A, T* __restrict__ L) {
     static_assert(AX == 1 || AX == 2, "the x' axis is the x sweep's");
     const int n0 = A.n[0], n1 = A.n[1];
     const int nA = A.n[AX];
-    const int x = blockIdx.x * SWEEP_THREADS + threadIdx.x;
-    const bool xin = x < n0;
-    const int xl = xin ? x : n0 - 1;                   // lanes past the row load a valid cell
-    const int o = blockIdx.y;                          // z' (AX = 1) or y' (AX = 2)
+    // columns (x', z') for AX = 1, (x', y') for AX = 2, x' fastest
+    const long long q = blockIdx.x * (long long)SWEEP_THREADS + threadIdx.x;
+    const long long columns = (long long)n0 * A.n[AX == 1 ? 2 : 1];
+    const bool xin = q < columns;
+    const long long ql = xin ? q : columns - 1;        // lanes past the last column load a valid cell
     const long long stride = AX == 1 ? (long long)n0 : (long long)n0 * n1;
-    const long long base = (AX == 1 ? (long long)o * n1 * n0 : (long long)o * n0) + xl;
+    const long long base = AX == 1 ? column_base(ql, n0, n1) : ql;
     const long long N = A.N;
-    const int a0 = blockIdx.z * A.zchunk;
+    const int a0 = blockIdx.y * A.zchunk;
     const int a1 = min(a0 + A.zchunk, nA);
     const T gamma = A.gamma;
     const T gx = sizeof(T) == 4 ? A.igm1 : A.gm1;
@@ -303,7 +311,7 @@ weno_march_kernel(const StageArgs<T> A, T* __restrict__ L) {
         }
     }
     if constexpr (LAST) {
-        const long long blk = ((long long)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+        const long long blk = (long long)blockIdx.y * gridDim.x + blockIdx.x;
         sweep_epilogue(A, bad, rate_max, tot, blk);
     }
 }
@@ -383,13 +391,13 @@ advect_march_kernel(const AdvectArgs<T> A, T* __restrict__ L) {
     static_assert(AX == 1 || AX == 2, "the x' axis is the x sweep's");
     const int n0 = A.n[0], n1 = A.n[1];
     const int nA = A.n[AX];
-    const int x = blockIdx.x * SWEEP_THREADS + threadIdx.x;
-    const bool xin = x < n0;
-    const int xl = xin ? x : n0 - 1;
-    const int o = blockIdx.y;
+    const long long q = blockIdx.x * (long long)SWEEP_THREADS + threadIdx.x;
+    const long long columns = (long long)n0 * A.n[AX == 1 ? 2 : 1];
+    const bool xin = q < columns;
+    const long long ql = xin ? q : columns - 1;
     const long long stride = AX == 1 ? (long long)n0 : (long long)n0 * n1;
-    const long long base = (AX == 1 ? (long long)o * n1 * n0 : (long long)o * n0) + xl;
-    const int a0 = blockIdx.z * A.zchunk;
+    const long long base = AX == 1 ? column_base(ql, n0, n1) : ql;
+    const int a0 = blockIdx.y * A.zchunk;
     const int a1 = min(a0 + A.zchunk, nA);
     const T dt = (T)A.dt;
     const bool two = A.stage == 2;
