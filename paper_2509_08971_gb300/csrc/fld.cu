@@ -16,7 +16,9 @@
 //   * restriction: the mean of the children's residuals; prolongation:
 //     the coarse correction added to every child (piecewise constant).
 // grad E of R: central differences, the edge cell repeated at a non-periodic
-// boundary.  Everything is bandwidth-bound stencil work over the levels.
+// boundary.  Everything is bandwidth-bound stencil work over the levels, which
+// are stored by colour (fld_split.cuh) unless an odd periodic axis breaks the
+// colouring or the level belongs to the one-block set.
 #include <cmath>
 #include <new>
 
@@ -35,18 +37,20 @@ struct FldLevel {
     double dx[3];
     long long N;
     bool coarsened[3];       // this level's axes halved into the next level
-    void* x;                 // solution / correction (level 0: the caller's Er)
-    void* b;                 // right-hand side
-    void* D;                 // cell coefficient
+    int stride = 0;          // > 0: x, b, D stored by colour, rows of this many entries (fld_split.cuh)
+    void* x = nullptr;       // solution / correction (level 0 in mesh order: the caller's Er)
+    void* b = nullptr;       // right-hand side
+    void* D = nullptr;       // cell coefficient
 };
 
 struct FldHierarchy {
     int dtype;
     int nl;
+    int ls;                  // levels ls .. nl-1 run in one block (small_vcycle_kernel)
     int n0[3];
     int bc_lo[3], bc_hi[3];
     FldLevel L[FLD_MAX_LEVELS];
-    double* norms;           // device: sum r^2, sum b^2
+    double* norms = nullptr; // device: sum r^2, sum b^2
 };
 
 namespace {
@@ -159,7 +163,13 @@ __device__ __forceinline__ void stencil(const LvlArgs<T>& a, int i, int j, int k
     stencil_eval(a, v, diag, off);
 }
 
-// Launch shape of the level kernels: x along threads (and blockIdx.x), one
+}  // namespace
+}  // namespace hh
+#include "fld_split.cuh"
+namespace hh {
+namespace {
+
+// Launch shape of the level kernels of a level in mesh order: x along threads (and blockIdx.x), one
 // row j per blockIdx.y (SMOOTH_ROWS rows for the smoother), one plane k per
 // blockIdx.z: no index division.
 //
@@ -187,6 +197,7 @@ constexpr int FLD_FINE_ROWS = HH_FLD_FINE_ROWS;       // and on level 0
 template <typename T, int SR>
 __global__ void __launch_bounds__(128) smooth_kernel(const LvlArgs<T> a, int color, int lg) {
     griddep_wait();
+    griddep_launch_dependents();
     const int k = blockIdx.z;
     const int p = blockIdx.x * (1 << lg) + (threadIdx.x & ((1 << lg) - 1));
     const int j0 = (blockIdx.y * (128 >> lg) + (threadIdx.x >> lg)) * SR;
@@ -217,7 +228,6 @@ __global__ void __launch_bounds__(128) smooth_kernel(const LvlArgs<T> a, int col
 #pragma unroll
     for (int r = 0; r < SR; ++r)
         if (on[r]) a.x[qs[r]] = bq[r];
-    griddep_launch_dependents();
 }
 
 // Residual of level l restricted to level l+1 in one pass: one thread per
@@ -237,6 +247,7 @@ __global__ void __launch_bounds__(128) residual_restrict_kernel(const LvlArgs<T>
                                                                 int nc0, int nc1, int h0, int h1,
                                                                 int h2) {
     griddep_wait();
+    griddep_launch_dependents();
     const int J = blockIdx.y, K = blockIdx.z;
     const int I = blockIdx.x * blockDim.x + threadIdx.x;
     if (I >= nc0) return;
@@ -282,7 +293,6 @@ __global__ void __launch_bounds__(128) residual_restrict_kernel(const LvlArgs<T>
     const int Q = (K * nc1 + J) * nc0 + I;
     bc[Q] = sum / T(h0 * h1 * h2);
     xc[Q] = T(0);
-    griddep_launch_dependents();
 }
 
 // Convergence check of the fine level: sum r^2 and sum b^2 (r = b - A x) into
@@ -297,6 +307,7 @@ __global__ void __launch_bounds__(128) residual_restrict_kernel(const LvlArgs<T>
 template <typename T>
 __global__ void __launch_bounds__(128) residual_norms_kernel(const LvlArgs<T> a, double* norms) {
     griddep_wait();
+    griddep_launch_dependents();
     __shared__ double sr[4], sb[4];
     double rr = 0.0, bb = 0.0;
     const int segs = (a.n[0] + 127) / 128;
@@ -360,7 +371,6 @@ __global__ void __launch_bounds__(128) residual_norms_kernel(const LvlArgs<T> a,
         atomicAdd(norms, tr);
         atomicAdd(norms + 1, tb);
     }
-    griddep_launch_dependents();
 }
 
 // The same check once the fine level's post-smoothing has ended with a
@@ -374,6 +384,7 @@ template <typename T>
 __global__ void __launch_bounds__(128) residual_norm_color_kernel(const LvlArgs<T> a, int color,
                                                                   double* norms) {
     griddep_wait();
+    griddep_launch_dependents();
     const int k = blockIdx.z;
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     StencilVals<T> v[SMOOTH_ROWS];
@@ -421,7 +432,6 @@ __global__ void __launch_bounds__(128) residual_norm_color_kernel(const LvlArgs<
         const double t = sr[0] + sr[1] + sr[2] + sr[3];
         if (t != 0.0) atomicAdd(norms, t);
     }
-    griddep_launch_dependents();
 }
 
 // sum b^2 of the fine level into *out (once per solve; b does not change).
@@ -538,6 +548,7 @@ template <typename T>
 __global__ void __launch_bounds__(FLD_SMALL_THREADS)
 small_vcycle_kernel(const __grid_constant__ SmallLevels<T> S) {
     griddep_wait();
+    griddep_launch_dependents();
     extern __shared__ __align__(16) unsigned char fld_smem[];
     T* sm = reinterpret_cast<T*>(fld_smem);
     for (int l = 0; l < S.count; ++l) {
@@ -583,30 +594,50 @@ small_vcycle_kernel(const __grid_constant__ SmallLevels<T> S) {
         __syncthreads();
     }
     // the coarsest level: red-black sweeps until a sweep changes nothing
-    // (every later sweep would return the same values) or `coarse` sweeps
+    // (every later sweep would return the same values) or `coarse` sweeps.
+    // One warp sweeps a level of at most 64 cells: the barriers between its
+    // half-sweeps are a warp's, not a block's.
     {
         __shared__ int changed[2];
         const int lc = S.count - 1;
         const LvlArgs<T> s = small_level(S, sm, lc);
         const int N = (int)s.N, n0 = s.n[0], n1 = s.n[1];
-        if (threadIdx.x == 0) changed[0] = 0;
-        __syncthreads();
-        for (int it = 0; it < S.coarse; ++it) {
-            for (int color = 0; color < 2; ++color) {
-                if (color == 1 && threadIdx.x == 0) changed[(it + 1) & 1] = 0;
-                for (int q = threadIdx.x; q < N; q += blockDim.x) {
-                    const int t = small_div(q, S.mg[lc][0], n0), i = q - t * n0;
-                    const int k = small_div(t, S.mg[lc][1], n1), j = t - k * n1;
-                    if (((i + j + k) & 1) != color) continue;
-                    T diag, off;
-                    stencil(s, i, j, k, q, diag, off);
-                    const T nx = (s.b[q] + off) / diag;
-                    if (!(nx == s.x[q])) changed[it & 1] = 1;    // also NaN: keep sweeping
-                    s.x[q] = nx;
-                }
-                __syncthreads();
+        const bool one = N <= 64;
+        const int step = one ? 32 : (int)blockDim.x;
+        auto half = [&](int color) {
+            bool ch = false;
+            for (int q = threadIdx.x; q < N; q += step) {
+                const int t = small_div(q, S.mg[lc][0], n0), i = q - t * n0;
+                const int k = small_div(t, S.mg[lc][1], n1), j = t - k * n1;
+                if (((i + j + k) & 1) != color) continue;
+                T diag, off;
+                stencil(s, i, j, k, q, diag, off);
+                const T nx = (s.b[q] + off) / diag;
+                ch |= !(nx == s.x[q]);                       // also NaN: keep sweeping
+                s.x[q] = nx;
             }
-            if (!changed[it & 1]) break;          // the same value in every thread
+            return ch;
+        };
+        if (one) {
+            if (threadIdx.x < 32)
+                for (int it = 0; it < S.coarse; ++it) {
+                    bool ch = half(0);
+                    __syncwarp();
+                    ch |= half(1);
+                    if (!__any_sync(0xffffffffu, ch)) break;
+                }
+            __syncthreads();
+        } else {
+            if (threadIdx.x == 0) changed[0] = 0;
+            __syncthreads();
+            for (int it = 0; it < S.coarse; ++it) {
+                if (half(0)) changed[it & 1] = 1;
+                __syncthreads();
+                if (threadIdx.x == 0) changed[(it + 1) & 1] = 0;
+                if (half(1)) changed[it & 1] = 1;
+                __syncthreads();
+                if (!changed[it & 1]) break;                 // the same value in every thread
+            }
         }
     }
     // up: add the coarse correction to the children, smooth
@@ -630,7 +661,6 @@ small_vcycle_kernel(const __grid_constant__ SmallLevels<T> S) {
         const int N = (int)S.lv[0].N;
         for (int q = threadIdx.x; q < N; q += blockDim.x) S.lv[0].x[q] = sm[S.off[0] + q];
     }
-    griddep_launch_dependents();
 }
 
 // coarse[I] = mean of the children fine[...] (restriction of D): one thread
@@ -656,6 +686,7 @@ template <typename T>
 __global__ void __launch_bounds__(128) prolong_kernel(T* fine, const T* coarse, int nf0, int nf1,
                                                       int nc0, int nc1, int h0, int h1, int h2) {
     griddep_wait();
+    griddep_launch_dependents();
     const int k = blockIdx.z;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nf0) return;
@@ -676,7 +707,6 @@ __global__ void __launch_bounds__(128) prolong_kernel(T* fine, const T* coarse, 
 #pragma unroll
     for (int r = 0; r < SMOOTH_ROWS; ++r)
         if (on[r]) fine[qs[r]] = f[r] + c[r];
-    griddep_launch_dependents();
 }
 
 // D = c lambda(R) / (kappa rho), R = |grad E| / (rho kappa E), on level 0:
@@ -686,8 +716,11 @@ __global__ void __launch_bounds__(128) prolong_kernel(T* fine, const T* coarse, 
 // wrap or, at a wall, the cell itself.  h0, h1, h2: 1 / (2 dx) per axis; the
 // limiter's quotient and the last one are taken together,
 // D = c (2 + R) / ((6 + 3R + R^2) kappa rho).
-template <typename T>
-__global__ void __launch_bounds__(128) coeff_kernel(const T* U, const T* E, T* D, LvlArgs<T> a,
+// SPLIT: D goes to a level stored by colour, with E as its b and (colour 1, all
+// that the first half-sweep reads) its x.
+template <typename T, bool SPLIT>
+__global__ void __launch_bounds__(128) coeff_kernel(const T* U, const T* E, CellArray<T> D,
+                                                    CellArray<T> b, CellArray<T> x, LvlArgs<T> a,
                                                     T c, T kappa, T h0, T h1, T h2) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.z;
     if (i >= a.n[0]) return;
@@ -729,7 +762,21 @@ __global__ void __launch_bounds__(128) coeff_kernel(const T* U, const T* E, T* D
         }
         const T R = sqrt(grad2) / (rho[r] * kappa * Ec[r]);
         const T den = (T(6) + T(3) * R + R * R) * (kappa * rho[r]);
-        if (on[r]) D[qs[r]] = c * (T(2) + R) / den;
+        if (!on[r]) continue;
+        const T d = c * (T(2) + R) / den;
+        if constexpr (SPLIT) {
+            const int q = D.index(i, blockIdx.y * SMOOTH_ROWS + r, k);
+            D.a[q] = d;
+            b.a[q] = Ec[r];
+            const bool odd = (i + blockIdx.y * SMOOTH_ROWS + r + k) & 1;
+            if (odd) x.a[q] = Ec[r];
+            if (a.per[0]) {
+                wrap_entry(D, i, q, d);
+                if (odd) wrap_entry(x, i, q, Ec[r]);
+            }
+        } else {
+            D.a[qs[r]] = d;
+        }
     }
 }
 
@@ -762,7 +809,96 @@ LvlArgs<T> level_args(const FldHierarchy* H, int l, double dt) {
 }
 
 template <typename T>
+CellArray<T> cells(const FldLevel& L, void* p) {
+    return CellArray<T>{static_cast<T*>(p), L.n[0], L.n[1], L.n[2], L.stride};
+}
+
+template <typename T>
+SplitArgs<T> split_args(const FldHierarchy* H, int l, double dt) {
+    const LvlArgs<T> v = level_args<T>(H, l, dt);
+    const FldLevel& L = H->L[l];
+    SplitArgs<T> a;
+    a.x = v.x;
+    a.b = v.b;
+    a.D = v.D;
+    a.h = (L.n[0] + 1) / 2;
+    a.stride = L.stride;
+    a.groups = (a.h + VecOf<T>::V - 1) / VecOf<T>::V;
+    a.color = L.n[1] * L.n[2] * L.stride;
+    for (int ax = 0; ax < 3; ++ax) {
+        a.n[ax] = v.n[ax];
+        a.wk[ax] = v.wk[ax];
+        a.per[ax] = v.per[ax];
+    }
+    return a;
+}
+
+// Blocks of `per_row` threads for each of `rows` rows, times `y`.
+dim3 flat_grid(int per_row, int rows, int y) {
+    return dim3((unsigned)(((long long)per_row * rows + 127) / 128), (unsigned)y);
+}
+
+// Planes per block of a marching kernel: up to eight, as long as six blocks
+// per SM remain (a longer march reads fewer planes twice).
+template <typename T>
+int split_chunk(const SplitArgs<T>& a) {
+    int c = 8;
+    while (c > 1 && (long long)flat_grid(a.groups, a.n[1], 1).x * ((a.n[2] + c - 1) / c) < 152 * 6) c /= 2;
+    return c;
+}
+
+template <typename T>
+cudaError_t smooth_split(const FldHierarchy* H, int l, double dt, int sweeps, cudaStream_t s) {
+    const SplitArgs<T> a = split_args<T>(H, l, dt);
+    const int chunk = split_chunk(a);
+    const dim3 g = flat_grid(a.groups, a.n[1], (a.n[2] + chunk - 1) / chunk);
+    auto kern = a.per[0] ? split_smooth_kernel<T, false> : split_smooth_kernel<T, true>;
+    for (int it = 0; it < 2 * sweeps; ++it) {
+        const cudaError_t e = launch_pdl(kern, g, dim3(128), 0, s, a, it & 1, chunk);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+// sum r^2 over the colours of `colors` (bit 0, bit 1) into *out.
+template <typename T>
+cudaError_t norm_split(const FldHierarchy* H, double dt, int colors, double* out, cudaStream_t s) {
+    const SplitArgs<T> a = split_args<T>(H, 0, dt);
+    const int chunk = split_chunk(a);
+    const dim3 g = flat_grid(a.groups, a.n[1], (a.n[2] + chunk - 1) / chunk);
+    auto kern = a.per[0] ? split_norm_kernel<T, false> : split_norm_kernel<T, true>;
+    for (int c = 0; c < 2; ++c) {
+        if (!(colors >> c & 1)) continue;
+        const cudaError_t e = launch_pdl(kern, g, dim3(128), 0, s, a, c, chunk, out);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+template <typename T>
+cudaError_t down_split(const FldHierarchy* H, int l, double dt, cudaStream_t s) {
+    const FldLevel &F = H->L[l], &C = H->L[l + 1];
+    const SplitArgs<T> a = split_args<T>(H, l, dt);
+    const int h1 = F.coarsened[1] ? 2 : 1, h2 = F.coarsened[2] ? 2 : 1;
+    auto kern = !F.coarsened[0] ? split_restrict_x_kernel<T, true>
+                : a.per[0]      ? split_restrict_kernel<T, false>
+                                : split_restrict_kernel<T, true>;
+    return launch_pdl(kern, flat_grid(F.coarsened[0] ? a.groups : C.n[0], C.n[1], C.n[2]), dim3(128),
+                      0, s, a, cells<T>(C, C.b), cells<T>(C, C.x), h1, h2);
+}
+
+template <typename T>
+cudaError_t up_split(const FldHierarchy* H, int l, double dt, cudaStream_t s) {
+    const FldLevel &F = H->L[l], &C = H->L[l + 1];
+    const SplitArgs<T> a = split_args<T>(H, l, dt);
+    return launch_pdl(split_prolong_kernel<T>, flat_grid(a.groups, a.n[1], a.n[2]), dim3(128), 0, s, a,
+                      cells<T>(C, C.x), F.coarsened[0] ? 2 : 1, F.coarsened[1] ? 2 : 1,
+                      F.coarsened[2] ? 2 : 1);
+}
+
+template <typename T>
 cudaError_t smooth(const FldHierarchy* H, int l, double dt, int sweeps, cudaStream_t s) {
+    if (H->L[l].stride) return smooth_split<T>(H, l, dt, sweeps, s);
     const LvlArgs<T> a = level_args<T>(H, l, dt);
     const FldLevel& L = H->L[l];
     const int hx = (L.n[0] + 1) / 2;                  // cells of a colour in a row (at most)
@@ -782,12 +918,18 @@ cudaError_t smooth(const FldHierarchy* H, int l, double dt, int sweeps, cudaStre
 }
 
 template <typename T>
-void restrict_to(const FldHierarchy* H, int l, const void* fine, void* coarse, cudaStream_t s) {
+void restrict_D(const FldHierarchy* H, int l, cudaStream_t s) {
     const FldLevel& F = H->L[l];
     const FldLevel& C = H->L[l + 1];
-    restrict_kernel<T><<<rows_grid(C, 1), 128, 0, s>>>(
-        static_cast<const T*>(fine), static_cast<T*>(coarse), F.n[0], F.n[1], C.n[0], C.n[1],
-        F.coarsened[0] ? 2 : 1, F.coarsened[1] ? 2 : 1, F.coarsened[2] ? 2 : 1);
+    const int h0 = F.coarsened[0] ? 2 : 1, h1 = F.coarsened[1] ? 2 : 1, h2 = F.coarsened[2] ? 2 : 1;
+    if (F.stride || C.stride) {
+        const bool wrap = C.stride && H->bc_lo[0] == 0 && H->bc_hi[0] == 0;
+        restrict_any_kernel<T><<<flat_grid(C.n[0], C.n[1], C.n[2]), 128, 0, s>>>(
+            cells<T>(F, F.D), cells<T>(C, C.D), wrap, h0, h1, h2);
+        return;
+    }
+    restrict_kernel<T><<<rows_grid(C, 1), 128, 0, s>>>(static_cast<const T*>(F.D), static_cast<T*>(C.D),
+                                                       F.n[0], F.n[1], C.n[0], C.n[1], h0, h1, h2);
 }
 
 template <typename T>
@@ -795,23 +937,27 @@ cudaError_t solve_t(FldHierarchy* H, const MeshDesc& m, const void* U, void* Er,
                     double c, double kappa, double rtol, int max_cycles, int* cycles,
                     double* rel_resid, cudaStream_t s) {
     FldLevel& L0 = H->L[0];
-    L0.x = Er;
-    cudaError_t e = cudaMemcpyAsync(L0.b, Er, sizeof(T) * L0.N, cudaMemcpyDeviceToDevice, s);
-    if (e != cudaSuccess) return e;
+    const bool split = L0.stride > 0;
+    cudaError_t e = cudaSuccess;
+    if (!split) {
+        L0.x = Er;
+        e = cudaMemcpyAsync(L0.b, Er, sizeof(T) * L0.N, cudaMemcpyDeviceToDevice, s);
+        if (e != cudaSuccess) return e;
+    }
     {
         const LvlArgs<T> a = level_args<T>(H, 0, dt);
         dim3 g = rows_grid(L0, 1);
         g.y = (g.y + SMOOTH_ROWS - 1) / SMOOTH_ROWS;
-        coeff_kernel<T><<<g, 128, 0, s>>>(
-            static_cast<const T*>(U), static_cast<const T*>(L0.b), static_cast<T*>(L0.D), a,
-            (T)c, (T)kappa, (T)(0.5 / m.dxk[0]), (T)(0.5 / m.dxk[1]), (T)(0.5 / m.dxk[2]));
+        auto kern = split ? coeff_kernel<T, true> : coeff_kernel<T, false>;
+        kern<<<g, 128, 0, s>>>(static_cast<const T*>(U), static_cast<const T*>(Er), cells<T>(L0, L0.D),
+                               cells<T>(L0, L0.b), cells<T>(L0, L0.x), a, (T)c, (T)kappa,
+                               (T)(0.5 / m.dxk[0]), (T)(0.5 / m.dxk[1]), (T)(0.5 / m.dxk[2]));
     }
-    for (int l = 0; l + 1 < H->nl; ++l) restrict_to<T>(H, l, H->L[l].D, H->L[l + 1].D, s);
+    for (int l = 0; l + 1 < H->nl; ++l) restrict_D<T>(H, l, s);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
 
     // the small levels at the bottom run in one block per cycle
-    int ls = H->nl;
-    while (ls > 0 && H->L[ls - 1].N <= FLD_SMALL_CELLS && H->nl - (ls - 1) <= FLD_SMALL_MAX) --ls;
+    const int ls = H->ls;
     SmallLevels<T> S;
     size_t small_bytes = 0;
     if (ls < H->nl) {
@@ -846,10 +992,11 @@ cudaError_t solve_t(FldHierarchy* H, const MeshDesc& m, const void* U, void* Er,
     bool color_check = ls > 0 && H->nl > 1;
     for (int ax = 0; ax < 3; ++ax)
         if (L0.n[ax] > 1 && m.bc_lo[ax] == HARD_BC_PERIODIC && (L0.n[ax] & 1)) color_check = false;
-    if (rtol > 0.0 && color_check) {
+    if (rtol > 0.0 && (color_check || split)) {
         if ((e = cudaMemsetAsync(H->norms, 0, 2 * sizeof(double), s)) != cudaSuccess) return e;
         sumsq_kernel<T><<<grid_for(L0.N) < 152 * 8 ? grid_for(L0.N) : 152 * 8, 256, 0, s>>>(
-            static_cast<const T*>(L0.b), L0.N, H->norms + 1);
+            static_cast<const T*>(L0.b), split ? 2ll * L0.n[1] * L0.n[2] * L0.stride : L0.N,
+            H->norms + 1);                           // padding entries of b are zero
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
 
@@ -862,6 +1009,10 @@ cudaError_t solve_t(FldHierarchy* H, const MeshDesc& m, const void* U, void* Er,
             if ((e = smooth<T>(H, l, dt, FLD_PRE, s)) != cudaSuccess) return e;
             const FldLevel& F = H->L[l];
             const FldLevel& C = H->L[l + 1];
+            if (F.stride) {
+                if ((e = down_split<T>(H, l, dt, s)) != cudaSuccess) return e;
+                continue;
+            }
             const bool h2 = F.coarsened[0] && F.coarsened[1] && F.coarsened[2];
             bool proper = true;                      // red-black is a two-colouring of level l
             for (int ax = 0; ax < 3; ++ax)
@@ -887,6 +1038,11 @@ cudaError_t solve_t(FldHierarchy* H, const MeshDesc& m, const void* U, void* Er,
             if (l + 1 >= H->nl) continue;
             const FldLevel& F = H->L[l];
             const FldLevel& C = H->L[l + 1];
+            if (F.stride) {
+                if ((e = up_split<T>(H, l, dt, s)) != cudaSuccess) return e;
+                if ((e = smooth<T>(H, l, dt, FLD_POST, s)) != cudaSuccess) return e;
+                continue;
+            }
             dim3 gp = rows_grid(F, 1);
             gp.y = (gp.y + SMOOTH_ROWS - 1) / SMOOTH_ROWS;
             e = launch_pdl(prolong_kernel<T>, gp, dim3(128), 0, s, static_cast<T*>(F.x),
@@ -897,7 +1053,10 @@ cudaError_t solve_t(FldHierarchy* H, const MeshDesc& m, const void* U, void* Er,
             if ((e = smooth<T>(H, l, dt, FLD_POST, s)) != cudaSuccess) return e;
         }
         done = cyc + 1;
-        if (rtol > 0.0 && color_check) {
+        if (rtol > 0.0 && split) {
+            if ((e = cudaMemsetAsync(H->norms, 0, sizeof(double), s)) != cudaSuccess) return e;
+            if ((e = norm_split<T>(H, dt, color_check ? 1 : 3, H->norms, s)) != cudaSuccess) return e;
+        } else if (rtol > 0.0 && color_check) {
             if ((e = cudaMemsetAsync(H->norms, 0, sizeof(double), s)) != cudaSuccess) return e;
             dim3 g = rows_grid(L0, 2);
             g.y = (g.y + SMOOTH_ROWS - 1) / SMOOTH_ROWS;
@@ -922,14 +1081,31 @@ cudaError_t solve_t(FldHierarchy* H, const MeshDesc& m, const void* U, void* Er,
             if (!(rel > rtol)) break;             // converged (or NaN: stop and report it)
         }
     }
+    if (split) {
+        const SplitArgs<T> a = split_args<T>(H, 0, dt);
+        e = launch_pdl(split_merge_kernel<T>, flat_grid(a.groups, a.n[1], a.n[2]), dim3(128), 0, s, a,
+                       static_cast<T*>(Er), L0.n[0] * sizeof(T) % 16 == 0);
+        if (e != cudaSuccess) return e;
+    }
     if (cycles) *cycles = done;
     if (rel_resid) *rel_resid = rel;
     return cudaGetLastError();
 }
 
+// Row length of a level stored by colour, 0 for mesh order: where red and
+// black is no proper two-colouring (an odd periodic axis), for rows too short
+// to fill a vector, and beyond 32-bit entries.
+int split_stride(const FldLevel& L, const int* bc_lo, const int* bc_hi) {
+    for (int ax = 0; ax < 3; ++ax)
+        if (L.n[ax] > 1 && bc_lo[ax] == HARD_BC_PERIODIC && bc_hi[ax] == HARD_BC_PERIODIC && (L.n[ax] & 1))
+            return 0;
+    const int stride = ((L.n[0] + 1) / 2 + 3) / 4 * 4;
+    return L.n[0] < 8 || 2ll * L.n[1] * L.n[2] * stride >= (1ll << 31) ? 0 : stride;
+}
+
 }  // namespace
 
-FldHierarchy* fld_create(const MeshDesc& m, int dtype) {
+FldHierarchy* fld_create(const MeshDesc& m, int dtype, cudaStream_t s) {
     FldHierarchy* H = new (std::nothrow) FldHierarchy();
     if (!H) return nullptr;
     H->dtype = dtype;
@@ -954,12 +1130,7 @@ FldHierarchy* fld_create(const MeshDesc& m, int dtype) {
             L.n[a] = n[a];
             L.dx[a] = dx[a];
         }
-        L.x = nullptr;
-        if (nl > 0 && cudaMalloc(&L.x, es * L.N) != cudaSuccess) ok = false;
-        if (cudaMalloc(&L.b, es * L.N) != cudaSuccess) ok = false;
-        if (cudaMalloc(&L.D, es * L.N) != cudaSuccess) ok = false;
         ++nl;
-        if (!ok) break;
         bool any = false;
         for (int a = 0; a < 3; ++a) {
             L.coarsened[a] = n[a] >= 4 && n[a] % 2 == 0;
@@ -976,6 +1147,21 @@ FldHierarchy* fld_create(const MeshDesc& m, int dtype) {
             }
     }
     H->nl = nl;
+    int ls = nl;
+    while (ls > 0 && H->L[ls - 1].N <= FLD_SMALL_CELLS && nl - (ls - 1) <= FLD_SMALL_MAX) --ls;
+    H->ls = ls;
+    for (int l = 0; l < nl && ok; ++l) {
+        FldLevel& L = H->L[l];
+        const int stride = split_stride(L, H->bc_lo, H->bc_hi);
+        if (l < ls) L.stride = stride;
+        const size_t bytes = es * (L.stride ? 2ull * L.n[1] * L.n[2] * L.stride : (size_t)L.N);
+        for (void** p : {&L.x, &L.b, &L.D}) {
+            if (p == &L.x && l == 0 && !L.stride) continue;    // the caller's Er
+            if (cudaMalloc(p, bytes) != cudaSuccess) ok = false;
+            // padding entries are read (with weight zero) before they are written
+            else if (L.stride && cudaMemsetAsync(*p, 0, bytes, s) != cudaSuccess) ok = false;
+        }
+    }
     if (ok && cudaMalloc(&H->norms, 2 * sizeof(double)) != cudaSuccess) ok = false;
     if (!ok) {
         fld_destroy(H);
@@ -988,7 +1174,7 @@ FldHierarchy* fld_create(const MeshDesc& m, int dtype) {
 void fld_destroy(FldHierarchy* H) {
     if (!H) return;
     for (int l = 0; l < H->nl; ++l) {
-        if (l > 0) cudaFree(H->L[l].x);
+        if (l > 0 || H->L[0].stride) cudaFree(H->L[l].x);
         cudaFree(H->L[l].b);
         cudaFree(H->L[l].D);
     }

@@ -9,9 +9,9 @@ namespace hh {
 struct FldHierarchy;      // grid levels and their device arrays (fld.cu)
 
 // Levels of a mesh: every active axis of even length >= 4 halves, until no
-// axis can (or the level has at most 64 cells).  Allocates the device arrays;
-// returns nullptr on a failed allocation.
-FldHierarchy* fld_create(const MeshDesc& m, int dtype);
+// axis can (or the level has at most 64 cells).  Allocates the device arrays
+// and clears those stored by colour on stream s; nullptr on a failed allocation.
+FldHierarchy* fld_create(const MeshDesc& m, int dtype, cudaStream_t s);
 void fld_destroy(FldHierarchy* H);
 bool fld_matches(const FldHierarchy* H, const MeshDesc& m, int dtype);
 int fld_levels(const FldHierarchy* H);

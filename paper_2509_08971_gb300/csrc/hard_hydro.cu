@@ -678,12 +678,12 @@ int hard_hydro_fld_step(hard_hydro_t h, const void* U, void* Er, double dt, doub
     if (h->mesh.N >= (1ll << 31)) return HARD_EUNSUPPORTED;  // 32-bit cell indices
     // the level kernels take a row per blockIdx.y and a plane per blockIdx.z
     if (h->mesh.n[1] > 65535 || h->mesh.n[2] > 65535) return HARD_EUNSUPPORTED;
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (!hh::fld_matches(h->fld, h->mesh, h->dtype)) {
         hh::fld_destroy(h->fld);
-        h->fld = hh::fld_create(h->mesh, h->dtype);
+        h->fld = hh::fld_create(h->mesh, h->dtype, s);
         if (!h->fld) return HARD_ENOMEM;
     }
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
     h->last = s;
     int cyc = 0;
     double rel = -1.0;
