@@ -26,9 +26,7 @@
 
 namespace hh {
 
-// The face and cell passes are launched as programmatic dependents (pdl.h):
-// each waits for the pass before it on the device and triggers the next one
-// when its loop is done.
+// The face and cell passes are launched as programmatic dependents (pdl.h).
 // The primitive cotangent accumulator holds one 8-slot record per cell (5
 // used), so that FP32 contributions land with one 16-byte vector reduction
 // plus one scalar reduction.
@@ -338,6 +336,7 @@ constexpr int FACES_VJP_THREADS = 128;
 template <typename T, int DIM, int PX, int PY>
 __global__ void __launch_bounds__(FACES_VJP_THREADS, 7) faces_vjp_kernel(const AdjArgs<T> A) {
     griddep_wait();
+    griddep_launch_dependents();
     // 32-bit index arithmetic (the launcher keeps DIM * total below 2^31)
     const unsigned e0 = A.n[0] + 1, e1 = DIM >= 2 ? A.n[1] + 1 : 1, e2 = DIM >= 3 ? A.n[2] + 1 : 1;
     const unsigned total = e0 * e1 * e2;
@@ -358,7 +357,6 @@ __global__ void __launch_bounds__(FACES_VJP_THREADS, 7) faces_vjp_kernel(const A
             if (DIM >= 3 && in0 && in1) face_vjp_one<T, 2, 2>(A, c3, gacc);
         }
     }
-    griddep_launch_dependents();
     // block sum of the explicit d/dgamma, one atomic per block
     __shared__ double red[8];
 #pragma unroll
@@ -383,6 +381,7 @@ __global__ void __launch_bounds__(256) cell_vjp_kernel(const T* Uc, T* gW, const
                                                        long long N, T gamma, double* g_gamma,
                                                        bool clear_gW) {
     griddep_wait();
+    griddep_launch_dependents();
     double gacc = 0.0;
     const T g1 = gamma - T(1);
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
@@ -418,7 +417,6 @@ __global__ void __launch_bounds__(256) cell_vjp_kernel(const T* Uc, T* gW, const
             if (out0) out0[f * N + c] = a * Gc[f];
         }
     }
-    griddep_launch_dependents();
     __shared__ double red[8];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) gacc += __shfl_xor_sync(0xffffffffu, gacc, o);

@@ -12,10 +12,9 @@
 //         r = block max of that rate;  t += dt         (FP64)
 // A problem's cells are evaluated by strip_rows, as on a single 1D or 2D mesh,
 // so a problem advanced here matches the same problem advanced alone bit for
-// bit: the block's warps take strips of 28 cells by a chunk of rows.  State is
-// read through the coherent cache path because the block rewrites it within
-// the launch.  A block never waits on another block: problems are disjoint and
-// the rate reduction is block-local.
+// bit: the block's warps take strips of 28 cells by a chunk of rows.  A block
+// never waits on another block: problems are disjoint and the rate reduction is
+// block-local.
 //
 // What bounds it: instruction issue (strip.cuh).  The FP64 scalars of a
 // problem (widths, dt, t) are one thread's work: a warp's FP64 instruction
@@ -194,12 +193,12 @@ __global__ void __launch_bounds__(32 * NW) batched_kernel(const BatchArgs<T> B) 
                         const unsigned c = it / (unsigned)strips;
                         const int y0 = (int)c * chunk;
                         if (y0 < P.ny)
-                            strip_rows<T, 2, 0, 1, false, 0>(A, (int)(it - c * strips) * STRIP, y0,
+                            strip_rows<T, 2, 0, 1, 0>(A, (int)(it - c * strips) * STRIP, y0,
                                                              min(y0 + chunk, P.ny), acc);
                     }
                 } else {
                     for (int it = warp; it < strips; it += NW)
-                        strip_rows<T, 1, 0, 0, false, 1>(A, it * STRIP, 0, 1, acc);
+                        strip_rows<T, 1, 0, 0, 1>(A, it * STRIP, 0, 1, acc);
                 }
                 if (stage == 2) warp_rate_max(acc.rate_max, red);
                 __syncthreads();            // every cell of this stage written

@@ -10,6 +10,7 @@
 #include "hard_hydro.h"
 #include "launch.h"
 #include "fld_launch.h"
+#include "pdl.h"
 #include "rad_launch.h"
 #include "weno_launch.h"
 
@@ -286,6 +287,8 @@ __device__ void finalize_dt(unsigned long long* slot, double cfl, double t_end, 
 
 __global__ void finalize_dt_kernel(unsigned long long* slot, double cfl, double t_end, double* t,
                                    double* dt_out, double* dt_log, int step, int* status) {
+    hh::griddep_wait();
+    hh::griddep_launch_dependents();
     finalize_dt(slot, cfl, t_end, t, dt_out, dt_log, step, status);
 }
 
@@ -327,6 +330,8 @@ __global__ void finalize_step_kernel(const double* partial, long long rows, doub
                                      double* out5, unsigned long long* slot, double cfl,
                                      double t_end, double* t, double* dt_out, double* dt_log,
                                      int next_step, int* status) {
+    hh::griddep_wait();
+    hh::griddep_launch_dependents();
     if ((threadIdx.x >> 5) < 5) finalize_totals(partial, rows, dV, out5);
     else if (threadIdx.x == 160 && next_step >= 0)
         finalize_dt(slot, cfl, t_end, t, dt_out, dt_log, next_step, status);
@@ -339,8 +344,8 @@ namespace hh {
 cudaError_t launch_finalize_dt(unsigned long long* rs, double cfl, double t_end, double* t_dev,
                                double* dt_dev, double* dt_log, int step, int* status,
                                cudaStream_t s) {
-    finalize_dt_kernel<<<1, 1, 0, s>>>(rs, cfl, t_end, t_dev, dt_dev, dt_log, step, status);
-    return cudaGetLastError();
+    return launch_pdl(finalize_dt_kernel, dim3(1), dim3(1), 0, s, rs, cfl, t_end, t_dev, dt_dev, dt_log,
+                      step, status);
 }
 
 cudaError_t launch_finalize_totals(const double* partial, long long rows, double dV, double* out5,
@@ -354,9 +359,8 @@ cudaError_t launch_finalize_step(const double* partial, long long rows, double d
                                  unsigned long long* rs, double cfl, double t_end, double* t_dev,
                                  double* dt_dev, double* dt_log, int next_step, int* status,
                                  cudaStream_t s) {
-    finalize_step_kernel<<<1, 192, 0, s>>>(partial, rows, dV, out5, rs, cfl, t_end, t_dev, dt_dev,
-                                           dt_log, next_step, status);
-    return cudaGetLastError();
+    return launch_pdl(finalize_step_kernel, dim3(1), dim3(192), 0, s, partial, rows, dV, out5, rs, cfl,
+                      t_end, t_dev, dt_dev, dt_log, next_step, status);
 }
 
 }  // namespace hh

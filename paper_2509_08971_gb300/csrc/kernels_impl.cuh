@@ -10,6 +10,7 @@
 #include "batched.cuh"
 #include "devattr.h"
 #include "launch.h"
+#include "pdl.h"
 #include "stage_kernel.cuh"
 #include "stage_tma.cuh"
 #include "strip.cuh"
@@ -67,8 +68,7 @@ cudaError_t run_stage(const MeshDesc& m, const TileDesc& td, const StageCall& c,
     static std::atomic<unsigned long long> attr{0};
     cudaError_t e = smem_attr_once(kern, smem, attr);
     if (e != cudaSuccess) return e;
-    kern<<<grid, TX * TY, smem, s>>>(A);
-    return cudaGetLastError();
+    return launch_pdl(kern, grid, dim3(TX * TY), smem, s, A);
 }
 
 // 1D and 2D meshes: one warp per strip and td.zc rows (strip.cuh).
@@ -79,8 +79,8 @@ cudaError_t run_strip(const MeshDesc& m, const TileDesc& td, const StageCall& c,
     const long long strips = cdiv(m.n[0], STRIP), warps = strips * cdiv(m.n[1], td.zc);
     const long long blocks = cdiv<long long>(warps, NWARP);
     if (blocks >= (1ll << 31)) return cudaErrorInvalidValue;
-    strip_kernel<T, DIM, PX, PY, RR, NWARP><<<(unsigned)blocks, 32 * NWARP, 0, s>>>(A);
-    return cudaGetLastError();
+    return launch_pdl(strip_kernel<T, DIM, PX, PY, RR, NWARP>, dim3((unsigned)blocks), dim3(32 * NWARP), 0,
+                      s, A);
 }
 
 // ---- TMA path (3D meshes whose rows are 16-byte multiples) ----
@@ -201,9 +201,8 @@ cudaError_t run_stage_tma(const MeshDesc& m, const TileDesc& td, const StageCall
         cudaError_t e = c.stage == 1 ? smem_attr_once(stage_tma_kernel<T, TX, TY, 1>, b1, attr1)
                                      : smem_attr_once(stage_tma_kernel<T, TX, TY, 2>, b2, attr2);
         if (e != cudaSuccess) return e;
-        kern<<<grid, TX * TY, c.stage == 1 ? b1 : b2, s>>>(A, maps);
         used = true;
-        return cudaGetLastError();
+        return launch_pdl(kern, grid, dim3(TX * TY), c.stage == 1 ? b1 : b2, s, A, maps);
     }
 }
 
@@ -261,14 +260,16 @@ cudaError_t run_stage_ws(const MeshDesc& m, const TileDesc& td, const StageCall&
         if (c.stage == 1) {
             e = smem_attr_once(stage_ws_kernel<32, TY, NCW, 1, RPW, TMA>, L1::bytes, attr1);
             if (e != cudaSuccess) return e;
-            stage_ws_kernel<32, TY, NCW, 1, RPW, TMA><<<grid, L1::NT, L1::bytes, s>>>(A, maps);
+            e = launch_pdl(stage_ws_kernel<32, TY, NCW, 1, RPW, TMA>, grid, dim3(L1::NT), L1::bytes, s, A,
+                           maps);
         } else {
             e = smem_attr_once(stage_ws_kernel<32, TY, NCW, 2, RPW, TMA>, L2::bytes, attr2);
             if (e != cudaSuccess) return e;
-            stage_ws_kernel<32, TY, NCW, 2, RPW, TMA><<<grid, L2::NT, L2::bytes, s>>>(A, maps);
+            e = launch_pdl(stage_ws_kernel<32, TY, NCW, 2, RPW, TMA>, grid, dim3(L2::NT), L2::bytes, s, A,
+                           maps);
         }
         used = true;
-        return cudaGetLastError();
+        return e;
     }
 }
 // TMA where the mesh allows it; other meshes whose planes have 32-bit offsets
@@ -294,9 +295,11 @@ __global__ void pointwise_stage_kernel(const T* U0, const T* Uc, T* Uo, long lon
     }
 }
 
-__global__ void rate_kernel(const T* __restrict__ U, long long N, T gamma, T gm1, bool a0,
+__global__ void rate_kernel(const T* U, long long N, T gamma, T gm1, bool a0,
                             bool a1, bool a2, width_t<T> r0, width_t<T> r1, width_t<T> r2, unsigned long long* slot,
                             int* status) {
+    griddep_wait();
+    griddep_launch_dependents();
     const bool act[3] = {a0, a1, a2};
     const width_t<T> rdx[3] = {r0, r1, r2};
     T rmax = T(0);
@@ -305,7 +308,7 @@ __global__ void rate_kernel(const T* __restrict__ U, long long N, T gamma, T gm1
          c += (long long)gridDim.x * blockDim.x) {
         T Uc[NF], W[NF];
 #pragma unroll
-        for (int f = 0; f < NF; ++f) Uc[f] = __ldg(U + f * N + c);
+        for (int f = 0; f < NF; ++f) Uc[f] = *(U + f * N + c);
         cons_to_prim(Uc, gm1, W);
         bad |= nonphys(W);
         T r = cell_rate(W, gamma, act, rdx);
@@ -498,11 +501,10 @@ cudaError_t HH_CAT(launch_rate_, HH_SUFFIX)(const MeshDesc& m, const void* U,
                                              cudaStream_t s) {
     long long blocks = (m.N + 255) / 256;
     if (blocks > 152 * 8) blocks = 152 * 8;
-    rate_kernel<<<(int)blocks, 256, 0, s>>>(
-        static_cast<const T*>(U), m.N, (T)m.gamma, (T)(m.gamma - 1.0), m.act[0], m.act[1],
-        m.act[2], make_width<T>(m.dx[0]), make_width<T>(m.dx[1]), make_width<T>(m.dx[2]), rate_slot,
-        status);
-    return cudaGetLastError();
+    return launch_pdl(rate_kernel, dim3((unsigned)blocks), dim3(256), 0, s, static_cast<const T*>(U), m.N,
+                      (T)m.gamma, (T)(m.gamma - 1.0), m.act[0], m.act[1], m.act[2],
+                      make_width<T>(m.dx[0]), make_width<T>(m.dx[1]), make_width<T>(m.dx[2]), rate_slot,
+                      status);
 }
 
 cudaError_t HH_CAT(launch_totals_, HH_SUFFIX)(const MeshDesc& m, const void* U, double* partial,

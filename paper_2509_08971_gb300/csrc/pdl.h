@@ -1,11 +1,16 @@
 // Programmatic dependent launch (sm_90 and later).  A kernel launched with
 // programmatic stream serialization may begin while the kernel before it in
-// the stream is still running, so its launch latency overlaps that kernel's
-// tail.  Such a kernel calls griddep_wait() before its first access to memory
-// that the previous kernel writes (a hardware wait for that grid to complete
-// and its writes to be visible, not a spin), and griddep_launch_dependents()
-// once it has done its work, which lets the next such kernel be scheduled.
-// Chains of short dependent kernels (the adjoint's passes, the multigrid
+// the stream is still running, so its launch latency and set-up overlap that
+// kernel.  Such a kernel calls griddep_wait() before its first access to memory
+// that an earlier kernel reads or writes (a hardware wait for that grid to complete
+// and its writes to be visible, not a spin), and griddep_launch_dependents() at
+// once after it: the next such kernel may then take free slots of the chip and wait
+// there.  It may not do more than that before this grid is complete, so the
+// trigger's place changes no order.
+// Such a kernel loads what others write with plain loads: not __ldg and not
+// through __restrict__ pointers, which a compiler may move above the wait and the
+// read-only path need not keep coherent while the grids overlap.
+// Chains of short dependent kernels (the time loop, the adjoint's passes, the multigrid
 // levels) lose most of their launch gaps this way.
 #pragma once
 #include <cuda_runtime.h>

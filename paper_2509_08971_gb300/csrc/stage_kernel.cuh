@@ -18,6 +18,7 @@
 // normal momentum component of each sweep.
 #pragma once
 #include "hydro_math.cuh"
+#include "pdl.h"
 #include "tma.cuh"
 
 namespace hh {
@@ -108,7 +109,7 @@ __device__ __forceinline__ void load_prim(const StageArgs<T>& A, int gx, int gy,
     const long long c = ((long long)sz * A.n[1] + sy) * A.n[0] + sx;
     T U[NF];
 #pragma unroll
-    for (int f = 0; f < NF; ++f) U[f] = __ldg(src + f * fstride + c);
+    for (int f = 0; f < NF; ++f) U[f] = *(src + f * fstride + c);
     if (fx) U[1 + PX] = -U[1 + PX];
     if (fy) U[1 + PY] = -U[1 + PY];
     if (fz) U[3] = -U[3];
@@ -329,6 +330,8 @@ template <typename T, int TX, int TY, int PX, int PY>
 __global__ void __launch_bounds__(TX * TY)
 stage_kernel(const StageArgs<T> A) {
     constexpr int NT = TX * TY;
+    griddep_wait();
+    griddep_launch_dependents();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ double red_tot[NT / 32][NF];
     __shared__ unsigned long long red_rate[NT / 32];

@@ -126,6 +126,8 @@ stage_tma_kernel(const __grid_constant__ StageArgs<T> A, const __grid_constant__
                               (px_hi ? L::XS_BYTES : 0) + (py_lo ? L::YS_BYTES : 0) +
                               (py_hi ? L::YS_BYTES : 0);
 
+    griddep_wait();                                   // nothing above reads the state or dt
+    griddep_launch_dependents();
     const T dt = (T)(A.dt_dev ? *A.dt_dev : A.dt);
     const T gamma = A.gamma, gm1 = A.gm1, igm1 = A.igm1;
     constexpr int NPF = HXP * HYP;                    // one field of the primitive plane

@@ -385,6 +385,8 @@ stage_ws_kernel(const __grid_constant__ StageArgs<float> A, const __grid_constan
         s_abort[0] = s_abort[1] = 0;
         if (TMA) prefetch_tmap(&M.main);
     }
+    griddep_wait();                                     // the set-up above reads no state
+    griddep_launch_dependents();
     __syncthreads();
     if (loads) {
         issue(0);

@@ -21,6 +21,7 @@
 // rows per warp, so a problem of a batch equals the same mesh advanced alone
 // bit for bit.
 #pragma once
+#include "pdl.h"
 #include "stage_kernel.cuh"
 
 namespace hh {
@@ -50,7 +51,7 @@ __device__ __forceinline__ void strip_x(const StageArgs<T>& A, const T W[NF], T 
 // issued before any arithmetic and the rows unrolled (small meshes: one memory
 // round trip); RR = 0: a walk of any length with the next row's loads in
 // flight.  1D: y0 = 0, y1 = 1, RR = 1.
-template <typename T, int DIM, int PX, int PY, bool NC, int RR>
+template <typename T, int DIM, int PX, int PY, int RR>
 __device__ __forceinline__ void strip_rows(const StageArgs<T>& A, int xs, int y0, int y1,
                                            TileAcc<T>& acc) {
     const int lane = threadIdx.x & 31;
@@ -63,7 +64,6 @@ __device__ __forceinline__ void strip_rows(const StageArgs<T>& A, int xs, int y0
     const T dt = (T)(A.dt_dev ? *A.dt_dev : A.dt);
     const bool two = A.stage == 2;
 
-    auto get = [](const T* p) { return NC ? __ldg(p) : *p; };
     // conserved state of row j through the boundary map; fly: normal momentum
     // along y changes sign
     auto fetch = [&](int j, T U[NF], bool& fly) {
@@ -71,7 +71,7 @@ __device__ __forceinline__ void strip_rows(const StageArgs<T>& A, int xs, int y0
         const int sy = DIM >= 2 ? bc_map(j, A.n[1], A.bc_lo[1], A.bc_hi[1], fly) : 0;
         const T* p = Uc + (long long)sy * n0;
 #pragma unroll
-        for (int f = 0; f < NF; ++f) U[f] = get(p + f * N);
+        for (int f = 0; f < NF; ++f) U[f] = p[f * N];
     };
     auto prim = [&](T U[NF], bool fly, T W[NF]) {
         if (flx) U[1 + PX] = -U[1 + PX];
@@ -103,7 +103,7 @@ __device__ __forceinline__ void strip_rows(const StageArgs<T>& A, int xs, int y0
     auto fetch0 = [&](int k, T u0[NF]) {
         const T* p = A.U0 + (long long)k * n0 + (own ? gx : 0);
 #pragma unroll
-        for (int f = 0; f < NF; ++f) u0[f] = two && k < y1 ? get(p + f * N) : T(0);
+        for (int f = 0; f < NF; ++f) u0[f] = two && k < y1 ? p[f * N] : T(0);
     };
 
     if constexpr (DIM == 1) {
@@ -230,6 +230,8 @@ __device__ __forceinline__ void strip_epilogue(const StageArgs<T>& A, const Tile
 // One strip of A.zchunk rows per warp, x fastest.
 template <typename T, int DIM, int PX, int PY, int RR, int NWARP>
 __global__ void __launch_bounds__(32 * NWARP) strip_kernel(const StageArgs<T> A) {
+    griddep_wait();
+    griddep_launch_dependents();
     const long long item = (long long)blockIdx.x * NWARP + (threadIdx.x >> 5);
     const int strips = (A.n[0] + STRIP - 1) / STRIP;
     const long long chunk = item / strips;
@@ -240,7 +242,7 @@ __global__ void __launch_bounds__(32 * NWARP) strip_kernel(const StageArgs<T> A)
     for (int f = 0; f < NF; ++f) acc.tot[f] = T(0);
     const long long y0 = chunk * A.zchunk;
     if (y0 < A.n[1])
-        strip_rows<T, DIM, PX, PY, true, RR>(A, (int)(item - chunk * strips) * STRIP, (int)y0,
+        strip_rows<T, DIM, PX, PY, RR>(A, (int)(item - chunk * strips) * STRIP, (int)y0,
                                              min((int)y0 + A.zchunk, A.n[1]), acc);
     strip_epilogue<T, NWARP>(A, acc);
 }

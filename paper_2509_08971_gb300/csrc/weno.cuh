@@ -244,7 +244,7 @@ __device__ __forceinline__ void load_prim3(const StageArgs<T>& A, int gx, int gy
     const long long c = ((long long)sz * A.n[1] + sy) * A.n[0] + sx;
     T U[NF];
 #pragma unroll
-    for (int f = 0; f < NF; ++f) U[f] = __ldg(A.Uc + f * A.N + c);
+    for (int f = 0; f < NF; ++f) U[f] = *(A.Uc + f * A.N + c);
     if (fx) U[1 + PX] = -U[1 + PX];
     if (DIM >= 2 && fy) U[1 + PY] = -U[1 + PY];
     if (DIM >= 3 && fz) U[3] = -U[3];
@@ -267,6 +267,8 @@ struct WenoSmem {
 template <typename T, int TX, int TY, int DIM, int PX, int PY>
 __global__ void __launch_bounds__(TX * TY)
 weno_stage_kernel(const StageArgs<T> A) {
+    griddep_wait();
+    griddep_launch_dependents();
     using S = WenoSmem<T, TX, TY, DIM>;
     constexpr int NT = TX * TY;
     constexpr int HX = S::HX, HY = S::HY;
@@ -555,12 +557,12 @@ __device__ __forceinline__ void load_ev(const AdvectArgs<T>& A, int gx, int gy, 
     if (DIM >= 2) sy = bc_map3(gy, A.n[1], A.bc_lo[1], A.bc_hi[1], fy);
     if (DIM >= 3) sz = bc_map3(gz, A.n[2], A.bc_lo[2], A.bc_hi[2], fz);
     const long long c = ((long long)sz * A.n[1] + sy) * A.n[0] + sx;
-    const T rho = __ldg(A.U + c);
-    T m[3] = {__ldg(A.U + A.N + c), __ldg(A.U + 2 * A.N + c), __ldg(A.U + 3 * A.N + c)};
+    const T rho = *(A.U + c);
+    T m[3] = {*(A.U + A.N + c), *(A.U + 2 * A.N + c), *(A.U + 3 * A.N + c)};
     if (fx) m[PX] = -m[PX];
     if (DIM >= 2 && fy) m[PY] = -m[PY];
     if (DIM >= 3 && fz) m[2] = -m[2];
-    out[0] = __ldg(A.Ec + c);
+    out[0] = *(A.Ec + c);
     out[1] = m[PX] / rho;
     out[2] = DIM >= 2 ? m[PY] / rho : T(0);
     out[3] = DIM >= 3 ? m[2] / rho : T(0);
@@ -591,6 +593,8 @@ struct AdvectSmem {
 // face-by-face form.
 template <typename T, int TX, int TY, int DIM, int PX, int PY>
 __global__ void __launch_bounds__(TX * TY) weno_advect_kernel(const AdvectArgs<T> A) {
+    griddep_wait();
+    griddep_launch_dependents();
     using S = AdvectSmem<T, TX, TY, DIM>;
     constexpr int NT = TX * TY;
     constexpr int HX = S::HX, HY = S::HY, NPF = S::NPF, NQX = S::NQX, NQY = S::NQY;

@@ -3,6 +3,7 @@
 // HH_SUFFIX (f32 or f64) defined.
 #pragma once
 #include "devattr.h"
+#include "pdl.h"
 #include "weno.cuh"
 #include "weno_launch.h"
 #include "weno_sweep.cuh"
@@ -57,8 +58,7 @@ cudaError_t run_weno(const MeshDesc& m, const StageCall& c, cudaStream_t s) {
     static std::atomic<unsigned long long> attr{0};
     const cudaError_t e = smem_attr_once(kern, smem, attr);
     if (e != cudaSuccess) return e;
-    kern<<<grid, TX * TY, smem, s>>>(A);
-    return cudaGetLastError();
+    return launch_pdl(kern, grid, dim3(TX * TY), smem, s, A);
 }
 
 // Grid of a march along kernel axis ax, whose chunk it sets.
@@ -74,16 +74,13 @@ cudaError_t run_weno_sweeps(const MeshDesc& m, const StageCall& c, cudaStream_t 
     T* L = static_cast<T*>(c.scratch);
     if (m.n[1] > 65535 || m.n[2] > 65535) return cudaErrorInvalidValue;
     const dim3 gx(wcdiv(m.n[0], WX_SEG), wcdiv(m.n[1], SWEEP_THREADS / 32), m.n[2]);
-    weno_x_kernel<T, 0><<<gx, SWEEP_THREADS, 0, s>>>(A, L);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_pdl(weno_x_kernel<T, 0>, gx, dim3(SWEEP_THREADS), 0, s, A, L);
     if (e != cudaSuccess) return e;
     const dim3 gy = march_grid(m, 1, A.zchunk);
-    weno_march_kernel<T, 1, 1, false><<<gy, SWEEP_THREADS, 0, s>>>(A, L);
-    e = cudaGetLastError();
+    e = launch_pdl(weno_march_kernel<T, 1, 1, false>, gy, dim3(SWEEP_THREADS), 0, s, A, L);
     if (e != cudaSuccess) return e;
     const dim3 gz = march_grid(m, 2, A.zchunk);
-    weno_march_kernel<T, 2, 2, true><<<gz, SWEEP_THREADS, 0, s>>>(A, L);
-    return cudaGetLastError();
+    return launch_pdl(weno_march_kernel<T, 2, 2, true>, gz, dim3(SWEEP_THREADS), 0, s, A, L);
 }
 
 template <int TX, int TY, int DIM, int PX, int PY>
@@ -95,24 +92,20 @@ cudaError_t run_advect(const MeshDesc& m, const AdvectArgs<T>& A, cudaStream_t s
     static std::atomic<unsigned long long> attr{0};
     const cudaError_t e = smem_attr_once(kern, smem, attr);
     if (e != cudaSuccess) return e;
-    kern<<<grid, TX * TY, smem, s>>>(A);
-    return cudaGetLastError();
+    return launch_pdl(kern, grid, dim3(TX * TY), smem, s, A);
 }
 
 // The three sweeps of one advection stage on a 3D mesh (weno_sweep.cuh).
 cudaError_t run_advect_sweeps(const MeshDesc& m, AdvectArgs<T> A, T* L, cudaStream_t s) {
     if (m.n[1] > 65535 || m.n[2] > 65535) return cudaErrorInvalidValue;
     const dim3 gx(wcdiv(m.n[0], WX_SEG), wcdiv(m.n[1], SWEEP_THREADS / 32), m.n[2]);
-    advect_x_kernel<T, 0><<<gx, SWEEP_THREADS, 0, s>>>(A, L);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_pdl(advect_x_kernel<T, 0>, gx, dim3(SWEEP_THREADS), 0, s, A, L);
     if (e != cudaSuccess) return e;
     const dim3 gy = march_grid(m, 1, A.zchunk);
-    advect_march_kernel<T, 1, 1, false><<<gy, SWEEP_THREADS, 0, s>>>(A, L);
-    e = cudaGetLastError();
+    e = launch_pdl(advect_march_kernel<T, 1, 1, false>, gy, dim3(SWEEP_THREADS), 0, s, A, L);
     if (e != cudaSuccess) return e;
     const dim3 gz = march_grid(m, 2, A.zchunk);
-    advect_march_kernel<T, 2, 2, true><<<gz, SWEEP_THREADS, 0, s>>>(A, L);
-    return cudaGetLastError();
+    return launch_pdl(advect_march_kernel<T, 2, 2, true>, gz, dim3(SWEEP_THREADS), 0, s, A, L);
 }
 
 }  // namespace

@@ -42,7 +42,7 @@ __device__ __forceinline__ void sweep_load(const StageArgs<T>& A, long long base
     const long long c = base + (long long)s * stride;
     T U[NF];
 #pragma unroll
-    for (int f = 0; f < NF; ++f) U[f] = __ldg(A.Uc + f * A.N + c);
+    for (int f = 0; f < NF; ++f) U[f] = *(A.Uc + f * A.N + c);
     if (flip) U[1 + PA] = -U[1 + PA];
     cons_to_prim(U, A.gm1, W);
     bad |= nonphys(W);
@@ -92,7 +92,9 @@ __device__ __forceinline__ void sweep_epilogue(const StageArgs<T>& A, bool bad, 
 // per lane; a block takes one segment of four consecutive rows.  Writes L.
 template <typename T, int PX>
 __global__ void __launch_bounds__(SWEEP_THREADS)
-weno_x_kernel(const StageArgs<T> A, T* __restrict__ L) {
+weno_x_kernel(const StageArgs<T> A, T* L) {
+    griddep_wait();
+    griddep_launch_dependents();
     __shared__ T win[SWEEP_THREADS / 32][NF][WX_WIN];
     const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
     const int n0 = A.n[0], n1 = A.n[1];
@@ -177,7 +179,9 @@ __device__ __forceinline__ long long column_base(long long q, int n0, int n1) {
 #endif
 template <typename T, int AX, int PA, bool LAST>
 __global__ void __launch_bounds__(SWEEP_THREADS, HH_WENO_MINB)
-weno_march_kernel(const StageArgs<T> A, T* __restrict__ L) {
+weno_march_kernel(const StageArgs<T> A, T* L) {
+    griddep_wait();
+    griddep_launch_dependents();
     static_assert(AX == 1 || AX == 2, "the x' axis is the x sweep's");
     const int n0 = A.n[0], n1 = A.n[1];
     const int nA = A.n[AX];
@@ -205,7 +209,7 @@ weno_march_kernel(const StageArgs<T> A, T* __restrict__ L) {
         const int sidx = bc_map3(m, nA, A.bc_lo[AX], A.bc_hi[AX], flip);
         const long long c = base + (long long)sidx * stride;
 #pragma unroll
-        for (int f = 0; f < NF; ++f) U[f] = __ldg(A.Uc + f * N + c);
+        for (int f = 0; f < NF; ++f) U[f] = *(A.Uc + f * N + c);
     };
     // the operands of interior cell k's update: its flux difference so far
     // and, when this sweep combines, its state and U^n
@@ -215,7 +219,7 @@ weno_march_kernel(const StageArgs<T> A, T* __restrict__ L) {
         for (int f = 0; f < NF; ++f) Lk[f] = L[f * N + c];
         if constexpr (LAST) {
 #pragma unroll
-            for (int f = 0; f < NF; ++f) Uk[f] = __ldg(A.Uc + f * N + c);
+            for (int f = 0; f < NF; ++f) Uk[f] = *(A.Uc + f * N + c);
             if (two) {
 #pragma unroll
                 for (int f = 0; f < NF; ++f) U0k[f] = A.U0[f * N + c];
@@ -335,16 +339,18 @@ __device__ __forceinline__ void sweep_ev(const AdvectArgs<T>& A, long long base,
     bool flip;
     const int sidx = bc_map3(m, nA, A.bc_lo[AX], A.bc_hi[AX], flip);
     const long long c = base + (long long)sidx * stride;
-    const T rho = __ldg(A.U + c);
-    T mom = __ldg(A.U + (1 + PA) * A.N + c);
+    const T rho = *(A.U + c);
+    T mom = *(A.U + (1 + PA) * A.N + c);
     if (flip) mom = -mom;
-    e = __ldg(A.Ec + c);
+    e = *(A.Ec + c);
     u = sweep_ratio(mom, rho);
 }
 
 template <typename T, int PX>
 __global__ void __launch_bounds__(SWEEP_THREADS)
-advect_x_kernel(const AdvectArgs<T> A, T* __restrict__ L) {
+advect_x_kernel(const AdvectArgs<T> A, T* L) {
+    griddep_wait();
+    griddep_launch_dependents();
     __shared__ T win[SWEEP_THREADS / 32][2][WX_WIN];
     const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
     const int n0 = A.n[0], n1 = A.n[1];
@@ -387,7 +393,9 @@ advect_x_kernel(const AdvectArgs<T> A, T* __restrict__ L) {
 
 template <typename T, int AX, int PA, bool LAST>
 __global__ void __launch_bounds__(SWEEP_THREADS)
-advect_march_kernel(const AdvectArgs<T> A, T* __restrict__ L) {
+advect_march_kernel(const AdvectArgs<T> A, T* L) {
+    griddep_wait();
+    griddep_launch_dependents();
     static_assert(AX == 1 || AX == 2, "the x' axis is the x sweep's");
     const int n0 = A.n[0], n1 = A.n[1];
     const int nA = A.n[AX];
@@ -413,9 +421,9 @@ advect_march_kernel(const AdvectArgs<T> A, T* __restrict__ L) {
     auto fetch = [&](int m, T& r, T& mo, T& e, bool& flip) {
         const int sidx = bc_map3(m, nA, A.bc_lo[AX], A.bc_hi[AX], flip);
         const long long c = base + (long long)sidx * stride;
-        r = __ldg(A.U + c);
-        mo = __ldg(A.U + (1 + PA) * A.N + c);
-        e = __ldg(A.Ec + c);
+        r = *(A.U + c);
+        mo = *(A.U + (1 + PA) * A.N + c);
+        e = *(A.Ec + c);
     };
     T rn, mn, en, Lk = T(0), E0k = T(0);
     bool fn;
