@@ -336,7 +336,6 @@ constexpr int FACES_VJP_THREADS = 128;
 template <typename T, int DIM, int PX, int PY>
 __global__ void __launch_bounds__(FACES_VJP_THREADS, 7) faces_vjp_kernel(const AdjArgs<T> A) {
     griddep_wait();
-    griddep_launch_dependents();
     // 32-bit index arithmetic (the launcher keeps DIM * total below 2^31)
     const unsigned e0 = A.n[0] + 1, e1 = DIM >= 2 ? A.n[1] + 1 : 1, e2 = DIM >= 3 ? A.n[2] + 1 : 1;
     const unsigned total = e0 * e1 * e2;
@@ -381,7 +380,6 @@ __global__ void __launch_bounds__(256) cell_vjp_kernel(const T* Uc, T* gW, const
                                                        long long N, T gamma, double* g_gamma,
                                                        bool clear_gW) {
     griddep_wait();
-    griddep_launch_dependents();
     double gacc = 0.0;
     const T g1 = gamma - T(1);
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;

@@ -197,7 +197,6 @@ constexpr int FLD_FINE_ROWS = HH_FLD_FINE_ROWS;       // and on level 0
 template <typename T, int SR>
 __global__ void __launch_bounds__(128) smooth_kernel(const LvlArgs<T> a, int color, int lg) {
     griddep_wait();
-    griddep_launch_dependents();
     const int k = blockIdx.z;
     const int p = blockIdx.x * (1 << lg) + (threadIdx.x & ((1 << lg) - 1));
     const int j0 = (blockIdx.y * (128 >> lg) + (threadIdx.x >> lg)) * SR;
@@ -247,7 +246,6 @@ __global__ void __launch_bounds__(128) residual_restrict_kernel(const LvlArgs<T>
                                                                 int nc0, int nc1, int h0, int h1,
                                                                 int h2) {
     griddep_wait();
-    griddep_launch_dependents();
     const int J = blockIdx.y, K = blockIdx.z;
     const int I = blockIdx.x * blockDim.x + threadIdx.x;
     if (I >= nc0) return;
@@ -307,7 +305,6 @@ __global__ void __launch_bounds__(128) residual_restrict_kernel(const LvlArgs<T>
 template <typename T>
 __global__ void __launch_bounds__(128) residual_norms_kernel(const LvlArgs<T> a, double* norms) {
     griddep_wait();
-    griddep_launch_dependents();
     __shared__ double sr[4], sb[4];
     double rr = 0.0, bb = 0.0;
     const int segs = (a.n[0] + 127) / 128;
@@ -384,7 +381,6 @@ template <typename T>
 __global__ void __launch_bounds__(128) residual_norm_color_kernel(const LvlArgs<T> a, int color,
                                                                   double* norms) {
     griddep_wait();
-    griddep_launch_dependents();
     const int k = blockIdx.z;
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     StencilVals<T> v[SMOOTH_ROWS];
@@ -548,7 +544,7 @@ template <typename T>
 __global__ void __launch_bounds__(FLD_SMALL_THREADS)
 small_vcycle_kernel(const __grid_constant__ SmallLevels<T> S) {
     griddep_wait();
-    griddep_launch_dependents();
+    griddep_launch_dependents();         // one block: the chip is free for the next grid's
     extern __shared__ __align__(16) unsigned char fld_smem[];
     T* sm = reinterpret_cast<T*>(fld_smem);
     for (int l = 0; l < S.count; ++l) {
@@ -594,50 +590,30 @@ small_vcycle_kernel(const __grid_constant__ SmallLevels<T> S) {
         __syncthreads();
     }
     // the coarsest level: red-black sweeps until a sweep changes nothing
-    // (every later sweep would return the same values) or `coarse` sweeps.
-    // One warp sweeps a level of at most 64 cells: the barriers between its
-    // half-sweeps are a warp's, not a block's.
+    // (every later sweep would return the same values) or `coarse` sweeps
     {
         __shared__ int changed[2];
         const int lc = S.count - 1;
         const LvlArgs<T> s = small_level(S, sm, lc);
         const int N = (int)s.N, n0 = s.n[0], n1 = s.n[1];
-        const bool one = N <= 64;
-        const int step = one ? 32 : (int)blockDim.x;
-        auto half = [&](int color) {
-            bool ch = false;
-            for (int q = threadIdx.x; q < N; q += step) {
-                const int t = small_div(q, S.mg[lc][0], n0), i = q - t * n0;
-                const int k = small_div(t, S.mg[lc][1], n1), j = t - k * n1;
-                if (((i + j + k) & 1) != color) continue;
-                T diag, off;
-                stencil(s, i, j, k, q, diag, off);
-                const T nx = (s.b[q] + off) / diag;
-                ch |= !(nx == s.x[q]);                       // also NaN: keep sweeping
-                s.x[q] = nx;
-            }
-            return ch;
-        };
-        if (one) {
-            if (threadIdx.x < 32)
-                for (int it = 0; it < S.coarse; ++it) {
-                    bool ch = half(0);
-                    __syncwarp();
-                    ch |= half(1);
-                    if (!__any_sync(0xffffffffu, ch)) break;
+        if (threadIdx.x == 0) changed[0] = 0;
+        __syncthreads();
+        for (int it = 0; it < S.coarse; ++it) {
+            for (int color = 0; color < 2; ++color) {
+                if (color == 1 && threadIdx.x == 0) changed[(it + 1) & 1] = 0;
+                for (int q = threadIdx.x; q < N; q += blockDim.x) {
+                    const int t = small_div(q, S.mg[lc][0], n0), i = q - t * n0;
+                    const int k = small_div(t, S.mg[lc][1], n1), j = t - k * n1;
+                    if (((i + j + k) & 1) != color) continue;
+                    T diag, off;
+                    stencil(s, i, j, k, q, diag, off);
+                    const T nx = (s.b[q] + off) / diag;
+                    if (!(nx == s.x[q])) changed[it & 1] = 1;    // also NaN: keep sweeping
+                    s.x[q] = nx;
                 }
-            __syncthreads();
-        } else {
-            if (threadIdx.x == 0) changed[0] = 0;
-            __syncthreads();
-            for (int it = 0; it < S.coarse; ++it) {
-                if (half(0)) changed[it & 1] = 1;
                 __syncthreads();
-                if (threadIdx.x == 0) changed[(it + 1) & 1] = 0;
-                if (half(1)) changed[it & 1] = 1;
-                __syncthreads();
-                if (!changed[it & 1]) break;                 // the same value in every thread
             }
+            if (!changed[it & 1]) break;          // the same value in every thread
         }
     }
     // up: add the coarse correction to the children, smooth
@@ -686,7 +662,6 @@ template <typename T>
 __global__ void __launch_bounds__(128) prolong_kernel(T* fine, const T* coarse, int nf0, int nf1,
                                                       int nc0, int nc1, int h0, int h1, int h2) {
     griddep_wait();
-    griddep_launch_dependents();
     const int k = blockIdx.z;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nf0) return;
@@ -1094,13 +1069,17 @@ cudaError_t solve_t(FldHierarchy* H, const MeshDesc& m, const void* U, void* Er,
 
 // Row length of a level stored by colour, 0 for mesh order: where red and
 // black is no proper two-colouring (an odd periodic axis), for rows too short
-// to fill a vector, and beyond 32-bit entries.
+// to fill a vector, beyond 32-bit entries, and for small levels, whose
+// half-sweeps are a launch's latency and want one cell per thread (FP32 half-sweep
+// by colour against mesh order: 128^3 6.4 / 8.9 us, 64^3 3.1 / 3.4, 32^3 2.8 / 2.8; 67 x 45 x 11
+// ~15 % slower by colour).
+constexpr long long FLD_SPLIT_CELLS = 1 << 17;
 int split_stride(const FldLevel& L, const int* bc_lo, const int* bc_hi) {
     for (int ax = 0; ax < 3; ++ax)
         if (L.n[ax] > 1 && bc_lo[ax] == HARD_BC_PERIODIC && bc_hi[ax] == HARD_BC_PERIODIC && (L.n[ax] & 1))
             return 0;
     const int stride = ((L.n[0] + 1) / 2 + 3) / 4 * 4;
-    return L.n[0] < 8 || 2ll * L.n[1] * L.n[2] * stride >= (1ll << 31) ? 0 : stride;
+    return L.N < FLD_SPLIT_CELLS || L.n[0] < 8 || 2ll * L.n[1] * L.n[2] * stride >= (1ll << 31) ? 0 : stride;
 }
 
 }  // namespace

@@ -13,12 +13,13 @@
 // row's last cell repeats its first (x and D), so that the shifted neighbours
 // of a vector need no wrap of their own.  Other padding stays zero.
 //
-// Only for levels whose periodic axes are even (a proper two-colouring).
+// Only for levels whose periodic axes are even (a proper two-colouring), of
+// FLD_SPLIT_CELLS cells at least.
 //
 // What bounds it: memory.  A half-sweep of a 256^3 FP32 level moves 168 MB (x
 // of one colour, b and x of the other, D of both) in 34 us against 242 MB in 52 us
 // in mesh order; the prolongation corrects one colour only (19 us against 36), the
-// residual norm takes 34 us (53), the step to 1e-5 (four cycles) 2.27 ms (3.13).
+// residual norm takes 34 us (53), the step to 1e-5 (four cycles) 2.23 ms (3.11).
 #pragma once
 #include <type_traits>
 
@@ -241,7 +242,7 @@ __device__ __forceinline__ void split_store(const SplitArgs<T>& a, int c, int j,
 template <typename T, bool WALLS>
 __global__ void __launch_bounds__(128, 4) split_smooth_kernel(const SplitArgs<T> a, int c, int chunk) {
     griddep_wait();
-    griddep_launch_dependents();
+    if (griddep_many_blocks()) griddep_launch_dependents();
     constexpr int V = VecOf<T>::V;
     int p0, j;
     if (split_column(a, p0, j)) {
@@ -262,7 +263,7 @@ template <typename T, bool WALLS>
 __global__ void __launch_bounds__(128) split_norm_kernel(const SplitArgs<T> a, int c, int chunk,
                                                          double* out) {
     griddep_wait();
-    griddep_launch_dependents();
+    if (griddep_many_blocks()) griddep_launch_dependents();
     constexpr int V = VecOf<T>::V;
     T sum = T(0);
     int p0, j;
@@ -313,7 +314,7 @@ template <typename T, bool WALLS>
 __global__ void __launch_bounds__(128) split_restrict_kernel(const SplitArgs<T> a, CellArray<T> cb,
                                                              CellArray<T> cx, int h1, int h2) {
     griddep_wait();
-    griddep_launch_dependents();
+    if (griddep_many_blocks()) griddep_launch_dependents();
     constexpr int V = VecOf<T>::V;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int J = t / a.groups, p0 = (t - J * a.groups) * V, K = blockIdx.y;
@@ -348,7 +349,7 @@ __global__ void __launch_bounds__(128) split_restrict_x_kernel(const SplitArgs<T
                                                                CellArray<T> cb, CellArray<T> cx,
                                                                int h1, int h2) {
     griddep_wait();
-    griddep_launch_dependents();
+    if (griddep_many_blocks()) griddep_launch_dependents();
     constexpr int V = VecOf<T>::V;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int J = t / a.n[0], i = t - J * a.n[0], K = blockIdx.y;
@@ -380,7 +381,7 @@ template <typename T>
 __global__ void __launch_bounds__(128) split_prolong_kernel(const SplitArgs<T> a, CellArray<T> cx,
                                                             int h0, int h1, int h2) {
     griddep_wait();
-    griddep_launch_dependents();
+    if (griddep_many_blocks()) griddep_launch_dependents();
     constexpr int V = VecOf<T>::V;
     int p0, j;
     if (split_column(a, p0, j)) {
@@ -404,7 +405,7 @@ __global__ void __launch_bounds__(128) split_prolong_kernel(const SplitArgs<T> a
 template <typename T>
 __global__ void __launch_bounds__(128) split_merge_kernel(const SplitArgs<T> a, T* E, bool wide) {
     griddep_wait();
-    griddep_launch_dependents();
+    if (griddep_many_blocks()) griddep_launch_dependents();
     constexpr int V = VecOf<T>::V;
     int p0, j;
     if (!split_column(a, p0, j)) return;

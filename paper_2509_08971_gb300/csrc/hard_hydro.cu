@@ -288,7 +288,6 @@ __device__ void finalize_dt(unsigned long long* slot, double cfl, double t_end, 
 __global__ void finalize_dt_kernel(unsigned long long* slot, double cfl, double t_end, double* t,
                                    double* dt_out, double* dt_log, int step, int* status) {
     hh::griddep_wait();
-    hh::griddep_launch_dependents();
     finalize_dt(slot, cfl, t_end, t, dt_out, dt_log, step, status);
 }
 
@@ -331,7 +330,6 @@ __global__ void finalize_step_kernel(const double* partial, long long rows, doub
                                      double t_end, double* t, double* dt_out, double* dt_log,
                                      int next_step, int* status) {
     hh::griddep_wait();
-    hh::griddep_launch_dependents();
     if ((threadIdx.x >> 5) < 5) finalize_totals(partial, rows, dV, out5);
     else if (threadIdx.x == 160 && next_step >= 0)
         finalize_dt(slot, cfl, t_end, t, dt_out, dt_log, next_step, status);

@@ -299,7 +299,6 @@ __global__ void rate_kernel(const T* U, long long N, T gamma, T gm1, bool a0,
                             bool a1, bool a2, width_t<T> r0, width_t<T> r1, width_t<T> r2, unsigned long long* slot,
                             int* status) {
     griddep_wait();
-    griddep_launch_dependents();
     const bool act[3] = {a0, a1, a2};
     const width_t<T> rdx[3] = {r0, r1, r2};
     T rmax = T(0);

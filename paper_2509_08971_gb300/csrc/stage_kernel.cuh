@@ -331,7 +331,6 @@ __global__ void __launch_bounds__(TX * TY)
 stage_kernel(const StageArgs<T> A) {
     constexpr int NT = TX * TY;
     griddep_wait();
-    griddep_launch_dependents();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ double red_tot[NT / 32][NF];
     __shared__ unsigned long long red_rate[NT / 32];

@@ -231,7 +231,6 @@ __device__ __forceinline__ void strip_epilogue(const StageArgs<T>& A, const Tile
 template <typename T, int DIM, int PX, int PY, int RR, int NWARP>
 __global__ void __launch_bounds__(32 * NWARP) strip_kernel(const StageArgs<T> A) {
     griddep_wait();
-    griddep_launch_dependents();
     const long long item = (long long)blockIdx.x * NWARP + (threadIdx.x >> 5);
     const int strips = (A.n[0] + STRIP - 1) / STRIP;
     const long long chunk = item / strips;

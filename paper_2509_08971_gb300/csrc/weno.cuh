@@ -268,7 +268,6 @@ template <typename T, int TX, int TY, int DIM, int PX, int PY>
 __global__ void __launch_bounds__(TX * TY)
 weno_stage_kernel(const StageArgs<T> A) {
     griddep_wait();
-    griddep_launch_dependents();
     using S = WenoSmem<T, TX, TY, DIM>;
     constexpr int NT = TX * TY;
     constexpr int HX = S::HX, HY = S::HY;
@@ -594,7 +593,6 @@ struct AdvectSmem {
 template <typename T, int TX, int TY, int DIM, int PX, int PY>
 __global__ void __launch_bounds__(TX * TY) weno_advect_kernel(const AdvectArgs<T> A) {
     griddep_wait();
-    griddep_launch_dependents();
     using S = AdvectSmem<T, TX, TY, DIM>;
     constexpr int NT = TX * TY;
     constexpr int HX = S::HX, HY = S::HY, NPF = S::NPF, NQX = S::NQX, NQY = S::NQY;

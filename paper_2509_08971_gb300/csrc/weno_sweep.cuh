@@ -94,7 +94,6 @@ template <typename T, int PX>
 __global__ void __launch_bounds__(SWEEP_THREADS)
 weno_x_kernel(const StageArgs<T> A, T* L) {
     griddep_wait();
-    griddep_launch_dependents();
     __shared__ T win[SWEEP_THREADS / 32][NF][WX_WIN];
     const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
     const int n0 = A.n[0], n1 = A.n[1];
@@ -181,7 +180,6 @@ template <typename T, int AX, int PA, bool LAST>
 __global__ void __launch_bounds__(SWEEP_THREADS, HH_WENO_MINB)
 weno_march_kernel(const StageArgs<T> A, T* L) {
     griddep_wait();
-    griddep_launch_dependents();
     static_assert(AX == 1 || AX == 2, "the x' axis is the x sweep's");
     const int n0 = A.n[0], n1 = A.n[1];
     const int nA = A.n[AX];
@@ -350,7 +348,6 @@ template <typename T, int PX>
 __global__ void __launch_bounds__(SWEEP_THREADS)
 advect_x_kernel(const AdvectArgs<T> A, T* L) {
     griddep_wait();
-    griddep_launch_dependents();
     __shared__ T win[SWEEP_THREADS / 32][2][WX_WIN];
     const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
     const int n0 = A.n[0], n1 = A.n[1];
@@ -395,7 +392,6 @@ template <typename T, int AX, int PA, bool LAST>
 __global__ void __launch_bounds__(SWEEP_THREADS)
 advect_march_kernel(const AdvectArgs<T> A, T* L) {
     griddep_wait();
-    griddep_launch_dependents();
     static_assert(AX == 1 || AX == 2, "the x' axis is the x sweep's");
     const int n0 = A.n[0], n1 = A.n[1];
     const int nA = A.n[AX];
