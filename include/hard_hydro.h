@@ -388,6 +388,30 @@ int hard_hydro_fld_step(hard_hydro_t h, const void* U, void* Er, double dt, doub
 int hard_hydro_step_backward(hard_hydro_t h, const void* U_in, const void* gU_out, void* gU_in,
                              double dt, double* g_gamma, void* stream);
 
+/* ---- rollouts: a sequence of steps in one call ----
+ * hard_hydro_steps advances U_in through n steps of the given lengths, the
+ * state after step i in out[i] (an input of step i + 1: out[i] may not be
+ * out[i - 1]; older buffers may be used again).  hard_hydro_steps_backward
+ * applies hard_hydro_step_backward for i = n-1 .. 0 with states[i] the input of
+ * step i, in place on gU.  The arrays are host memory; the errors are those of
+ * the single calls, all lengths checked before the first step. */
+int hard_hydro_steps(hard_hydro_t h, const void* U_in, void* const* out, const double* dts, int n,
+                     void* stream);
+int hard_hydro_steps_backward(hard_hydro_t h, const void* const* states, void* gU,
+                              const double* dts, int n, double* g_gamma, void* stream);
+
+/* Device memory that the caller lends a handle in place of the scratch that it
+ * would allocate with cudaMalloc and free in hard_hydro_destroy: adjoint = 0 what
+ * hard_hydro_step needs (the intermediate stage and the status), adjoint = 1 what
+ * hard_hydro_step_backward needs besides.  hard_hydro_workspace_bytes returns the
+ * size for the handle's mesh and element type (negative: an error code);
+ * hard_hydro_set_workspace takes 16-byte aligned memory of at least that size and
+ * clears on `stream` what has to start at zero (the status among it).  The memory
+ * stays the caller's: it has to outlive the handle's work on every stream, until
+ * the handle is destroyed, given other memory or set to the other element type. */
+long long hard_hydro_workspace_bytes(hard_hydro_t h, int adjoint);
+int hard_hydro_set_workspace(hard_hydro_t h, int adjoint, void* mem, long long bytes, void* stream);
+
 /* Device status flag: returns HARD_OK, HARD_ENONPHYS (a non-physical state
  * was met) or HARD_ETIMEOUT (a bounded wait of a TMA-fed stage ran out and
  * that stage left its output incomplete), and clears the flag.  Synchronises

@@ -66,6 +66,10 @@ def _declare(lib):
         "hard_hydro_step_noalloc": (ctypes.c_int, [_vp, _vp, _vp, ctypes.c_double, _vp]),
         "hard_hydro_step_backward": (ctypes.c_int, [_vp, _vp, _vp, _vp, ctypes.c_double, _vp,
                                                     _vp]),
+        "hard_hydro_steps": (ctypes.c_int, [_vp, _vp, _vp, _dp, ctypes.c_int, _vp]),
+        "hard_hydro_steps_backward": (ctypes.c_int, [_vp, _vp, _vp, _dp, ctypes.c_int, _vp, _vp]),
+        "hard_hydro_workspace_bytes": (ctypes.c_longlong, [_vp, ctypes.c_int]),
+        "hard_hydro_set_workspace": (ctypes.c_int, [_vp, ctypes.c_int, _vp, ctypes.c_longlong, _vp]),
         "hard_hydro_get_error": (ctypes.c_int, [_vp]),
         "hard_hydro_noalloc_get_error": (ctypes.c_int, []),
         "hard_hydro_set_cells": (ctypes.c_int, [_vp, ctypes.c_double, ctypes.c_double,
@@ -290,6 +294,31 @@ def hard_hydro_step_backward(h, U_in, gU_out, gU_in, dt, g_gamma, stream):
     return lib().hard_hydro_step_backward(h, U_in, gU_out, gU_in, float(dt), g_gamma, stream)
 
 
+def _rollout_arrays(pointers, dts):
+    n = len(dts)
+    if len(pointers) != n:
+        raise ValueError("one buffer per step")
+    return (ctypes.c_void_p * n)(*pointers), (ctypes.c_double * n)(*[float(dt) for dt in dts]), n
+
+
+def hard_hydro_steps(h, U_in, out, dts, stream):
+    out, dts, n = _rollout_arrays(out, dts)
+    return lib().hard_hydro_steps(h, U_in, out, dts, n, stream)
+
+
+def hard_hydro_steps_backward(h, states, gU, dts, g_gamma, stream):
+    states, dts, n = _rollout_arrays(states, dts)
+    return lib().hard_hydro_steps_backward(h, states, gU, dts, n, g_gamma, stream)
+
+
+def hard_hydro_workspace_bytes(h, adjoint):
+    return lib().hard_hydro_workspace_bytes(h, int(adjoint))
+
+
+def hard_hydro_set_workspace(h, adjoint, mem, nbytes, stream):
+    return lib().hard_hydro_set_workspace(h, int(adjoint), mem, int(nbytes), stream)
+
+
 def hard_hydro_get_error(h):
     return lib().hard_hydro_get_error(h)
 
@@ -453,6 +482,15 @@ class HardHydro:
                                        self._check(out), dt, g_gamma.data_ptr(), self._stream()),
               "hard_hydro_step_backward")
         return out
+
+    def workspace(self, adjoint, device):
+        """A buffer of the caching allocator lent to the handle as scratch; the
+        caller keeps it as long as the handle uses it."""
+        n = hard_hydro_workspace_bytes(self.h, adjoint)
+        mem = self.torch.empty(n, dtype=self.torch.uint8, device=device)
+        check(hard_hydro_set_workspace(self.h, adjoint, mem.data_ptr(), n, self._stream()),
+              "hard_hydro_set_workspace")
+        return mem
 
     def get_error(self):
         return hard_hydro_get_error(self.h)

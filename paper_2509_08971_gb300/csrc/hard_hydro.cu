@@ -43,6 +43,7 @@ struct hard_hydro_s {
     void* adj = nullptr;             // adjoint scratch: primitive cotangent | stage-1 cotangent
     size_t adj_bytes = 0;
     hh::FldHierarchy* fld = nullptr; // radiation diffusion multigrid levels, on first use
+    bool lent[2] = {false, false};   // slots and U1 / adj are the caller's (hard_hydro_set_workspace)
     cudaStream_t last = nullptr;
 };
 
@@ -113,10 +114,12 @@ void build_mesh(hard_hydro_s* h) {
 void free_scratch(hard_hydro_s* h) {
     hh::fld_destroy(h->fld);
     h->fld = nullptr;
-    if (h->adj) cudaFree(h->adj);
+    if (h->lent[0]) h->slots = nullptr;
+    if (h->adj && !h->lent[1]) cudaFree(h->adj);
     h->adj = nullptr;
     h->adj_bytes = 0;
-    if (h->U1) cudaFree(h->U1);
+    if (h->U1 && !h->lent[0]) cudaFree(h->U1);
+    h->lent[0] = h->lent[1] = false;
     if (h->wL) cudaFree(h->wL);
     h->wL = nullptr;
     h->wL_bytes = 0;
@@ -169,8 +172,10 @@ int ensure_U1(hard_hydro_s* h) {
 // Adjoint scratch: the primitive cotangent accumulator (8 slots per cell,
 // zero between calls: zeroed here once, cleared by each cell pass) and the
 // cotangent of the intermediate stage.
+size_t adj_gw_bytes(const hard_hydro_s* h) { return 8 * (size_t)h->mesh.N * elem_size(h); }
+
 int ensure_adj(hard_hydro_s* h) {
-    const size_t gw_bytes = 8 * (size_t)h->mesh.N * elem_size(h);
+    const size_t gw_bytes = adj_gw_bytes(h);
     const size_t need = gw_bytes + state_bytes(h);
     if (h->adj && h->adj_bytes >= need) return HARD_OK;
     if (h->adj) cudaFree(h->adj);
@@ -736,6 +741,64 @@ int hard_hydro_step_backward(hard_hydro_t h, const void* U_in, const void* gU_ou
     e = h->dtype == HARD_F64 ? hh::launch_adjoint_stage_f64(h->mesh, a1, s)
                              : hh::launch_adjoint_stage_f32(h->mesh, a1, s);
     return from_cuda(e);
+}
+
+static bool valid_lengths(const double* dts, int n) {
+    for (int i = 0; i < n; ++i)
+        if (!(dts[i] > 0.0) || !std::isfinite(dts[i])) return false;
+    return true;
+}
+
+int hard_hydro_steps(hard_hydro_t h, const void* U_in, void* const* out, const double* dts, int n,
+                     void* stream) {
+    if (!h || !U_in || n < 0 || (n > 0 && (!out || !dts))) return HARD_EINVAL;
+    if (!valid_lengths(dts, n)) return HARD_EINVAL;
+    const void* U = U_in;
+    for (int i = 0; i < n; ++i) {
+        if (out[i] == U) return HARD_EINVAL;
+        const int rc = hard_hydro_step(h, U, out[i], dts[i], stream);
+        if (rc) return rc;
+        U = out[i];
+    }
+    return HARD_OK;
+}
+
+int hard_hydro_steps_backward(hard_hydro_t h, const void* const* states, void* gU,
+                              const double* dts, int n, double* g_gamma, void* stream) {
+    if (!h || !gU || !g_gamma || n < 0 || (n > 0 && (!states || !dts))) return HARD_EINVAL;
+    if (!valid_lengths(dts, n)) return HARD_EINVAL;
+    for (int i = n - 1; i >= 0; --i) {
+        const int rc = hard_hydro_step_backward(h, states[i], gU, gU, dts[i], g_gamma, stream);
+        if (rc) return rc;
+    }
+    return HARD_OK;
+}
+
+long long hard_hydro_workspace_bytes(hard_hydro_t h, int adjoint) {
+    if (!h || (adjoint != 0 && adjoint != 1)) return HARD_EINVAL;
+    return adjoint ? (long long)(adj_gw_bytes(h) + state_bytes(h)) : (long long)(256 + state_bytes(h));
+}
+
+int hard_hydro_set_workspace(hard_hydro_t h, int adjoint, void* mem, long long bytes, void* stream) {
+    const long long need = hard_hydro_workspace_bytes(h, adjoint);
+    if (need < 0 || !mem || !aligned16(mem) || bytes < need) return HARD_EINVAL;
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    if (adjoint) {
+        if (h->adj && !h->lent[1]) cudaFree(h->adj);
+        h->adj = mem;
+        h->adj_bytes = (size_t)need;
+        h->lent[1] = true;
+        return from_cuda(cudaMemsetAsync(mem, 0, adj_gw_bytes(h), s));
+    }
+    if (!h->lent[0]) {
+        if (h->slots) cudaFree(h->slots);
+        if (h->U1) cudaFree(h->U1);
+    }
+    h->slots = static_cast<unsigned char*>(mem);
+    h->U1 = h->slots + 256;
+    h->U1_bytes = state_bytes(h);
+    h->lent[0] = true;
+    return from_cuda(cudaMemsetAsync(mem, 0, 256, s));
 }
 
 int hard_hydro_set_cells(hard_hydro_t h, double dx, double dy, double dz) {
