@@ -61,9 +61,11 @@ __device__ __forceinline__ double div_by(double a, double b, double y, bool ok) 
 }
 
 // A cell width as the kernels divide by it: FP64 the width and RN(1 / width)
-// (0 where the short division must not be used), FP32 1 / width.
+// (0 where the short division must not be used), `exact` for a power of two;
+// FP32 1 / width.
 struct Width64 {
     double w, inv;
+    int exact;
 };
 template <typename T> struct WidthOf { using type = float; };
 template <> struct WidthOf<double> { using type = Width64; };
@@ -72,7 +74,9 @@ template <typename T> using width_t = typename WidthOf<T>::type;
 template <typename T> inline __host__ __device__ width_t<T> make_width(double dx);
 template <> inline __host__ __device__ float make_width<float>(double dx) { return (float)(1.0 / dx); }
 template <> inline __host__ __device__ Width64 make_width<double>(double dx) {
-    return Width64{dx, dx > 1e-150 && dx < 1e150 ? 1.0 / dx : 0.0};
+    const bool mid = dx > 1e-150 && dx < 1e150;
+    int e;
+    return Width64{dx, mid ? 1.0 / dx : 0.0, mid && frexp(dx, &e) == 0.5};
 }
 
 // ---------------------------------------------------------------- minmod --
@@ -108,6 +112,17 @@ __device__ __forceinline__ double sub_over_dx(double acc, double diff, const Wid
 }
 __device__ __forceinline__ float sub_over_dx(float acc, float diff, float inv_dx) {
     return fmaf(-diff, inv_dx, acc);
+}
+
+// The same on 3D meshes, whose FP64 kernels fill the pipe: a quotient by a power
+// of two is the product with its reciprocal, one operation instead of three
+// (128^3, two steps: 12.89 -> 12.2 ms).  1D and 2D strips, bound by their
+// chains, lose 1-2 % by the test.
+__device__ __forceinline__ double sub_over_dx3(double acc, double diff, const Width64& dx) {
+    return dx.exact ? acc - diff * dx.inv : sub_over_dx(acc, diff, dx);
+}
+__device__ __forceinline__ float sub_over_dx3(float acc, float diff, float inv_dx) {
+    return sub_over_dx(acc, diff, inv_dx);
 }
 
 // ------------------------------------------------------- closure helpers --

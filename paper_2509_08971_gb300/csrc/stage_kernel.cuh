@@ -254,9 +254,9 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, unsigned char*
             for (int f = 0; f < NF; ++f) {
                 qj[f] = Ps[(f * HY + ty + 2) * HX + tx + 2];
                 T a = Fx[(f * TY + ty) * (TX + 1) + tx + 1] - Fx[(f * TY + ty) * (TX + 1) + tx];
-                Dj[f] = sub_over_dx(T(0), a, A.dxk[0]);
+                Dj[f] = sub_over_dx3(T(0), a, A.dxk[0]);
                 T b = Fy[(f * (TY + 1) + ty + 1) * TX + tx] - Fy[(f * (TY + 1) + ty) * TX + tx];
-                Dj[f] = sub_over_dx(Dj[f], b, A.dxk[1]);
+                Dj[f] = sub_over_dx3(Dj[f], b, A.dxk[1]);
             }
         } else {
             // warm-up / look-ahead plane: only this column's primitives
@@ -284,7 +284,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, unsigned char*
         const int k = cnt >= 4 ? j - 2 : -1;                             // the cell completed
         if (k >= 0) {
 #pragma unroll
-            for (int f = 0; f < NF; ++f) L[f] = sub_over_dx(Da[f], Fz[f] - Fzp[f], A.dxk[2]);
+            for (int f = 0; f < NF; ++f) L[f] = sub_over_dx3(Da[f], Fz[f] - Fzp[f], A.dxk[2]);
         }
 #pragma unroll
         for (int f = 0; f < NF; ++f) {

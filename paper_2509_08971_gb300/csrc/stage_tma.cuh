@@ -368,8 +368,8 @@ stage_tma_kernel(const __grid_constant__ StageArgs<T> A, const __grid_constant__
             for (int f = 0; f < NF; ++f) {
                 const T a = Fx[(f * TY + ty) * (TX + 1) + tx + 1] - Fown_x[f];
                 const T b = Fy[(f * (TY + 1) + ty + 1) * TX + tx] - Fown_y[f];
-                Dj[f] = sub_over_dx(T(0), a, A.dxk[0]);
-                Dj[f] = sub_over_dx(Dj[f], b, A.dxk[1]);
+                Dj[f] = sub_over_dx3(T(0), a, A.dxk[0]);
+                Dj[f] = sub_over_dx3(Dj[f], b, A.dxk[1]);
             }
             if (own) bad |= nonphys(qj);
         } else {
@@ -395,7 +395,7 @@ stage_tma_kernel(const __grid_constant__ StageArgs<T> A, const __grid_constant__
             T Uo[NF];
 #pragma unroll
             for (int f = 0; f < NF; ++f) {
-                const T Lf = sub_over_dx(Da[f], Fz[f] - Fzp[f], A.dxk[2]);
+                const T Lf = sub_over_dx3(Da[f], Fz[f] - Fzp[f], A.dxk[2]);
                 const T uc = Sk[(f * HYC + ty + 2) * HXC + tx + 4];
                 Uo[f] = STAGE == 1
                             ? madd(dt, Lf, uc)
