@@ -51,3 +51,6 @@ def test_fld_levels(shape, bc):
         cyc2, _ = m.fld_step(Ud, again, dt, C, KAPPA, rtol=rtol, max_cycles=200)
         err = float((again.double() - first.double()).norm() / first.double().norm())
         assert cyc2 == cyc and err <= tol, (dtype, cyc, cyc2, err)
+        # no half-sweep reads what it writes, unless a periodic axis is odd
+        if bc != 0 or all(n == 1 or n % 2 == 0 for n in shape):
+            assert torch.equal(again, first), dtype
