@@ -73,8 +73,10 @@ cudaError_t run_weno_sweeps(const MeshDesc& m, const StageCall& c, cudaStream_t 
     StageArgs<T> A = weno_args(m, 1, c);
     T* L = static_cast<T*>(c.scratch);
     if (m.n[1] > 65535 || m.n[2] > 65535) return cudaErrorInvalidValue;
-    const dim3 gx(wcdiv(m.n[0], WX_SEG), wcdiv(m.n[1], SWEEP_THREADS / 32), m.n[2]);
-    cudaError_t e = launch_pdl(weno_x_kernel<T, 0>, gx, dim3(SWEEP_THREADS), 0, s, A, L);
+    const int cells = wx_cells(m.n[0]);
+    const dim3 gx(wcdiv(m.n[0], 32 * cells - 2), wcdiv(m.n[1], SWEEP_THREADS / 32), m.n[2]);
+    auto kx = cells == 3 ? weno_x_kernel<T, 0, 3> : weno_x_kernel<T, 0, 2>;
+    cudaError_t e = launch_pdl(kx, gx, dim3(SWEEP_THREADS), 0, s, A, L);
     if (e != cudaSuccess) return e;
     const dim3 gy = march_grid(m, 1, A.zchunk);
     e = launch_pdl(weno_march_kernel<T, 1, 1, false>, gy, dim3(SWEEP_THREADS), 0, s, A, L);
@@ -98,8 +100,10 @@ cudaError_t run_advect(const MeshDesc& m, const AdvectArgs<T>& A, cudaStream_t s
 // The three sweeps of one advection stage on a 3D mesh (weno_sweep.cuh).
 cudaError_t run_advect_sweeps(const MeshDesc& m, AdvectArgs<T> A, T* L, cudaStream_t s) {
     if (m.n[1] > 65535 || m.n[2] > 65535) return cudaErrorInvalidValue;
-    const dim3 gx(wcdiv(m.n[0], WX_SEG), wcdiv(m.n[1], SWEEP_THREADS / 32), m.n[2]);
-    cudaError_t e = launch_pdl(advect_x_kernel<T, 0>, gx, dim3(SWEEP_THREADS), 0, s, A, L);
+    const int cells = wx_cells(m.n[0]);
+    const dim3 gx(wcdiv(m.n[0], 32 * cells - 2), wcdiv(m.n[1], SWEEP_THREADS / 32), m.n[2]);
+    auto kx = cells == 3 ? advect_x_kernel<T, 0, 3> : advect_x_kernel<T, 0, 2>;
+    cudaError_t e = launch_pdl(kx, gx, dim3(SWEEP_THREADS), 0, s, A, L);
     if (e != cudaSuccess) return e;
     const dim3 gy = march_grid(m, 1, A.zchunk);
     e = launch_pdl(advect_march_kernel<T, 1, 1, false>, gy, dim3(SWEEP_THREADS), 0, s, A, L);

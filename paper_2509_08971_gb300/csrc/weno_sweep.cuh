@@ -12,11 +12,11 @@
 // The sweeps serve 3D meshes (1D and 2D meshes, small enough to be bound by
 // launch latency, keep the fused kernel).  Each sweep reconstructs the two
 // face values of every cell once (weno5z_pair) and evaluates every face's
-// HLL flux once.  The x sweep gives each warp a 62-cell segment of a row:
-// lane l holds cells x_s - 1 + 2l and x_s + 2l, the window of their
+// HLL flux once.  The x sweep gives each warp a segment of a row: lane l holds
+// two or three cells from x_s - 1 + 2l or 3l on, the window of their
 // five-cell stencils sits in shared memory, and the face between two lanes
-// takes its left state from the lower lane by a shuffle.  The marches give each lane one x column and
-// walk the march axis with the five-cell stencil, the pending face state and
+// takes its left state from the lower lane by a shuffle.  The marches give each
+// lane one column and walk the march axis with the five-cell stencil, the pending face state and
 // the last face flux in registers: no block barrier and no shared plane.
 // Against the fused kernel this moves L through HBM between the sweeps
 // (about three times the state traffic) to cut the instructions per cell:
@@ -27,8 +27,10 @@
 
 namespace hh {
 
-constexpr int WX_SEG = 62;                    // cells per warp in the x sweeps (two per lane)
-constexpr int WX_WIN = WX_SEG + 6;            // their stencil window
+// The x sweeps' segments with C cells per lane: cells a warp completes, and their
+// stencil window.
+template <int C> constexpr int WX_SEG = 32 * C - 2;
+template <int C> constexpr int WX_WIN = 32 * C + 4;
 constexpr int SWEEP_THREADS = WENO_SWEEP_THREADS;
 
 // Conserved -> primitive of cell m along kernel axis AX (extent nA, element
@@ -88,72 +90,76 @@ __device__ __forceinline__ void sweep_epilogue(const StageArgs<T>& A, bool bad, 
     }
 }
 
-// x sweep: one warp per 62-cell segment of a row (y', z' fixed), two cells
-// per lane; a block takes one segment of four consecutive rows.  Writes L.
-template <typename T, int PX>
+// x sweep: one warp per segment of WX_SEG cells of a row (y', z' fixed), C cells
+// per lane (wx_cells); a block takes one segment of four consecutive rows.
+// Writes L.
+template <typename T, int PX, int C>
 __global__ void __launch_bounds__(SWEEP_THREADS)
 weno_x_kernel(const StageArgs<T> A, T* L) {
     griddep_wait();
-    __shared__ T win[SWEEP_THREADS / 32][NF][WX_WIN];
+    __shared__ T win[SWEEP_THREADS / 32][NF][WX_WIN<C>];
     const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
     const int n0 = A.n[0], n1 = A.n[1];
     // segment blockIdx.x of rows y' = 4 blockIdx.y + warp, z' = blockIdx.z
     const int yr = blockIdx.y * (SWEEP_THREADS / 32) + wq;
     const bool active = yr < n1;                       // warp-uniform
     const long long base = ((long long)blockIdx.z * n1 + (active ? yr : 0)) * n0;
-    const int xs = blockIdx.x * WX_SEG;
+    const int xs = blockIdx.x * WX_SEG<C>;
     const T gamma = A.gamma;
     const T gx = sizeof(T) == 4 ? A.igm1 : A.gm1;     // the HLL energy closure
     bool bad = false;                                  // reported by the combining sweep
 
-    // the window: cells xs-3 .. xs+64 (lane l loads cells xs-3+l and
-    // xs+29+l, and lanes 0..3 also cell xs+61+l)
+    // the window: cells xs-3 .. xs+32C (lane l loads cells xs-3+32h+l, and
+    // lanes 0..3 also cell xs-3+32C+l)
     {
         T W[NF];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < C; ++h) {
             sweep_load<T, 0, PX>(A, base, xs - 3 + 32 * h + lane, n0, 1, W, bad);
 #pragma unroll
             for (int f = 0; f < NF; ++f) win[wq][f][32 * h + lane] = W[f];
         }
-        if (lane < WX_WIN - 64) {
-            sweep_load<T, 0, PX>(A, base, xs + 61 + lane, n0, 1, W, bad);
+        if (lane < 4) {
+            sweep_load<T, 0, PX>(A, base, xs - 3 + 32 * C + lane, n0, 1, W, bad);
 #pragma unroll
-            for (int f = 0; f < NF; ++f) win[wq][f][64 + lane] = W[f];
+            for (int f = 0; f < NF; ++f) win[wq][f][32 * C + lane] = W[f];
         }
     }
     __syncwarp();
-    // lane l: cells c0 = xs-1+2l and c1 = c0+1, their stencils win[2l .. 2l+4]
-    // and win[2l+1 .. 2l+5]; the face left of c0 takes its left state from
-    // c1 of lane l-1, the face right of c1 is lane l+1's face left of its c0
-    T rv0[NF], lv0[NF], rv1[NF], lv1[NF];
+    // lane l: cells c_k = xs-1+Cl+k, their stencils win[Cl+k .. Cl+k+4]; the face
+    // left of c_0 takes its left state from the last cell of lane l-1, the face
+    // right of the last cell is lane l+1's face left of its c_0
+    T rv[C][NF], lv[C][NF];
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
-        const T* v = &win[wq][f][2 * lane];
-        weno5z_pair(v[0], v[1], v[2], v[3], v[4], rv0[f], lv0[f]);
-        weno5z_pair(v[1], v[2], v[3], v[4], v[5], rv1[f], lv1[f]);
+        const T* v = &win[wq][f][C * lane];
+#pragma unroll
+        for (int k = 0; k < C; ++k)
+            weno5z_pair(v[k], v[k + 1], v[k + 2], v[k + 3], v[k + 4], rv[k][f], lv[k][f]);
     }
-    T qL[NF], Fl[NF], Fm[NF];
+    T qL[NF], F[NF], Fn[NF], F0[NF];
 #pragma unroll
-    for (int f = 0; f < NF; ++f) qL[f] = __shfl_up_sync(0xffffffffu, rv1[f], 1);
-    hll_face<PX>(qL, lv0, gamma, gx, Fl);              // face c0 - 1/2
-    hll_face<PX>(rv0, lv1, gamma, gx, Fm);             // face c0 + 1/2
-    T D0[NF], D1[NF];
+    for (int f = 0; f < NF; ++f) qL[f] = __shfl_up_sync(0xffffffffu, rv[C - 1][f], 1);
+    hll_face<PX>(qL, lv[0], gamma, gx, F);             // face c_0 - 1/2
 #pragma unroll
-    for (int f = 0; f < NF; ++f) {
-        const T Fr = __shfl_down_sync(0xffffffffu, Fl[f], 1);   // face c1 + 1/2
-        D0[f] = sub_over_dx(T(0), Fm[f] - Fl[f], A.dxk[0]);
-        D1[f] = sub_over_dx(T(0), Fr - Fm[f], A.dxk[0]);
-    }
-    // cells xs .. xs+61: c1 of lanes 0..30, c0 of lanes 1..31
-    const int x0 = xs - 1 + 2 * lane;
-    if (active && lane >= 1 && x0 < n0) {
+    for (int f = 0; f < NF; ++f) F0[f] = F[f];
+    // cells xs .. xs+32C-3: all but c_0 of lane 0 and the last of lane 31
+    const int x0 = xs - 1 + C * lane;
 #pragma unroll
-        for (int f = 0; f < NF; ++f) L[f * A.N + base + x0] = D0[f];
-    }
-    if (active && lane <= 30 && x0 + 1 < n0) {
+    for (int k = 0; k < C; ++k) {
+        if (k + 1 < C) {
+            hll_face<PX>(rv[k], lv[k + 1 < C ? k + 1 : 0], gamma, gx, Fn);
+        } else {
 #pragma unroll
-        for (int f = 0; f < NF; ++f) L[f * A.N + base + x0 + 1] = D1[f];
+            for (int f = 0; f < NF; ++f) Fn[f] = __shfl_down_sync(0xffffffffu, F0[f], 1);
+        }
+        const bool mine = active && x0 + k < n0 && (k > 0 || lane >= 1) && (k + 1 < C || lane <= 30);
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+            const T D = sub_over_dx(T(0), Fn[f] - F[f], A.dxk[0]);
+            if (mine) L[f * A.N + base + x0 + k] = D;
+            F[f] = Fn[f];
+        }
     }
 }
 
@@ -344,48 +350,54 @@ __device__ __forceinline__ void sweep_ev(const AdvectArgs<T>& A, long long base,
     u = sweep_ratio(mom, rho);
 }
 
-template <typename T, int PX>
+template <typename T, int PX, int C>
 __global__ void __launch_bounds__(SWEEP_THREADS)
 advect_x_kernel(const AdvectArgs<T> A, T* L) {
     griddep_wait();
-    __shared__ T win[SWEEP_THREADS / 32][2][WX_WIN];
+    __shared__ T win[SWEEP_THREADS / 32][2][WX_WIN<C>];
     const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
     const int n0 = A.n[0], n1 = A.n[1];
     const int yr = blockIdx.y * (SWEEP_THREADS / 32) + wq;     // as in weno_x_kernel
     const bool active = yr < n1;
     const long long base = ((long long)blockIdx.z * n1 + (active ? yr : 0)) * n0;
-    const int xs = blockIdx.x * WX_SEG;
+    const int xs = blockIdx.x * WX_SEG<C>;
     {
         T e, u;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < C; ++h) {
             sweep_ev<T, 0, PX>(A, base, xs - 3 + 32 * h + lane, n0, 1, e, u);
             win[wq][0][32 * h + lane] = e;
             win[wq][1][32 * h + lane] = u;
         }
-        if (lane < WX_WIN - 64) {
-            sweep_ev<T, 0, PX>(A, base, xs + 61 + lane, n0, 1, e, u);
-            win[wq][0][64 + lane] = e;
-            win[wq][1][64 + lane] = u;
+        if (lane < 4) {
+            sweep_ev<T, 0, PX>(A, base, xs - 3 + 32 * C + lane, n0, 1, e, u);
+            win[wq][0][32 * C + lane] = e;
+            win[wq][1][32 * C + lane] = u;
         }
     }
     __syncwarp();
-    // two cells per lane, as in weno_x_kernel
-    const T* ve = &win[wq][0][2 * lane];
-    const T* vu = &win[wq][1][2 * lane];
-    T er0, el0, ur0, ul0, er1, el1, ur1, ul1;
-    weno5z_pair(ve[0], ve[1], ve[2], ve[3], ve[4], er0, el0);
-    weno5z_pair(vu[0], vu[1], vu[2], vu[3], vu[4], ur0, ul0);
-    weno5z_pair(ve[1], ve[2], ve[3], ve[4], ve[5], er1, el1);
-    weno5z_pair(vu[1], vu[2], vu[3], vu[4], vu[5], ur1, ul1);
-    const T eL = __shfl_up_sync(0xffffffffu, er1, 1), uL = __shfl_up_sync(0xffffffffu, ur1, 1);
-    const T Fl = rusanov_e(eL, el0, uL, ul0);                   // face c0 - 1/2
-    const T Fm = rusanov_e(er0, el1, ur0, ul1);                 // face c0 + 1/2
-    const T Fr = __shfl_down_sync(0xffffffffu, Fl, 1);          // face c1 + 1/2
-    const int x0 = xs - 1 + 2 * lane;
-    if (active && lane >= 1 && x0 < n0) L[base + x0] = sub_over_dx(T(0), Fm - Fl, A.dxk[0]);
-    if (active && lane <= 30 && x0 + 1 < n0)
-        L[base + x0 + 1] = sub_over_dx(T(0), Fr - Fm, A.dxk[0]);
+    // C cells per lane, as in weno_x_kernel
+    const T* ve = &win[wq][0][C * lane];
+    const T* vu = &win[wq][1][C * lane];
+    T er[C], el[C], ur[C], ul[C];
+#pragma unroll
+    for (int k = 0; k < C; ++k) {
+        weno5z_pair(ve[k], ve[k + 1], ve[k + 2], ve[k + 3], ve[k + 4], er[k], el[k]);
+        weno5z_pair(vu[k], vu[k + 1], vu[k + 2], vu[k + 3], vu[k + 4], ur[k], ul[k]);
+    }
+    const T eL = __shfl_up_sync(0xffffffffu, er[C - 1], 1), uL = __shfl_up_sync(0xffffffffu, ur[C - 1], 1);
+    const T F0 = rusanov_e(eL, el[0], uL, ul[0]);               // face c_0 - 1/2
+    T F = F0;
+    const int x0 = xs - 1 + C * lane;
+#pragma unroll
+    for (int k = 0; k < C; ++k) {
+        const int k1 = k + 1 < C ? k + 1 : 0;
+        const T Fn = k + 1 < C ? rusanov_e(er[k], el[k1], ur[k], ul[k1])
+                               : __shfl_down_sync(0xffffffffu, F0, 1);
+        if (active && x0 + k < n0 && (k > 0 || lane >= 1) && (k + 1 < C || lane <= 30))
+            L[base + x0 + k] = sub_over_dx(T(0), Fn - F, A.dxk[0]);
+        F = Fn;
+    }
 }
 
 template <typename T, int AX, int PA, bool LAST>

@@ -51,10 +51,31 @@ def test_rows_of_any_length(shape, bc):
             assert torch.allclose(tot[-1], want, rtol=1e-6, atol=1e-6), (dtype, tile)
 
 
-@pytest.mark.parametrize("shape", [(3, 3, 3), (4, 5, 127), (9, 3, 43), (30, 6, 130), (75, 7, 20)])
+# rows at the edges of the x sweeps' segments (62 and 94 cells), columns that are
+# no multiple of a block, rows shared by blocks, one and several chunks
+SWEEPS = [(3, 3, 3), (4, 5, 127), (9, 3, 43), (30, 6, 130), (75, 7, 20), (3, 4, 62), (3, 5, 63), (4, 3, 94),
+          (3, 3, 95), (3, 4, 187), (3, 3, 189)]
+
+
+@pytest.mark.parametrize("shape", SWEEPS)
 @pytest.mark.parametrize("bc", [0, 1, 2])
-def test_weno_marches(shape, bc):
-    """Columns that are no multiple of a block, rows shared by blocks, one and several chunks."""
+def test_advect_sweeps(shape, bc):
+    gam = 1.4
+    U = _state(shape, gam)
+    E = 1.0 + 0.5 * np.random.default_rng(4).random(shape)
+    g = oracle.Grid(shape, gam, bc)
+    dt = 0.3 / g.max_rate(U)
+    ref = g.advect_E(U, E, dt)
+    for dtype, tol in ((torch.float64, 1e-12), (torch.float32, 3e-6)):   # one step of O(30) roundings
+        m = hh.HardHydro(shape, gam, bc, dtype=dtype)
+        Ed = torch.tensor(E, dtype=dtype, device="cuda")
+        m.advect_E(torch.tensor(U, dtype=dtype, device="cuda"), Ed, dt)
+        assert np.abs(Ed.double().cpu().numpy() - ref).max() <= tol * np.abs(ref).max(), dtype
+
+
+@pytest.mark.parametrize("shape", SWEEPS)
+@pytest.mark.parametrize("bc", [0, 1, 2])
+def test_weno_sweeps(shape, bc):
     gam = 1.4
     U = _state(shape, gam)
     ref, _, _ = oracle.Grid(shape, gam, bc, scheme=1).run(U, 2, 0.3)
