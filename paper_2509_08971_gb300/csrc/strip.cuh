@@ -14,7 +14,7 @@
 // small meshes the latency of one strip.  It replaces a 32 x 8 tile per block
 // (primitives and both face fluxes through shared memory, two barriers, every
 // slope twice): 757 issue slots per cell-stage there.  Measured, bit-identical: 4096 batched
-// problems, five steps, 15.45 -> 10.52 ms; 100 FP64 steps of a 400-cell mesh
+// problems, five steps, 15.45 -> 10.40 ms; 100 FP64 steps of a 400-cell mesh
 // (15 SMs instead of 4) 4.73 -> 3.09 ms; 50 FP32 steps at 256^2 0.92 -> 0.84 ms.
 //
 // strip_rows evaluates the same expressions in the same order whatever the
@@ -180,7 +180,7 @@ __device__ __forceinline__ void strip_rows(const StageArgs<T>& A, int xs, int y0
             T Un[NF];
             bool fn;
             fetch(y0 - 2, Un, fn);
-#pragma unroll 2
+#pragma unroll 1       // by two: 4096 batched problems 10.53 ms, one by one 10.40
             for (int r = y0 - 2; r <= y1 + 1; ++r) {
                 T U[NF], u0[NF];
                 const bool fl = fn;
