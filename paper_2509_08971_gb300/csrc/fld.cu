@@ -1107,7 +1107,9 @@ cudaError_t solve_t(FldHierarchy* H, const MeshDesc& m, const void* U, void* Er,
 
 // Row length of a level stored by colour, 0 for mesh order: where red and
 // black is no proper two-colouring (an odd periodic axis), for rows too short
-// to fill a vector, beyond 32-bit entries, and for small levels, whose
+// to fill a vector, beyond 32-bit entries (and then every level below, since the
+// kernels of a level in mesh order take the next one in mesh order), and for small
+// levels, whose
 // half-sweeps are a launch's latency and want one cell per thread (FP32 half-sweep
 // by colour against mesh order: 128^3 6.4 / 8.9 us, 64^3 3.1 / 3.4, 32^3 2.8 / 2.8; 67 x 45 x 11
 // ~15 % slower by colour).
@@ -1170,7 +1172,7 @@ FldHierarchy* fld_create(const MeshDesc& m, int dtype, cudaStream_t s) {
     for (int l = 0; l < nl && ok; ++l) {
         FldLevel& L = H->L[l];
         const int stride = split_stride(L, H->bc_lo, H->bc_hi);
-        if (l < ls) L.stride = stride;
+        if (l < ls && (l == 0 || H->L[l - 1].stride)) L.stride = stride;
         const size_t bytes = es * (L.stride ? 2ull * L.n[1] * L.n[2] * L.stride : (size_t)L.N);
         for (void** p : {&L.x, &L.b, &L.D}) {
             if (p == &L.x && l == 0 && !L.stride) continue;    // the caller's Er
