@@ -179,10 +179,6 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) batched_kernel(const BatchAr
             __syncthreads();
             const double dt = s_dt;
             TileAcc<T> acc;
-            acc.rate_max = T(0);
-            acc.bad = false;
-#pragma unroll
-            for (int f = 0; f < NF; ++f) acc.tot[f] = T(0);
 #pragma unroll 1
             for (int stage = 1; stage <= 2; ++stage) {
                 StageArgs<T> A = batch_stage_args<T>(P, sc, U, W, stage, dt);

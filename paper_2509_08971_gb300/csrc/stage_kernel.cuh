@@ -117,13 +117,41 @@ __device__ __forceinline__ void load_prim(const StageArgs<T>& A, int gx, int gy,
     bad |= nonphys(W);
 }
 
+// A lane's sum of a field over the cells it completes.  FP32 keeps the rounding error
+// of each addition (Knuth's two-sum, The Art of Computer Programming vol. 2, 4.2.2) in a
+// second word, so the totals are as good as summed in FP64 whatever the cells per lane:
+// seven FP32 operations a field, where FP64 additions and conversions would hold the
+// SM's FP64 pipe as long as the rest of the cell takes to issue.  add_down (Dekker's
+// fast two-sum, four operations) keeps all of the error where |x| does not exceed the
+// sum's magnitude, as in a column of like cells, and else at least what a plain
+// addition does.
+template <typename T>
+struct LaneSum {
+    T s = T(0);
+    __device__ __forceinline__ void add(T x) { s += x; }
+};
+template <>
+struct LaneSum<float> {
+    float s = 0.f, err = 0.f;
+    __device__ __forceinline__ void add(float x) {
+        const float t = s + x, b = t - s;
+        err += (s - (t - b)) + (x - b);
+        s = t;
+    }
+    __device__ __forceinline__ void add_down(float x) {
+        const float t = s + x;
+        err += x - (t - s);
+        s = t;
+    }
+};
+
 // What a block accumulates over the cells it completes: the largest signal
 // rate, the conserved totals and the non-physical flag.
 template <typename T>
 struct TileAcc {
-    T rate_max;
-    T tot[NF];
-    bool bad;
+    T rate_max = T(0);
+    LaneSum<T> tot[NF];
+    bool bad = false;
 };
 
 // Warp sum of the five per-lane FP64 totals as a reduce-scatter butterfly:
@@ -133,43 +161,60 @@ struct TileAcc {
 // warp's total of field sum5_field(lane) in the lanes where sum5_writer(lane)
 // holds: field 0 in lane 0, 1 in lane 4, 2 in lane 8, 3 in lane 16, 4 in
 // lane 24.  The order of the additions is fixed, so the sum is deterministic.
-__device__ __forceinline__ double warp_sum5(const double v[NF], int lane) {
+template <typename V>
+__device__ __forceinline__ V warp_sum5(const V v[NF], int lane) {
     const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
     // offset 16: lanes 0-15 keep fields 0, 1, 2; lanes 16-31 keep 3, 4
-    double a0 = h16 ? v[3] : v[0];
-    double a1 = h16 ? v[4] : v[1];
-    double a2 = h16 ? 0.0 : v[2];
-    const double s0 = h16 ? v[0] : v[3];
-    const double s1 = h16 ? v[1] : v[4];
-    const double s2 = h16 ? v[2] : 0.0;
+    V a0 = h16 ? v[3] : v[0];
+    V a1 = h16 ? v[4] : v[1];
+    V a2 = h16 ? V(0) : v[2];
+    const V s0 = h16 ? v[0] : v[3];
+    const V s1 = h16 ? v[1] : v[4];
+    const V s2 = h16 ? v[2] : V(0);
     a0 += __shfl_xor_sync(0xffffffffu, s0, 16);
     a1 += __shfl_xor_sync(0xffffffffu, s1, 16);
     a2 += __shfl_xor_sync(0xffffffffu, s2, 16);
     // offset 8: lanes 0-7 keep fields 0, 1; 8-15 field 2; 16-23 field 3;
     // 24-31 field 4
-    double c0, c1, t0, t1;
+    V c0, c1, t0, t1;
     if (!h16) {
         c0 = h8 ? a2 : a0;
-        c1 = h8 ? 0.0 : a1;
+        c1 = h8 ? V(0) : a1;
         t0 = h8 ? a0 : a2;
-        t1 = h8 ? a1 : 0.0;
+        t1 = h8 ? a1 : V(0);
     } else {
         c0 = h8 ? a1 : a0;
-        c1 = 0.0;
+        c1 = V(0);
         t0 = h8 ? a0 : a1;
-        t1 = 0.0;
+        t1 = V(0);
     }
     c0 += __shfl_xor_sync(0xffffffffu, t0, 8);
     c1 += __shfl_xor_sync(0xffffffffu, t1, 8);
     // offset 4: lanes 0-3 keep field 0, 4-7 field 1; every other lane holds
     // one field already and adds its partner's share of it
     const bool two = !h16 && !h8;
-    double k = (two && h4) ? c1 : c0;
-    const double t = two ? (h4 ? c0 : c1) : c0;
+    V k = (two && h4) ? c1 : c0;
+    const V t = two ? (h4 ? c0 : c1) : c0;
     k += __shfl_xor_sync(0xffffffffu, t, 4);
     k += __shfl_xor_sync(0xffffffffu, k, 2);
     k += __shfl_xor_sync(0xffffffffu, k, 1);
     return k;
+}
+// The same of lane sums, in FP64; the error words, a 2^-24th of the sums, in FP32.
+// ERR = false: lanes of one cell, which have none.
+template <bool ERR = true, typename T>
+__device__ __forceinline__ double warp_totals(const LaneSum<T> tot[NF], int lane) {
+    double v[NF];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) v[f] = (double)tot[f].s;
+    double s = warp_sum5(v, lane);
+    if constexpr (ERR && sizeof(T) == 4) {
+        float e[NF];
+#pragma unroll
+        for (int f = 0; f < NF; ++f) e[f] = tot[f].err == tot[f].err ? tot[f].err : 0.f;   // none of an infinite sum
+        s += (double)warp_sum5(e, lane);
+    }
+    return s;
 }
 __device__ __forceinline__ int sum5_field(int lane) {
     return (lane & 16) ? ((lane & 8) ? 4 : 3) : ((lane & 8) ? 2 : ((lane & 4) ? 1 : 0));
@@ -317,7 +362,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, unsigned char*
             }
             if (A.tot_partial) {
 #pragma unroll
-                for (int f = 0; f < NF; ++f) acc.tot[f] += Uo[f];
+                for (int f = 0; f < NF; ++f) acc.tot[f].add(Uo[f]);
             }
         }
     }
@@ -340,16 +385,9 @@ stage_kernel(const StageArgs<T> A) {
     const int z0 = A.zlo + blockIdx.z * A.zchunk;
     const int z1 = min(z0 + A.zchunk, A.zhi);
     TileAcc<T> acc;
-    acc.rate_max = T(0);
-    acc.bad = false;
-#pragma unroll
-    for (int f = 0; f < NF; ++f) acc.tot[f] = T(0);
     stage_tile<T, TX, TY, PX, PY>(A, smem_raw, x0, y0, z0, z1, acc);
     const T rate_max = acc.rate_max;
     const bool bad = acc.bad;
-    T tot[NF];
-#pragma unroll
-    for (int f = 0; f < NF; ++f) tot[f] = acc.tot[f];
 
     // ---- epilogue: block reductions ----
     const int lane = tid & 31, warp = tid >> 5;
@@ -363,10 +401,7 @@ stage_kernel(const StageArgs<T> A) {
         if (lane == 0) red_rate[warp] = b;
     }
     if (A.tot_partial) {
-        double v[NF];
-#pragma unroll
-        for (int f = 0; f < NF; ++f) v[f] = (double)tot[f];
-        const double s = warp_sum5(v, lane);
+        const double s = warp_totals(acc.tot, lane);
         if (sum5_writer(lane)) red_tot[warp][sum5_field(lane)] = s;
     }
     const int any_bad = __syncthreads_or(bad);

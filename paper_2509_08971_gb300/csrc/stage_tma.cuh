@@ -182,7 +182,7 @@ stage_tma_kernel(const __grid_constant__ StageArgs<T> A, const __grid_constant__
 
     bool bad = false;
     T rate_max = T(0);
-    T tot[NF] = {T(0), T(0), T(0), T(0), T(0)};
+    LaneSum<T> tot[NF];
     T qm1[NF], dprev[NF], qLp[NF], Fzp[NF], Da[NF], Db[NF];
 #pragma unroll
     for (int f = 0; f < NF; ++f) qm1[f] = dprev[f] = qLp[f] = Fzp[f] = Da[f] = Db[f] = T(0);
@@ -412,7 +412,7 @@ stage_tma_kernel(const __grid_constant__ StageArgs<T> A, const __grid_constant__
             }
             if (EPI && A.tot_partial) {
 #pragma unroll
-                for (int f = 0; f < NF; ++f) tot[f] += Uo[f];
+                for (int f = 0; f < NF; ++f) tot[f].add(Uo[f]);
             }
         }
 #pragma unroll
@@ -448,10 +448,7 @@ stage_tma_kernel(const __grid_constant__ StageArgs<T> A, const __grid_constant__
         if (lane == 0) red_rate[warp] = b;
     }
     if (EPI && A.tot_partial) {
-        double v[NF];
-#pragma unroll
-        for (int f = 0; f < NF; ++f) v[f] = (double)tot[f];
-        const double s = warp_sum5(v, lane);
+        const double s = warp_totals(tot, lane);
         if (sum5_writer(lane)) red_tot[warp][sum5_field(lane)] = s;
     }
     const int any_bad = __syncthreads_or(bad);

@@ -425,7 +425,7 @@ stage_ws_kernel(const __grid_constant__ StageArgs<float> A, const __grid_constan
         for (int f = 0; f < NF; ++f) qn[r][f] = dn[r][f] = qLz[r][f] = Fzb[r][f] = 0.f;
     bool bad = false;
     float rate_max = 0.f;
-    float tot[NF] = {0.f, 0.f, 0.f, 0.f, 0.f};
+    LaneSum<float> tot[NF];
 
     // One iteration (see the schedule above); returns true when a bounded
     // wait ran out somewhere in the block (every thread returns the same).
@@ -585,7 +585,7 @@ stage_ws_kernel(const __grid_constant__ StageArgs<float> A, const __grid_constan
                             }
                             if (EPI && A.tot_partial) {
 #pragma unroll
-                                for (int f = 0; f < NF; ++f) tot[f] += own[r] ? Uo[f] : 0.f;
+                                for (int f = 0; f < NF; ++f) tot[f].add_down(RPW == 1 || own[r] ? Uo[f] : 0.f);
                             }
                         }
 #pragma unroll
@@ -736,10 +736,10 @@ stage_ws_kernel(const __grid_constant__ StageArgs<float> A, const __grid_constan
         if (lane == 0) red_rate[warp] = b;
     }
     if (EPI && A.tot_partial && facew) {
-        double v[NF];
+        if (RPW == 1 && !own[0])                        // a lane's row is its own or it is not
 #pragma unroll
-        for (int f = 0; f < NF; ++f) v[f] = (double)tot[f];
-        const double s = warp_sum5(v, lane);
+            for (int f = 0; f < NF; ++f) tot[f] = LaneSum<float>();
+        const double s = warp_totals(tot, lane);
         if (sum5_writer(lane)) red_tot[warp][sum5_field(lane)] = s;
     }
     const int any_bad = __syncthreads_or(bad);

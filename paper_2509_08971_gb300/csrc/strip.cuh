@@ -97,7 +97,7 @@ __device__ __forceinline__ void strip_rows(const StageArgs<T>& A, int xs, int y0
         }
         if (A.tot_partial) {
 #pragma unroll
-            for (int f = 0; f < NF; ++f) acc.tot[f] += Uo[f];
+            for (int f = 0; f < NF; ++f) acc.tot[f].add(Uo[f]);
         }
     };
     auto fetch0 = [&](int k, T u0[NF]) {
@@ -196,7 +196,7 @@ __device__ __forceinline__ void strip_rows(const StageArgs<T>& A, int xs, int y0
 
 // Block reductions of what the block's warps accumulated: the non-physical
 // flag, the rate maximum, and the block's row of the totals partial array.
-template <typename T, int NWARP>
+template <typename T, int NWARP, bool ERR>
 __device__ __forceinline__ void strip_epilogue(const StageArgs<T>& A, const TileAcc<T>& acc) {
     __shared__ double red_tot[NWARP][NF];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -212,10 +212,7 @@ __device__ __forceinline__ void strip_epilogue(const StageArgs<T>& A, const Tile
         if (lane == 0) atomicMax(A.rate_slot, b);
     }
     if (A.tot_partial) {
-        double v[NF];
-#pragma unroll
-        for (int f = 0; f < NF; ++f) v[f] = (double)acc.tot[f];
-        const double s = warp_sum5(v, lane);
+        const double s = warp_totals<ERR>(acc.tot, lane);
         if (sum5_writer(lane)) red_tot[warp][sum5_field(lane)] = s;
         if (NWARP > 1) __syncthreads();
         else __syncwarp();
@@ -235,15 +232,11 @@ __global__ void __launch_bounds__(32 * NWARP) strip_kernel(const StageArgs<T> A)
     const int strips = (A.n[0] + STRIP - 1) / STRIP;
     const long long chunk = item / strips;
     TileAcc<T> acc;
-    acc.rate_max = T(0);
-    acc.bad = false;
-#pragma unroll
-    for (int f = 0; f < NF; ++f) acc.tot[f] = T(0);
     const long long y0 = chunk * A.zchunk;
     if (y0 < A.n[1])
         strip_rows<T, DIM, PX, PY, RR>(A, (int)(item - chunk * strips) * STRIP, (int)y0,
                                              min((int)y0 + A.zchunk, A.n[1]), acc);
-    strip_epilogue<T, NWARP>(A, acc);
+    strip_epilogue<T, NWARP, (DIM > 1)>(A, acc);
 }
 
 }  // namespace hh

@@ -294,7 +294,7 @@ weno_stage_kernel(const StageArgs<T> A) {
     const T gx = sizeof(T) == 4 ? A.igm1 : A.gm1;
     bool bad = false;
     T rate_max = T(0);
-    T tot[NF] = {T(0), T(0), T(0), T(0), T(0)};
+    LaneSum<T> tot[NF];
 
     // z stencil of this thread's column: primitives of the last five planes,
     // the pending left state of the next z face, the previous z-face flux and
@@ -469,7 +469,7 @@ weno_stage_kernel(const StageArgs<T> A) {
             }
             if (A.tot_partial) {
 #pragma unroll
-                for (int f = 0; f < NF; ++f) tot[f] += Uo[f];
+                for (int f = 0; f < NF; ++f) tot[f].add(Uo[f]);
             }
         }
     }
@@ -486,10 +486,7 @@ weno_stage_kernel(const StageArgs<T> A) {
         if (lane == 0) red_rate[warp] = b;
     }
     if (A.tot_partial) {
-        double v[NF];
-#pragma unroll
-        for (int f = 0; f < NF; ++f) v[f] = (double)tot[f];
-        const double s = warp_sum5(v, lane);
+        const double s = warp_totals(tot, lane);
         if (sum5_writer(lane)) red_tot[warp][sum5_field(lane)] = s;
     }
     const int any_bad = __syncthreads_or(bad);

@@ -54,7 +54,7 @@ __device__ __forceinline__ void sweep_load(const StageArgs<T>& A, long long base
 // the block's row of the totals partial array (every thread calls it).
 template <typename T>
 __device__ __forceinline__ void sweep_epilogue(const StageArgs<T>& A, bool bad, T rate_max,
-                                               const T tot[NF], long long blk) {
+                                               const LaneSum<T> tot[NF], long long blk) {
     __shared__ double red_tot[SWEEP_THREADS / 32][NF];
     __shared__ unsigned long long red_rate[SWEEP_THREADS / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -68,10 +68,7 @@ __device__ __forceinline__ void sweep_epilogue(const StageArgs<T>& A, bool bad, 
         if (lane == 0) red_rate[warp] = b;
     }
     if (A.tot_partial) {
-        double v[NF];
-#pragma unroll
-        for (int f = 0; f < NF; ++f) v[f] = (double)tot[f];
-        const double s = warp_sum5(v, lane);
+        const double s = warp_totals(tot, lane);
         if (sum5_writer(lane)) red_tot[warp][sum5_field(lane)] = s;
     }
     const int any_bad = __syncthreads_or(bad);
@@ -205,7 +202,7 @@ weno_march_kernel(const StageArgs<T> A, T* L) {
     const bool two = A.stage == 2;
     bool bad = false;
     T rate_max = T(0);
-    T tot[NF] = {T(0), T(0), T(0), T(0), T(0)};
+    LaneSum<T> tot[NF];
 
     // the conserved state of cell m through the axis' boundary map (raw:
     // the reflecting flip is applied when the value is used)
@@ -304,7 +301,7 @@ weno_march_kernel(const StageArgs<T> A, T* L) {
                         }
                         if (A.tot_partial) {
 #pragma unroll
-                            for (int f = 0; f < NF; ++f) tot[f] += Uo[f];
+                            for (int f = 0; f < NF; ++f) tot[f].add(Uo[f]);
                         }
                     } else {
 #pragma unroll
