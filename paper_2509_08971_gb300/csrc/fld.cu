@@ -24,6 +24,7 @@
 
 #include "devattr.h"
 #include "fld_launch.h"
+#include "fld_split.cuh"
 #include "pdl.h"
 #include "hard_hydro.h"
 
@@ -86,23 +87,6 @@ struct StencilVals {
     int face;                 // bit 2 ax + (s > 0): that face carries a flux
 };
 
-// Neighbour offsets of a cell along one axis (coordinate c of n cells, the
-// axis' element stride): lo / hi are added to the cell's index (across the
-// wrap on a periodic axis; 0 at a wall, whose face carries no flux), face
-// bit 0 / 1 set when the low / high face carries a flux.
-struct AxisNb {
-    int lo, hi, face;
-};
-
-__device__ __forceinline__ AxisNb axis_nb(int c, int n, bool per, int stride) {
-    const bool inl = c > 0, inh = c + 1 < n;
-    AxisNb b;
-    b.lo = inl ? -stride : (per ? (n - 1) * stride : 0);
-    b.hi = inh ? stride : (per ? -(n - 1) * stride : 0);
-    b.face = (inl || per ? 1 : 0) | (inh || per ? 2 : 0);
-    return b;
-}
-
 // The loads of cell q with the z-axis neighbours given (nbz: the same for
 // every cell of a plane, so a kernel that takes several rows of one plane
 // per thread computes it once).
@@ -162,12 +146,6 @@ __device__ __forceinline__ void stencil(const LvlArgs<T>& a, int i, int j, int k
     stencil_load(a, i, j, k, q, v);
     stencil_eval(a, v, diag, off);
 }
-
-}  // namespace
-}  // namespace hh
-#include "fld_split.cuh"
-namespace hh {
-namespace {
 
 // Launch shape of the level kernels of a level in mesh order: x along threads (and blockIdx.x), one
 // row j per blockIdx.y (SMOOTH_ROWS rows for the smoother), one plane k per

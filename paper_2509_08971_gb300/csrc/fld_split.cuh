@@ -21,10 +21,27 @@
 // in mesh order; the prolongation corrects one colour only (19 us against 36), the
 // residual norm takes 34 us (53), the step to 1e-5 (four cycles) 2.23 ms (3.11).
 #pragma once
-#include <type_traits>
+#include "pdl.h"
 
 namespace hh {
 namespace {
+
+// Neighbour offsets of a cell along one axis (coordinate c of n cells, the
+// axis' element stride): lo / hi are added to the cell's index (across the
+// wrap on a periodic axis; 0 at a wall, whose face carries no flux), face
+// bit 0 / 1 set when the low / high face carries a flux.
+struct AxisNb {
+    int lo, hi, face;
+};
+
+__device__ __forceinline__ AxisNb axis_nb(int c, int n, bool per, int stride) {
+    const bool inl = c > 0, inh = c + 1 < n;
+    AxisNb b;
+    b.lo = inl ? -stride : (per ? (n - 1) * stride : 0);
+    b.hi = inh ? stride : (per ? -(n - 1) * stride : 0);
+    b.face = (inl || per ? 1 : 0) | (inh || per ? 2 : 0);
+    return b;
+}
 
 template <typename T> struct VecOf;
 template <> struct VecOf<float> { using type = float4; static constexpr int V = 4; };
@@ -257,39 +274,37 @@ __global__ void __launch_bounds__(128, 4) split_smooth_kernel(const SplitArgs<T>
     }
 }
 
-// sum r^2 over the cells of colour c, r = b - A x, into *out.  FP32 sums a
-// thread's chunk in FP32 (at most 4 x chunk terms), then a warp's.
+// sum r^2 over the cells of colour c, r = b - A x, into *out.  The 2 V terms of two
+// planes are summed in the element type, everything after them in FP64 (with the FP64
+// addition at each plane the 256^3 step took 2.216 ms, without any 2.205).
 template <typename T, bool WALLS>
 __global__ void __launch_bounds__(128) split_norm_kernel(const SplitArgs<T> a, int c, int chunk,
                                                          double* out) {
     griddep_wait();
     if (griddep_many_blocks()) griddep_launch_dependents();
     constexpr int V = VecOf<T>::V;
+    double t = 0.0;
     T sum = T(0);
     int p0, j;
     if (split_column(a, p0, j)) {
         const int k0 = blockIdx.y * chunk, k1 = min(k0 + chunk, a.n[2]);
         split_march<WALLS, true>(a, c, p0, j, k0, k1,
-                    [&](int, const SplitRow<T>& v, const T (&diag)[V], const T (&off)[V]) {
+                    [&](int k, const SplitRow<T>& v, const T (&diag)[V], const T (&off)[V]) {
                         const int cnt = row_cells(a, v.s);
 #pragma unroll
                         for (int u = 0; u < V; ++u) {
                             const T r = v.b[u] - (diag[u] * v.x[u] - off[u]);
                             if (p0 + u < cnt) sum = fma(r, r, sum);
                         }
+                        if ((k & 1) || k + 1 == k1) {
+                            t += sum;
+                            sum = T(0);
+                        }
                     });
     }
     __shared__ double red[4];
-    double t;
-    if constexpr (std::is_same<T, double>::value) {
-        t = sum;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    } else {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        t = sum;
-    }
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = t;
     __syncthreads();
     if (threadIdx.x == 0) {
