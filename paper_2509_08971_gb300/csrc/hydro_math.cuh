@@ -29,14 +29,16 @@ template <> struct Rot<2> { static constexpr int n = 3, t1 = 1, t2 = 2; };
 // --------------------------------------------------- FP64 without its pipe --
 // GB300 issues one FP64 warp instruction per SM every 16 clocks and 64 others
 // in that time, so an FP64 kernel costs what it sends down that pipe.  The
-// helpers below return the bits of the plain expressions with fewer of those
-// instructions: comparisons on the integer pipe, and quotients by a divisor
-// that serves several of them as q = a y, q + (a - b q) y with y = RN(1/b)
-// (three operations instead of an IEEE division's seven or eight).  That last
-// step is Markstein's theorem (P. Markstein, IBM J. Res. Dev. 34, 1990): with
-// y the correctly rounded reciprocal and q within an ulp of a/b, the result
-// is the correctly rounded quotient as long as nothing under- or overflows;
-// operands outside 2^-500 .. 2^500 take the division. Measured, with the results
+// helpers below return the bits of the plain expressions, up to the sign of a zero
+// (div_by's quotient of -0 is +0, minmod passes on a -0 of its arguments; no sum
+// or difference of the schemes tells the two apart), with fewer of those
+// instructions: comparisons on the integer pipe, and quotients by a divisor that
+// serves several of them as q = RN(a y), q + (a - b q) y with y = RN(1/b) (three
+// operations instead of an IEEE division's seven or eight).  One product and two
+// fused operations with the correctly rounded reciprocal give the correctly rounded
+// quotient as long as nothing under- or overflows (Brisebarre, Muller and Raina, IEEE
+// Trans. Computers 53, 2004, after Markstein, IBM J. Res. Dev. 34, 1990); operands
+// outside 2^-500 .. 2^500 take the division.  Measured, with the results
 // bit-identical: two steps of a 128^3 mesh 20.0 -> 14.3 ms (984 -> ~690
 // FP64 warp instructions per 32 cells and stage), 100 steps of a 400-cell 1D
 // mesh 6.98 -> 4.73 ms.
