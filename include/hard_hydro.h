@@ -98,7 +98,8 @@ int hard_hydro_set_cells(hard_hydro_t h, double dx, double dy, double dz);
  * built-in default).  Tile ids index a table that depends on the number of
  * active axes of the handle's mesh: hard_hydro_tile_count returns its size
  * (or a negative error code) and hard_hydro_tile_info writes
- * {tile_x, tile_y, z_chunk, threads_per_block} of one entry; of a 1D or
+ * {tile_x, tile_y, z_chunk, threads_per_block} of one entry (tile -1: of the
+ * built-in default on the handle's mesh); of a 1D or
  * 2D mesh {32 lanes, warps per block, rows per warp, threads_per_block}. */
 int hard_hydro_set_kernel(hard_hydro_t h, int kernel, int tile);
 int hard_hydro_tile_count(hard_hydro_t h);

@@ -1,8 +1,8 @@
 """Tile autotuner for the stage kernel.
 
-For a mesh, element type and kernel variant it times every tile
-configuration the library offers (tile extents, threads per block, z-chunk
-length; `hard_hydro_tile_info`) on the caller's own state: each candidate
+For a mesh, element type and kernel variant it times the library's own choice
+(tile -1) and every tile configuration of its table (tile extents, threads per
+block, z-chunk length; `hard_hydro_tile_info`) on the caller's own state: each candidate
 runs a few untimed stage-1/stage-2 pairs, then a timed batch bracketed by
 CUDA events on the current stream.  The fastest tile is set on the handle and
 remembered in a JSON cache keyed by mesh shape, boundary kinds per face,
@@ -44,8 +44,9 @@ def _load_cache(path):
 
 def tune(m: HardHydro, U, kernel: int = 0, reps: int = 10, warmup: int = 2,
          cache_path: str | None = None, verbose: bool = False) -> dict:
-    """Pick the fastest tile for handle `m` on state `U` and set it.
-    Returns {"tile": best, "info": (tx, ty, zc, threads), "ms": {tile: ms}}."""
+    """Pick the fastest tile for handle `m` on state `U` and set it (-1: the
+    library's choice, in general no entry of the table).  Returns
+    {"tile": best, "info": (tx, ty, zc, threads), "ms": {tile: ms}}."""
     torch = m.torch
     cache_path = cache_path if cache_path is not None else os.environ.get("HARD_HYDRO_TUNE_CACHE")
     key = _key(m, kernel)
@@ -62,7 +63,7 @@ def tune(m: HardHydro, U, kernel: int = 0, reps: int = 10, warmup: int = 2,
     # two sweeps, the faster of each tile's two timings: a host-side stall in
     # one timed window (process start-up work, another process) cannot decide
     for sweep in range(2):
-        for tile in range(m.tile_count()):
+        for tile in range(-1, m.tile_count()):
             m.set_kernel(kernel, tile)
             for _ in range(warmup):
                 m.stage(1, None, U, dt, out=U1)

@@ -441,8 +441,8 @@ int hard_hydro_tile_count(hard_hydro_t h) {
 }
 
 int hard_hydro_tile_info(hard_hydro_t h, int tile, int out4[4]) {
-    if (!h || !out4 || tile < 0 || tile >= hh::tile_count(h->mesh.dim)) return HARD_EINVAL;
-    hh::TileDesc t = hh::tile_desc(h->mesh.dim, tile);
+    if (!h || !out4 || tile < -1 || tile >= hh::tile_count(h->mesh.dim)) return HARD_EINVAL;
+    const hh::TileDesc t = hh::launch_tile(h->mesh, tile, h->dtype == HARD_F64);
     out4[0] = t.tx;
     out4[1] = t.ty;
     out4[2] = t.zc;
