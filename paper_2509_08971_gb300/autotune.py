@@ -6,15 +6,15 @@ block, z-chunk length; `hard_hydro_tile_info`) on the caller's own state: each c
 runs a few untimed stage-1/stage-2 pairs, then a timed batch bracketed by
 CUDA events on the current stream.  The fastest tile is set on the handle and
 remembered in a JSON cache keyed by mesh shape, boundary kinds per face,
-extents, element type, kernel, scheme and gamma (``HARD_HYDRO_TUNE_CACHE``
-names the file; unset = in-memory only): the boundary kinds decide which tiles
-take the generic ghost path, so a tile tuned on one kind is not reused for
-another.
+extents, element type, kernel, scheme, gamma and the tile table
+(``HARD_HYDRO_TUNE_CACHE`` names the file; unset = in-memory only): the boundary
+kinds decide which tiles take the generic ghost path, so a tile tuned on one kind
+is not reused for another, and an id written under another table is not applied.
 
 ``tune_batch`` does the same for the persistent batched launch: it times each
 batched tile set (`hard_batch_tile_count`) on a few steps of the caller's
 packed batch and keeps the fastest, keyed by the batch's problem sizes,
-boundary kinds and element type.
+boundary kinds, element type and the batched tile table.
 """
 from __future__ import annotations
 
@@ -28,8 +28,13 @@ from . import HardHydro, hard_batch_tile_count
 _memory: dict[str, int] = {}
 
 
+# what the batched tile ids stand for (warps per block); ids of another table are not reused
+BATCH_TABLE = ("warps", 8, 4, 16)
+
+
 def _key(m: HardHydro, kernel: int) -> str:
-    return (f"{m.shape}|bc{m.bc6}|ext{m.extent}|{m.dtype}|k{kernel}|s{m.scheme}|g{m.gamma}")
+    table = [tuple(m.tile_info(t)) for t in range(m.tile_count())]
+    return (f"{m.shape}|bc{m.bc6}|ext{m.extent}|{m.dtype}|k{kernel}|s{m.scheme}|g{m.gamma}|tiles{table}")
 
 
 def _load_cache(path):
@@ -95,7 +100,7 @@ def tune(m: HardHydro, U, kernel: int = 0, reps: int = 10, warmup: int = 2,
 
 def _batch_key(B) -> str:
     h = hashlib.sha256()
-    h.update(repr((B.nx, B.ny, B.bcs, B.gammas, str(B.dtype))).encode())
+    h.update(repr((B.nx, B.ny, B.bcs, B.gammas, str(B.dtype), BATCH_TABLE)).encode())
     return "batch|" + h.hexdigest()[:32]
 
 

@@ -2,6 +2,8 @@
 beside the table and keeps it when it is the fastest; a cached choice is used as long as the
 tile ids mean what they meant when it was written."""
 import json
+import os
+import re
 from types import SimpleNamespace
 
 import pytest
@@ -67,3 +69,31 @@ def test_the_librarys_choice_is_timed(cost, best):
     assert m.timed == {-1, 0, 1} and got["tile"] == best == m.tile
     assert got["info"] == m.tile_info(best)
     assert got["ms"] == pytest.approx(cost)
+
+
+def test_a_cache_of_other_tables_is_not_used(tmp_path):
+    path = str(tmp_path / "tune.json")
+    cost = {-1: 3.0, 0: 2.0, 1: 1.0}
+    assert autotune.tune(Handle(cost, TABLE), object(), cache_path=path)["tile"] == 1
+    autotune._memory.clear()
+    again = Handle(cost, TABLE)
+    got = autotune.tune(again, object(), cache_path=path)
+    assert got["cached"] and got["tile"] == 1 and not again.timed
+    autotune._memory.clear()
+    other = Handle({-1: 3.0, 0: 1.0, 1: 2.0}, TABLE[::-1])
+    got = autotune.tune(other, object(), cache_path=path)
+    assert not got["cached"] and got["tile"] == 0 and len(json.load(open(path))) == 2
+
+
+def test_batch_cache_of_other_tables_is_not_used(monkeypatch):
+    B = SimpleNamespace(nx=[8], ny=[1], bcs=(0,), gammas=(1.4,), dtype="float32")
+    key = autotune._batch_key(B)
+    monkeypatch.setattr(autotune, "BATCH_TABLE", ("warps", 4, 2))
+    assert autotune._batch_key(B) != key
+
+
+def test_batch_table_is_the_librarys():
+    here = os.path.dirname(os.path.abspath(autotune.__file__))
+    text = open(os.path.join(here, "csrc", "launch.h")).read()
+    warps = re.search(r"BATCH_WARPS\[\] = \{([^}]*)\}", text).group(1)
+    assert autotune.BATCH_TABLE == ("warps", *(int(w) for w in warps.split(",")))
