@@ -397,7 +397,7 @@ cudaError_t dispatch_tile(const MeshDesc& m, int kernel, int tile, const StageCa
         }
     } else {
         if (td.ty == 1) return run_strip<1, PX, 0, 1, 1>(m, td, c, s);
-        return run_strip<1, PX, 0, 1, 4>(m, td, c, s);
+        return run_strip<1, PX, 0, 1, 8>(m, td, c, s);
     }
 }
 

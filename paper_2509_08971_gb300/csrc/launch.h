@@ -130,7 +130,7 @@ inline constexpr TileDesc TILES3[] = {{32, 8, 32}, {32, 8, 64}, {32, 16, 64}, {6
 // 1D and 2D meshes run one warp per strip of 28 cells (strip.cuh): 32 lanes, ty
 // warps per block, zc rows per warp.
 inline constexpr TileDesc TILES2[] = {{32, 2, 2}, {32, 2, 4}, {32, 2, 16}};
-inline constexpr TileDesc TILES1[] = {{32, 1, 1}, {32, 4, 1}};
+inline constexpr TileDesc TILES1[] = {{32, 1, 1}, {32, 8, 1}};
 inline constexpr int STRIP_CELLS = 28;
 
 inline int tile_count(int dim) {
@@ -146,7 +146,12 @@ inline TileDesc tile_desc(int dim, int tile) {
 // choice.  2D: rows per warp.  A warp of two rows pays ~1.3x (FP32) / 1.4x
 // (FP64) of the work per cell of a long one and of four ~1.15x / 1.2x, for
 // more warps and a shorter chain; FP32 hides its latencies with at least 8
-// warps per SM, FP64 keeps its pipe busy with 4.
+// warps per SM, FP64 keeps its pipe busy with 4.  1D: a block per strip for the
+// shortest chain and all SMs; once the SMs have five strips each, FP32 meshes take eight
+// warps to a block, for an eighth of the atomics on the rate slot and of the rows of
+// the totals array (a step of 10^6 cells 31.9 us against 57.8, with totals 68.6
+// against 159; of 16000 cells 6.1 against 5.9); FP64 ones, bound by their
+// pipe, do not (1168 us against 1108).
 inline TileDesc launch_tile(const MeshDesc& m, int tile, bool f64) {
     if (tile >= 0) return tile_desc(m.dim, tile);
     if (m.dim == 2) {
@@ -154,6 +159,7 @@ inline TileDesc launch_tile(const MeshDesc& m, int tile, bool f64) {
         const long long want = 152ll * (f64 ? 4 : 8);
         return TILES2[rows >= 16 * want ? 2 : rows >= 4 * want ? 1 : 0];
     }
+    if (m.dim == 1) return TILES1[!f64 && m.n[0] >= STRIP_CELLS * 5 * SMS ? 1 : 0];
     return m.dim == 3 ? m.auto3[f64] : tile_desc(m.dim, 0);
 }
 // Blocks the stage kernel launches (rows of the totals partial array).

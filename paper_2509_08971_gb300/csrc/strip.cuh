@@ -195,32 +195,41 @@ __device__ __forceinline__ void strip_rows(const StageArgs<T>& A, int xs, int y0
 }
 
 // Block reductions of what the block's warps accumulated: the non-physical
-// flag, the rate maximum, and the block's row of the totals partial array.
+// flag, the rate maximum (one atomic per block: the slot takes about one a
+// nanosecond from the whole chip), and the block's row of the totals partial array.
 template <typename T, int NWARP, bool ERR>
 __device__ __forceinline__ void strip_epilogue(const StageArgs<T>& A, const TileAcc<T>& acc) {
     __shared__ double red_tot[NWARP][NF];
+    __shared__ unsigned long long red_rate[NWARP];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool any_bad = __any_sync(FULL, acc.bad);
     if (any_bad && lane == 0) atomicOr(A.status, 1);
+    unsigned long long b = 0;
     if (A.rate_slot) {
-        unsigned long long b = rate_bits(acc.rate_max);
+        b = rate_bits(acc.rate_max);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             const unsigned long long v = __shfl_xor_sync(FULL, b, o);
             b = v > b ? v : b;
         }
-        if (lane == 0) atomicMax(A.rate_slot, b);
+        if (NWARP > 1 && lane == 0) red_rate[warp] = b;
     }
     if (A.tot_partial) {
         const double s = warp_totals<ERR>(acc.tot, lane);
         if (sum5_writer(lane)) red_tot[warp][sum5_field(lane)] = s;
-        if (NWARP > 1) __syncthreads();
-        else __syncwarp();
-        if (threadIdx.x < NF) {
-            double t = 0.0;
-            for (int w = 0; w < NWARP; ++w) t += red_tot[w][threadIdx.x];
-            A.tot_partial[(long long)blockIdx.x * NF + threadIdx.x] = t;
-        }
+    }
+    if (!A.rate_slot && !A.tot_partial) return;
+    if (NWARP > 1) __syncthreads();
+    else __syncwarp();
+    if (A.rate_slot && threadIdx.x == 0) {
+        if (NWARP > 1)
+            for (int w = 1; w < NWARP; ++w) b = red_rate[w] > b ? red_rate[w] : b;
+        atomicMax(A.rate_slot, b);
+    }
+    if (A.tot_partial && threadIdx.x < NF) {
+        double t = 0.0;
+        for (int w = 0; w < NWARP; ++w) t += red_tot[w][threadIdx.x];
+        A.tot_partial[(long long)blockIdx.x * NF + threadIdx.x] = t;
     }
 }
 
