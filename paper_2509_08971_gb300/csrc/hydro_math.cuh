@@ -30,7 +30,7 @@ template <> struct Rot<2> { static constexpr int n = 3, t1 = 1, t2 = 2; };
 // GB300 issues one FP64 warp instruction per SM every 16 clocks and 64 others
 // in that time, so an FP64 kernel costs what it sends down that pipe.  The
 // helpers below return the bits of the plain expressions, up to the sign of a zero
-// (div_by's quotient of -0 is +0, minmod passes on a -0 of its arguments; no sum
+// (the short quotient of -0 is +0, minmod passes on a -0 of its arguments; no sum
 // or difference of the schemes tells the two apart), with fewer of those
 // instructions: comparisons on the integer pipe, and quotients by a divisor that
 // serves several of them as q = RN(a y), q + (a - b q) y with y = RN(1/b) (three

