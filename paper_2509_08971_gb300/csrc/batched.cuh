@@ -97,8 +97,10 @@ __device__ __forceinline__ void warp_rate_max(T r, unsigned long long* red) {
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = b;
 }
 
-// NW warps per block; 16 warps per SM (128 registers a thread: of 24, 80 registers,
-// the walk spills, 10.5 -> 17.9 ms).
+// NW warps per block; 16 warps per SM (128 registers a thread).  FP32: of 24, 80
+// registers, the walk spills, 10.5 -> 17.9 ms.  FP64 spills ~560 bytes here; with the 252
+// registers that it wants, 8 warps per SM, 256 2D problems of 32 to 128 cells a side
+// take 9.5 ms against 16.3, but 8192 1D ones of 16 to 64 cells 2.55 against 1.43.
 template <typename T, int NW>
 __global__ void __launch_bounds__(32 * NW, 16 / NW) batched_kernel(const BatchArgs<T> B) {
     constexpr int NT = 32 * NW;
@@ -131,7 +133,8 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) batched_kernel(const BatchAr
         T* W = B.W + P.off;
         const bool two_d = P.ny > 1;
         const long long N = (long long)P.nx * P.ny;
-        const int strips = (P.nx + STRIP - 1) / STRIP;
+        const int strips = (P.nx + STRIP - 1) / STRIP;   // 1D
+        const StripPlan plan = strip_plan(P.nx);
         if (tid == 0) {
             s_sc.gamma = (T)P.gamma;
             s_sc.gm1 = (T)(P.gamma - 1.0);
@@ -145,7 +148,7 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) batched_kernel(const BatchAr
             // block's warps take the fewest rows (a chunk pays about three
             // rows for its warm-up and look-ahead)
             const int k = (tid & 31) + 1;
-            const long long cost = (((long long)strips * k + NW - 1) / NW) * ((P.ny + k - 1) / k + 3);
+            const long long cost = (long long)((strip_warps<unsigned>(plan, k) + NW - 1) / NW) * ((P.ny + k - 1) / k + 3);
             const unsigned key = ((unsigned)min(cost, (1ll << 25) - 1) << 6) | (unsigned)k;
             const unsigned best = __reduce_min_sync(FULL, key);
             if ((tid & 31) == 0) s_chunks = two_d ? (int)(best & 63u) : 1;
@@ -153,7 +156,8 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) batched_kernel(const BatchAr
         __syncthreads();
         const BatchScalars<T> sc = s_sc;
         const int chunk = (P.ny + s_chunks - 1) / s_chunks;
-        const long long items = (long long)strips * s_chunks;    // below 2^32: at most 32 chunks
+        const int chunks = (P.ny + chunk - 1) / chunk;           // s_chunks without empty ones
+        const unsigned items = strip_warps<unsigned>(plan, chunks);   // at most 32 chunks: below 2^32
 
         // signal rate of the initial state
         {
@@ -186,16 +190,11 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) batched_kernel(const BatchAr
                 // into acc (it never writes through the pointer)
                 A.rate_slot = stage == 2 ? red : nullptr;
                 if (two_d) {
-                    for (unsigned it = warp; it < (unsigned)items; it += NW) {
-                        const unsigned c = it / (unsigned)strips;
-                        const int y0 = (int)c * chunk;
-                        if (y0 < P.ny)
-                            strip_rows<T, 2, 0, 1, 0>(A, (int)(it - c * strips) * STRIP, y0,
-                                                             min(y0 + chunk, P.ny), acc);
-                    }
+                    for (unsigned it = warp; it < items; it += NW)
+                        strip_item<T, 0, 1, 0>(A, plan, it, chunks, chunk, acc);
                 } else {
                     for (int it = warp; it < strips; it += NW)
-                        strip_rows<T, 1, 0, 0, 1>(A, it * STRIP, 0, 1, acc);
+                        strip_rows<T, 1, 0, 0, 1>(A, it * STRIP, tid & 31, 0, 1, 1, acc);
                 }
                 if (stage == 2) warp_rate_max(acc.rate_max, red);
                 __syncthreads();            // every cell of this stage written

@@ -9,12 +9,17 @@
 // last difference, pending lower state, last face flux), so a cell is
 // converted, limited and differenced once per axis and every face evaluated
 // once, by one warp; two rows of warm-up and two of look-ahead per chunk.
+// A row's last cells take a strip of their own; where they are twelve or fewer, a
+// warp walks several of its row chunks side by side (strip_plan), so a row of 29
+// cells costs 28 + 5 lanes, not 64: a step of 50000 rows of 29 cells 121 -> 81 us
+// (block tiles: 96), FP64 5.97 -> 3.25 ms (5.05); 2048 batched problems of 29 to 32
+// cells a side, five steps, 0.80 -> 0.62 ms (0.62).
 //
 // What bounds it: instruction issue in FP32, the FP64 pipe in FP64, and on
 // small meshes the latency of one strip.  It replaces a 32 x 8 tile per block
 // (primitives and both face fluxes through shared memory, two barriers, every
 // slope twice): 757 issue slots per cell-stage there.  Measured, bit-identical: 4096 batched
-// problems, five steps, 15.45 -> 10.40 ms; 100 FP64 steps of a 400-cell mesh
+// problems, five steps, 15.45 -> 10.12 ms; 100 FP64 steps of a 400-cell mesh
 // (15 SMs instead of 4) 4.73 -> 3.09 ms; 50 FP32 steps at 256^2 0.92 -> 0.84 ms.
 //
 // strip_rows evaluates the same expressions in the same order whatever the
@@ -47,20 +52,22 @@ __device__ __forceinline__ void strip_x(const StageArgs<T>& A, const T W[NF], T 
         D[f] = sub_over_dx(T(0), __shfl_down_sync(FULL, Fl[f], 1) - Fl[f], A.dxk[0]);
 }
 
-// Rows [y0, y1) of the strip at xs.  RR > 0: at most RR rows, every load
+// Rows [y0, y1) of the strip at xs, of which the warp walks `rows` (as many, or more
+// where lanes have chunks of their own, past whose end the boundary map returns cells
+// nobody uses); pos: the lane's place in the strip.  RR > 0: RR rows, every load
 // issued before any arithmetic and the rows unrolled (small meshes: one memory
 // round trip); RR = 0: a walk of any length with the next row's loads in
 // flight.  1D: y0 = 0, y1 = 1, RR = 1.
 template <typename T, int DIM, int PX, int PY, int RR>
-__device__ __forceinline__ void strip_rows(const StageArgs<T>& A, int xs, int y0, int y1,
-                                           TileAcc<T>& acc) {
-    const int lane = threadIdx.x & 31;
-    const int n0 = A.n[0], gx = xs - 2 + lane;
+__device__ __forceinline__ void strip_rows(const StageArgs<T>& A, int xs, int pos, int y0, int y1,
+                                           int rows, TileAcc<T>& acc) {
+    const int n0 = A.n[0], gx = xs - 2 + pos;
     bool flx;
     const int sx = bc_map(gx, n0, A.bc_lo[0], A.bc_hi[0], flx);
-    const bool own = lane >= 2 && lane < 2 + STRIP && gx < n0;
+    const bool own = pos >= 2 && pos < 2 + STRIP && gx < n0;
     const long long N = A.N;
     const T* const Uc = A.Uc + sx;
+    const T* const U0 = A.U0 + (own ? gx : 0);
     const T dt = (T)(A.dt_dev ? *A.dt_dev : A.dt);
     const bool two = A.stage == 2;
 
@@ -101,13 +108,14 @@ __device__ __forceinline__ void strip_rows(const StageArgs<T>& A, int xs, int y0
         }
     };
     auto fetch0 = [&](int k, T u0[NF]) {
-        const T* p = A.U0 + (long long)k * n0 + (own ? gx : 0);
+        if (!two) return;
+        const T* p = U0 + (long long)min(k, A.n[1] - 1) * n0;
 #pragma unroll
-        for (int f = 0; f < NF; ++f) u0[f] = two && k < y1 ? p[f * N] : T(0);
+        for (int f = 0; f < NF; ++f) u0[f] = p[f * N];
     };
 
     if constexpr (DIM == 1) {
-        T U[NF], W[NF], D[NF], u0[NF];
+        T U[NF], W[NF], D[NF], u0[NF] = {};
         bool fly;
         fetch(0, U, fly);
         fetch0(0, u0);
@@ -130,7 +138,7 @@ __device__ __forceinline__ void strip_rows(const StageArgs<T>& A, int xs, int y0
 #pragma unroll
             for (int f = 0; f < NF; ++f) Uraw[f] = U[f];
             prim(U, fly, W);
-            if (cnt >= 3 && r - 1 < y1) strip_x<T, PX>(A, q, Dn);
+            if (cnt >= 3 && cnt < rows + 3) strip_x<T, PX>(A, q, Dn);
             if (cnt >= 1) {
 #pragma unroll
                 for (int f = 0; f < NF; ++f) dc[f] = W[f] - q[f];
@@ -168,7 +176,7 @@ __device__ __forceinline__ void strip_rows(const StageArgs<T>& A, int xs, int y0
             }
         };
         if constexpr (RR > 0) {
-            T U[RR + 4][NF], u0[RR][NF];
+            T U[RR + 4][NF], u0[RR][NF] = {};
             bool fl[RR + 4];
 #pragma unroll
             for (int i = 0; i < RR + 4; ++i) fetch(y0 - 2 + i, U[i], fl[i]);
@@ -181,17 +189,42 @@ __device__ __forceinline__ void strip_rows(const StageArgs<T>& A, int xs, int y0
             bool fn;
             fetch(y0 - 2, Un, fn);
 #pragma unroll 1       // by two: 4096 batched problems 10.53 ms, one by one 10.40
-            for (int r = y0 - 2; r <= y1 + 1; ++r) {
-                T U[NF], u0[NF];
+            for (int cnt = 0; cnt < rows + 4; ++cnt) {
+                const int r = y0 - 2 + cnt;
+                T U[NF], u0[NF] = {};
                 const bool fl = fn;
 #pragma unroll
                 for (int f = 0; f < NF; ++f) U[f] = Un[f];
-                if (r <= y1) fetch(r + 1, Un, fn);
-                if (r - 2 >= y0) fetch0(r - 2, u0);
-                row(r, r - (y0 - 2), U, fl, u0);
+                if (cnt < rows + 3) fetch(r + 1, Un, fn);
+                if (cnt >= 4) fetch0(r - 2, u0);
+                row(r, cnt, U, fl, u0);
             }
         }
     }
+}
+
+// Warp `item` of the plan p: a full strip of one of `chunks` chunks of `len` rows
+// (x fastest), or `groups` chunks of the last cells' strip.  I: a type that holds
+// the number of items.
+template <typename T, int PX, int PY, int RR, typename I>
+__device__ __forceinline__ void strip_item(const StageArgs<T>& A, const StripPlan& p, I item,
+                                           int chunks, int len, TileAcc<T>& acc) {
+    const int n1 = A.n[1];
+    const I full = (I)p.full * chunks;
+    int pos = threadIdx.x & 31, c, xs, rows;
+    if (item < full) {
+        c = (int)(item / (I)p.full);
+        xs = (int)(item - (I)c * p.full) * STRIP;
+        rows = min(len, n1 - c * len);
+    } else {
+        const int g = pos / p.width, first = (int)(item - full) * p.groups;
+        c = min(first + g, chunks - 1);
+        xs = p.full * STRIP;
+        rows = min(len, n1 - first * len);             // of the first chunk, the longest
+        pos = g < p.groups && first + g < chunks ? pos - g * p.width : 0;   // place 0 is a halo cell's
+    }
+    const int y0 = c * len;
+    strip_rows<T, 2, PX, PY, RR>(A, xs, pos, y0, min(y0 + len, n1), rows, acc);
 }
 
 // Block reductions of what the block's warps accumulated: the non-physical
@@ -238,13 +271,15 @@ template <typename T, int DIM, int PX, int PY, int RR, int NWARP>
 __global__ void __launch_bounds__(32 * NWARP) strip_kernel(const StageArgs<T> A) {
     griddep_wait();
     const long long item = (long long)blockIdx.x * NWARP + (threadIdx.x >> 5);
-    const int strips = (A.n[0] + STRIP - 1) / STRIP;
-    const long long chunk = item / strips;
     TileAcc<T> acc;
-    const long long y0 = chunk * A.zchunk;
-    if (y0 < A.n[1])
-        strip_rows<T, DIM, PX, PY, RR>(A, (int)(item - chunk * strips) * STRIP, (int)y0,
-                                             min((int)y0 + A.zchunk, A.n[1]), acc);
+    if constexpr (DIM == 1) {
+        if (item * STRIP < A.n[0])
+            strip_rows<T, DIM, PX, PY, RR>(A, (int)item * STRIP, threadIdx.x & 31, 0, 1, 1, acc);
+    } else {
+        const StripPlan p = strip_plan(A.n[0]);
+        const int chunks = (A.n[1] + A.zchunk - 1) / A.zchunk;
+        if (item < strip_warps<long long>(p, chunks)) strip_item<T, PX, PY, RR>(A, p, item, chunks, A.zchunk, acc);
+    }
     strip_epilogue<T, NWARP, (DIM > 1)>(A, acc);
 }
 
