@@ -108,7 +108,7 @@ void build_mesh(hard_hydro_s* h) {
     m.gamma = h->gamma;
     m.N = (long long)h->n[0] * h->n[1] * h->n[2];
     if (a == 3)
-        for (int f64 = 0; f64 < 2; ++f64) m.auto3[f64] = hh::choose_tile3(m.n, f64);
+        for (int r = 0; r < hh::RULES3; ++r) m.auto3[r] = hh::choose_tile3(m.n, (hh::Rule3)r);
 }
 
 void free_scratch(hard_hydro_s* h) {
@@ -224,7 +224,7 @@ bool halo_ready(const hard_hydro_s* h) {
 // blocks of one stage launch (rows of the totals partial array)
 long long launch_blocks(const hard_hydro_s* h) {
     if (weno(h)) return hh::weno_stage_blocks(h->mesh, h->mesh.dim == 3, h->dtype == HARD_F64);
-    return hh::stage_blocks(h->mesh, h->tile, h->dtype == HARD_F64);
+    return hh::stage_blocks(h->mesh, h->kernel, h->tile, h->dtype == HARD_F64);
 }
 
 cudaError_t stage_launch(hard_hydro_s* h, const StageCall& call, cudaStream_t s) {
@@ -442,7 +442,7 @@ int hard_hydro_tile_count(hard_hydro_t h) {
 
 int hard_hydro_tile_info(hard_hydro_t h, int tile, int out4[4]) {
     if (!h || !out4 || tile < -1 || tile >= hh::tile_count(h->mesh.dim)) return HARD_EINVAL;
-    const hh::TileDesc t = hh::launch_tile(h->mesh, tile, h->dtype == HARD_F64);
+    const hh::TileDesc t = hh::launch_tile(h->mesh, h->kernel, tile, h->dtype == HARD_F64);
     out4[0] = t.tx;
     out4[1] = t.ty;
     out4[2] = t.zc;

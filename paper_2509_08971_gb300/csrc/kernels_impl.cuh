@@ -360,7 +360,7 @@ __global__ void totals_kernel(const T* __restrict__ U, long long N, double* part
 template <int DIM, int PX, int PY>
 cudaError_t dispatch_tile(const MeshDesc& m, int kernel, int tile, const StageCall& c,
                           cudaStream_t s) {
-    const TileDesc td = launch_tile(m, tile, sizeof(T) == 8);
+    const TileDesc td = launch_tile(m, kernel, tile, sizeof(T) == 8);
     if constexpr (DIM == 3) {
         // the TMA kernel carries the rate / totals epilogue for stage 2 only
         const bool epi_ok = c.stage == 2 || (!c.rate_slot && !c.tot_partial);

@@ -24,7 +24,7 @@ struct MeshDesc {
     bool act[3];           // physical axis active
     double gamma;
     long long N;           // total cells
-    TileDesc auto3[2] = {{32, 8, 32}, {32, 8, 32}};   // 3D: choose_tile3 of FP32, FP64
+    TileDesc auto3[3] = {{32, 8, 32}, {32, 8, 32}, {32, 8, 32}};   // 3D: choose_tile3 by Rule3
 };
 
 // ---- chunk lengths by a schedule model ----
@@ -76,31 +76,54 @@ inline int choose_chunk(long long cols, int n, const Time& time, double* best = 
     if (best) *best = tb;
     return zb;
 }
-// Tile and z chunk of the 3D stage kernels.  Steps measured on 32-wide tiles:
-// FP32 (warp-specialised, bound by issue) 1.53 us a plane of 32 x 8 alone on its
-// SM, 1.85 us with a second block, 1.67 us of 32 x 16 (one block per SM), a
-// block's fixed cost ~3 planes; FP64 (bound by its pipe, whatever is
-// resident) 54.6 us of 32 x 8 and 35.1 us of 32 x 4 (58 us as one of two),
-// fixed cost ~1 plane.  One fixed 32 x 8 x 32 tile leaves most of the chip
-// idle on small meshes and most of the last wave on others.
-inline TileDesc choose_tile3(const int n[3], bool f64) {
-    struct Form { int ty, kmax; double over, step[2]; };
-    static constexpr Form F32[] = {{16, 1, 3.2, {1.67, 0}}, {8, 2, 3.0, {1.53, 1.85}}};
-    static constexpr Form F64[] = {{8, 1, 1.0, {54.6, 0}}, {4, 2, 1.2, {35.1, 58.0}}};
+// Tile and z chunk of the 3D stage kernels, of 32-wide tiles.  A form's time is
+// `first` + the span of its blocks, of which `over` planes each are warm-up and
+// fixed cost (and `more` where they share their SM and read planes of other
+// chunks), at step[k - 1] a plane where k blocks share an SM.  `sync` (if not 0):
+// the step of a first wave that runs in phase.  The blocks of a last wave that
+// leave a fifth of the SMs' places free take the step of fewer on an SM, and then
+// nothing stays in phase (FP32).  Fitted (us) to stages of 85 meshes of 4 to 512
+// planes by every tile: the fused kernels within 3 % at most sizes, the plain one
+// within 10 %.
+//
+// One fixed 32 x 8 x 32 tile leaves most of the chip idle on small meshes and most of
+// the last wave on others (64^3: 54 us a stage against 15).  FP32 by TMA: the 16-row tile
+// pays more per block and less per plane, so 4 planes of 1000^2 want 8 rows (154 us
+// a stage, 163 by 16), 32 planes either, 256^3 16 (407, 436 by 8).  By copies: 16 rows from
+// two waves on (4 x 601 x 499: 59 against 62).  FP64 is bound by its pipe, whatever is
+// resident.  The plain FP32 kernel fills an SM best with five blocks of 4 rows (512^3: 6.6 ms
+// a stage, 7.8 by 8 rows, 8.4 by 16).
+enum Rule3 { RULE_FUSED32, RULE_F64, RULE_PLAIN32, RULES3 };
+inline TileDesc choose_tile3(const int n[3], Rule3 rule) {
+    struct Form { int ty, kmax; double first, over, more, sync, step[5]; };
+    static constexpr Form TMA[] = {{16, 1, 3.3, 2.4, 0, 0, {1.71}}, {8, 2, 4.4, 2.05, 0.3, 1.94, {1.46, 1.74}}};
+    static constexpr Form COPIES[] = {{16, 1, 2.9, 2.4, 0, 0, {2.18}}, {8, 2, 3.2, 2.7, 0, 0, {1.58, 2.22}}};
+    static constexpr Form F64[] = {{8, 1, 0, 1.0, 0, 0, {54.6}}, {4, 2, 0, 1.2, 0, 0, {35.1, 58.0}}};
+    static constexpr Form PLAIN[] = {{8, 2, 2.1, 0.7, 0, 0, {3.26, 4.34}},
+                                     {4, 5, 1.0, 0.8, 0, 0, {3.0, 3.6, 4.0, 4.35, 4.65}}};
+    const Form* forms = rule == RULE_F64 ? F64 : rule == RULE_PLAIN32 ? PLAIN : n[0] % 4 ? COPIES : TMA;
     TileDesc td{32, 8, 32};
     double tb = 1e300;
-    for (const Form& f : f64 ? F64 : F32) {
-        const long long gy = (n[1] + f.ty - 1) / f.ty;
-        if (n[1] > 8 * 65535 || gy > 65535) continue;  // gridDim.y
+    for (const Form* f = forms; f < forms + 2; ++f) {
+        const long long gy = (n[1] + f->ty - 1) / f->ty;
+        // more rows than a grid of 8-row tiles takes are refused at the launch, as before the rule
+        if (n[1] > 8 * 65535 || gy > 65535) continue;
         const long long cols = (n[0] + 31) / 32 * gy;
         double t;
         const int z = choose_chunk(cols, n[2], [&](int zc, long long blocks) {
-            const int k = blocks > SMS ? f.kmax : 1;   // blocks on an SM
-            return span_steps(cols, n[2], zc, f.over, (long long)SMS * k) * f.step[k - 1];
+            const int k = (int)std::min<long long>(f->kmax, (blocks + SMS - 1) / SMS);   // blocks on an SM
+            const long long slots = (long long)SMS * k, rest = blocks % slots;
+            const double over = f->over + (k > 1 && zc < n[2] ? f->more : 0.0), w = zc + over, s = f->step[k - 1];
+            double t = f->first + span_steps(cols, n[2], zc, over, slots) * s;
+            const int last = (int)(rest / (SMS * 4 / 5)) + 1;        // on an SM in the last wave
+            if (rule != RULE_F64 && blocks > slots && rest && last < k && n[2] % zc == 0)
+                t -= w * (s - f->step[last - 1]);
+            else if (k > 1 && f->sync > 0) t += w * (f->sync - s);
+            return t;
         }, &t);
         if (t < tb) {
             tb = t;
-            td = TileDesc{32, f.ty, z};
+            td = TileDesc{32, f->ty, z};
         }
     }
     return td;
@@ -168,7 +191,7 @@ inline TileDesc tile_desc(int dim, int tile) {
 // the totals array (a step of 10^6 cells 31.9 us against 57.8, with totals 68.6
 // against 159; of 16000 cells 6.1 against 5.9); FP64 ones, bound by their
 // pipe, do not (1168 us against 1108).
-inline TileDesc launch_tile(const MeshDesc& m, int tile, bool f64) {
+inline TileDesc launch_tile(const MeshDesc& m, int kernel, int tile, bool f64) {
     if (tile >= 0) return tile_desc(m.dim, tile);
     if (m.dim == 2) {
         const long long rows = strip_warps<long long>(strip_plan(m.n[0]), m.n[1]);
@@ -176,12 +199,13 @@ inline TileDesc launch_tile(const MeshDesc& m, int tile, bool f64) {
         return TILES2[rows >= 16 * want ? 2 : rows >= 4 * want ? 1 : 0];
     }
     if (m.dim == 1) return TILES1[!f64 && m.n[0] >= STRIP_CELLS * 5 * SMS ? 1 : 0];
-    return m.dim == 3 ? m.auto3[f64] : tile_desc(m.dim, 0);
+    if (m.dim == 3) return m.auto3[f64 ? RULE_F64 : kernel == 0 ? RULE_FUSED32 : RULE_PLAIN32];
+    return tile_desc(m.dim, 0);
 }
 // Blocks the stage kernel launches (rows of the totals partial array).
-inline long long stage_blocks(const MeshDesc& m, int tile, bool f64) {
+inline long long stage_blocks(const MeshDesc& m, int kernel, int tile, bool f64) {
     if (m.dim == 0) return 1;
-    const TileDesc t = launch_tile(m, tile, f64);
+    const TileDesc t = launch_tile(m, kernel, tile, f64);
     if (m.dim < 3) {
         return (strip_warps<long long>(strip_plan(m.n[0]), (m.n[1] + t.zc - 1) / t.zc) + t.ty - 1) / t.ty;
     }

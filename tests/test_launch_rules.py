@@ -22,3 +22,18 @@ def test_1d_warps_per_block():
     for shape in ((1, 1, 32000), (1, 10 ** 6, 1), (10 ** 7, 1, 1)):
         assert _tile(shape) == (32, 8, 1, 256)
         assert _tile(shape, torch.float64) == (32, 1, 1, 32)
+
+
+def test_3d_tiles():
+    plain = {"kernel": hh.HARD_KERNEL_PLAIN}
+    # meshes of a few planes: 8 rows cost less per block; deep ones: 16 cost less per plane
+    for nz in (4, 5, 8):
+        assert _tile((nz, 1000, 1000))[:2] == (32, 8)
+    for n in (64, 128, 256, 512):
+        assert _tile((n, n, n))[:2] == (32, 16)
+        assert _tile((n, n, n), **plain)[:2] == (32, 4)
+    # rows that TMA does not take
+    assert _tile((93, 117, 150)) == (32, 8, 24, 256)
+    assert _tile((4, 601, 499))[:2] == (32, 16)
+    # beyond the rows that a grid of 8-row tiles takes nothing is chosen in its place
+    assert _tile((2, 8 * 65535 + 1, 2)) == _tile((2, 8 * 65535 + 1, 2), **plain) == (32, 8, 32, 256)
