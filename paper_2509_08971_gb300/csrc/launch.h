@@ -77,54 +77,59 @@ inline int choose_chunk(long long cols, int n, const Time& time, double* best = 
     return zb;
 }
 // Tile and z chunk of the 3D stage kernels, of 32-wide tiles.  A form's time is
-// `first` + the span of its blocks, of which `over` planes each are warm-up and
-// fixed cost (and `more` where they share their SM and read planes of other
-// chunks), at step[k - 1] a plane where k blocks share an SM.  `sync` (if not 0):
-// the step of a first wave that runs in phase.  The blocks of a last wave that
-// leave a fifth of the SMs' places free take the step of fewer on an SM, and then
-// nothing stays in phase (FP32).  Fitted (us) to stages of 85 meshes of 4 to 512
-// planes by every tile: the fused kernels within 3 % at most sizes, the plain one
-// within 10 %.
-//
-// One fixed 32 x 8 x 32 tile leaves most of the chip idle on small meshes and most of
-// the last wave on others (64^3: 54 us a stage against 15).  FP32 by TMA: the 16-row tile
-// pays more per block and less per plane, so 4 planes of 1000^2 want 8 rows (154 us
-// a stage, 163 by 16), 32 planes either, 256^3 16 (407, 436 by 8).  By copies: 16 rows from
-// two waves on (4 x 601 x 499: 59 against 62).  FP64 is bound by its pipe, whatever is
-// resident.  The plain FP32 kernel fills an SM best with five blocks of 4 rows (512^3: 6.6 ms
-// a stage, 7.8 by 8 rows, 8.4 by 16).
+// `first` + the span of its blocks at step[k - 1] a plane where k blocks share an SM,
+// `over` planes of each block standing for its warm-up and fixed cost.  Steps measured
+// (us): FP32 (warp-specialised, bound by issue) 1.53 a plane of 32 x 8 alone on its
+// SM, 1.85 with a second block, 1.67 of 32 x 16 (one block per SM), a block's fixed
+// cost ~3 planes; FP64 (bound by its pipe, whatever is resident) 54.6 of 32 x 8
+// and 35.1 of 32 x 4 (58 as one of two), fixed cost ~1 plane.  The plain FP32
+// kernel fills an SM best with five blocks of 4 rows (512^3: 6.6 ms a stage, 7.9 by
+// 8 rows, 8.4 by 16), and blocks of a last wave that leave a fifth of the SMs' places
+// free take the step of fewer on an SM.  One fixed 32 x 8 x 32 tile leaves most of
+// the chip idle on small meshes (64^3: 54 us a stage, 15 by the rule; plain 104
+// and 21) and most of the last wave on others.
 enum Rule3 { RULE_FUSED32, RULE_F64, RULE_PLAIN32, RULES3 };
 inline TileDesc choose_tile3(const int n[3], Rule3 rule) {
-    struct Form { int ty, kmax; double first, over, more, sync, step[5]; };
-    static constexpr Form TMA[] = {{16, 1, 3.3, 2.4, 0, 0, {1.71}}, {8, 2, 4.4, 2.05, 0.3, 1.94, {1.46, 1.74}}};
-    static constexpr Form COPIES[] = {{16, 1, 2.9, 2.4, 0, 0, {2.18}}, {8, 2, 3.2, 2.7, 0, 0, {1.58, 2.22}}};
-    static constexpr Form F64[] = {{8, 1, 0, 1.0, 0, 0, {54.6}}, {4, 2, 0, 1.2, 0, 0, {35.1, 58.0}}};
-    static constexpr Form PLAIN[] = {{8, 2, 2.1, 0.7, 0, 0, {3.26, 4.34}},
-                                     {4, 5, 1.0, 0.8, 0, 0, {3.0, 3.6, 4.0, 4.35, 4.65}}};
-    const Form* forms = rule == RULE_F64 ? F64 : rule == RULE_PLAIN32 ? PLAIN : n[0] % 4 ? COPIES : TMA;
+    struct Form { int ty, kmax; double first, over, step[5]; };
+    static constexpr Form F32[] = {{16, 1, 0, 3.2, {1.67}}, {8, 2, 0, 3.0, {1.53, 1.85}}};
+    static constexpr Form F64[] = {{8, 1, 0, 1.0, {54.6}}, {4, 2, 0, 1.2, {35.1, 58.0}}};
+    static constexpr Form PLAIN[] = {{8, 2, 2.1, 0.7, {3.26, 4.34}}, {4, 5, 1.0, 0.8, {3.0, 3.6, 4.0, 4.35, 4.65}}};
+    const Form* forms = rule == RULE_F64 ? F64 : rule == RULE_PLAIN32 ? PLAIN : F32;
+    const auto columns = [&](int ty) { return (n[0] + 31) / 32 * (long long)((n[1] + ty - 1) / ty); };
     TileDesc td{32, 8, 32};
     double tb = 1e300;
     for (const Form* f = forms; f < forms + 2; ++f) {
-        const long long gy = (n[1] + f->ty - 1) / f->ty;
         // more rows than a grid of 8-row tiles takes are refused at the launch, as before the rule
-        if (n[1] > 8 * 65535 || gy > 65535) continue;
-        const long long cols = (n[0] + 31) / 32 * gy;
+        if (n[1] > 8 * 65535 || (n[1] + f->ty - 1) / f->ty > 65535) continue;
+        const long long cols = columns(f->ty);
         double t;
         const int z = choose_chunk(cols, n[2], [&](int zc, long long blocks) {
             const int k = (int)std::min<long long>(f->kmax, (blocks + SMS - 1) / SMS);   // blocks on an SM
             const long long slots = (long long)SMS * k, rest = blocks % slots;
-            const double over = f->over + (k > 1 && zc < n[2] ? f->more : 0.0), w = zc + over, s = f->step[k - 1];
-            double t = f->first + span_steps(cols, n[2], zc, over, slots) * s;
+            const double s = f->step[k - 1];
+            double tz = f->first + span_steps(cols, n[2], zc, f->over, slots) * s;
             const int last = (int)(rest / (SMS * 4 / 5)) + 1;        // on an SM in the last wave
-            if (rule != RULE_F64 && blocks > slots && rest && last < k && n[2] % zc == 0)
-                t -= w * (s - f->step[last - 1]);
-            else if (k > 1 && f->sync > 0) t += w * (f->sync - s);
-            return t;
+            if (rule == RULE_PLAIN32 && blocks > slots && rest && last < k && n[2] % zc == 0)
+                tz -= (zc + f->over) * (s - f->step[last - 1]);
+            return tz;
         }, &t);
         if (t < tb) {
             tb = t;
             td = TileDesc{32, f->ty, z};
         }
+    }
+    // FP32 by TMA in one chunk, as thin meshes are: blocks of other columns come in by
+    // and by, which hides more of the fixed cost of the smaller ones.  16 rows
+    // (z + 2.4) 1.71 us a wave + 3.3; 8 rows (z + 2.05) 1.74 + 4.4, a last wave of
+    // up to 121 blocks at 1.46 (4 planes of 1000^2 163 us a stage against 154, 16 of 500^2
+    // 130 against 125, 16 of 256^2 35.5 against 39.0).
+    if (rule == RULE_FUSED32 && td.ty == 16 && td.zc == n[2] && n[0] % 4 == 0) {
+        const long long b8 = columns(8), b16 = columns(16), rest = b8 % (2 * SMS);
+        const double w8 = n[2] + 2.05;
+        const double t16 = 3.3 + (n[2] + 2.4) * 1.71 * (double)((b16 + SMS - 1) / SMS);
+        const double t8 = 4.4 + w8 * ((double)(b8 / (2 * SMS)) * 1.74 +
+                                      (!rest ? 0.0 : rest <= SMS * 4 / 5 ? 1.46 : 1.94));
+        if (t8 < t16) td.ty = 8;
     }
     return td;
 }
