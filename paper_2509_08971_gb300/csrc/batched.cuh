@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) batched_kernel(const BatchAr
     __shared__ unsigned long long red[NW];
     __shared__ BatchScalars<T> s_sc;
     __shared__ double s_dt, s_t;
-    __shared__ int s_next, s_chunks;
+    __shared__ int s_next, s_chunks, s_len;
     const int tid = threadIdx.x, warp = tid >> 5;
     bool bad = false;
 
@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) batched_kernel(const BatchAr
         const bool two_d = P.ny > 1;
         const long long N = (long long)P.nx * P.ny;
         const int strips = (P.nx + STRIP - 1) / STRIP;   // 1D
-        const StripPlan plan = strip_plan(P.nx);
+        const StripPlan plan = two_d ? strip_plan(P.nx, true) : StripPlan{strips, 0, 0};
         if (tid == 0) {
             s_sc.gamma = (T)P.gamma;
             s_sc.gm1 = (T)(P.gamma - 1.0);
@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) batched_kernel(const BatchAr
             s_sc.dy = make_width<T>(1.0 / P.ny);
             s_t = B.t[B.order[qi]];
         }
-        if (warp == NW - 1) {
+        if (two_d && warp == NW - 1) {
             // row chunks per strip: of 1 .. 32, the one whose rounds over the
             // block's warps take the fewest rows (a chunk pays about three
             // rows for its warm-up and look-ahead)
@@ -151,13 +151,16 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) batched_kernel(const BatchAr
             const long long cost = (long long)((strip_warps<unsigned>(plan, k) + NW - 1) / NW) * ((P.ny + k - 1) / k + 3);
             const unsigned key = ((unsigned)min(cost, (1ll << 25) - 1) << 6) | (unsigned)k;
             const unsigned best = __reduce_min_sync(FULL, key);
-            if ((tid & 31) == 0) s_chunks = two_d ? (int)(best & 63u) : 1;
+            if ((tid & 31) == 0) {
+                const int c = (int)(best & 63u);
+                s_len = (P.ny + c - 1) / c;
+                s_chunks = (P.ny + s_len - 1) / s_len;           // without empty ones
+            }
         }
         __syncthreads();
         const BatchScalars<T> sc = s_sc;
-        const int chunk = (P.ny + s_chunks - 1) / s_chunks;
-        const int chunks = (P.ny + chunk - 1) / chunk;           // s_chunks without empty ones
-        const unsigned items = strip_warps<unsigned>(plan, chunks);   // at most 32 chunks: below 2^32
+        const int chunk = s_len, chunks = s_chunks;              // 2D: rows of a chunk, chunks
+        const unsigned items = two_d ? strip_warps<unsigned>(plan, chunks) : 0;   // at most 32 chunks: below 2^32
 
         // signal rate of the initial state
         {

@@ -76,7 +76,7 @@ template <int DIM, int PX, int PY, int RR, int NWARP>
 cudaError_t run_strip(const MeshDesc& m, const TileDesc& td, const StageCall& c, cudaStream_t s) {
     static_assert(STRIP == STRIP_CELLS, "the launch rule counts the kernel's strips");
     const StageArgs<T> A = make_args(m, td, c);         // A.zchunk: rows per warp
-    const long long blocks = cdiv<long long>(strip_warps<long long>(strip_plan(m.n[0]), cdiv(m.n[1], td.zc)), NWARP);
+    const long long blocks = cdiv<long long>(strip_warps<long long>(strip_plan(m.n[0], strip_walks(td)), cdiv(m.n[1], td.zc)), NWARP);
     if (blocks >= (1ll << 31)) return cudaErrorInvalidValue;
     return launch_pdl(strip_kernel<T, DIM, PX, PY, RR, NWARP>, dim3((unsigned)blocks), dim3(32 * NWARP), 0,
                       s, A);

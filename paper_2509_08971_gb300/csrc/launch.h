@@ -160,17 +160,20 @@ inline constexpr TileDesc TILES3[] = {{32, 8, 32}, {32, 8, 64}, {32, 16, 64}, {6
 inline constexpr TileDesc TILES2[] = {{32, 2, 2}, {32, 2, 4}, {32, 2, 16}};
 inline constexpr TileDesc TILES1[] = {{32, 1, 1}, {32, 8, 1}};
 inline constexpr int STRIP_CELLS = 28;
-// The strips of rows of n0 cells: `full` of them at 32 lanes and, where the last
-// cells and their four halo cells leave half a warp and more, one whose warps
-// walk `groups` row chunks side by side, `width` lanes each.
+// The strips of rows of n0 cells: `full` of them at 32 lanes and, in long walks
+// (`share`) where the last cells and their four halo cells leave half a warp and more, one
+// whose warps walk `groups` row chunks side by side, `width` lanes each.  Short walks
+// are those of meshes that do not fill the chip, whose step is the longest warp's: loads
+// from several rows at a time only lengthen it (449 x 42 cells, 20 steps, 218 -> 228 us).
 struct StripPlan {
     int full, groups, width;
 };
-inline __host__ __device__ StripPlan strip_plan(int n0) {
+inline __host__ __device__ StripPlan strip_plan(int n0, bool share) {
     const int rest = n0 % STRIP_CELLS, g = 32 / (rest + 4);
-    if (rest == 0 || g == 1) return StripPlan{(n0 + STRIP_CELLS - 1) / STRIP_CELLS, 0, 0};
+    if (!share || rest == 0 || g == 1) return StripPlan{(n0 + STRIP_CELLS - 1) / STRIP_CELLS, 0, 0};
     return StripPlan{n0 / STRIP_CELLS, g, rest + 4};
 }
+inline bool strip_walks(const TileDesc& t) { return t.zc > 4; }   // rows in a loop, not unrolled
 // Warps of a plan over a number of row chunks (I holds the result).
 template <typename I>
 inline __host__ __device__ I strip_warps(const StripPlan& p, I chunks) {
@@ -199,7 +202,7 @@ inline TileDesc tile_desc(int dim, int tile) {
 inline TileDesc launch_tile(const MeshDesc& m, int kernel, int tile, bool f64) {
     if (tile >= 0) return tile_desc(m.dim, tile);
     if (m.dim == 2) {
-        const long long rows = strip_warps<long long>(strip_plan(m.n[0]), m.n[1]);
+        const long long rows = (long long)((m.n[0] + STRIP_CELLS - 1) / STRIP_CELLS) * m.n[1];
         const long long want = 152ll * (f64 ? 4 : 8);
         return TILES2[rows >= 16 * want ? 2 : rows >= 4 * want ? 1 : 0];
     }
@@ -212,7 +215,8 @@ inline long long stage_blocks(const MeshDesc& m, int kernel, int tile, bool f64)
     if (m.dim == 0) return 1;
     const TileDesc t = launch_tile(m, kernel, tile, f64);
     if (m.dim < 3) {
-        return (strip_warps<long long>(strip_plan(m.n[0]), (m.n[1] + t.zc - 1) / t.zc) + t.ty - 1) / t.ty;
+        const StripPlan p = strip_plan(m.n[0], strip_walks(t));
+        return (strip_warps<long long>(p, (m.n[1] + t.zc - 1) / t.zc) + t.ty - 1) / t.ty;
     }
     const long long gx = (m.n[0] + t.tx - 1) / t.tx;
     const long long gy = (m.n[1] + t.ty - 1) / t.ty;

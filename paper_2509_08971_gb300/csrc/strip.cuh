@@ -10,8 +10,8 @@
 // converted, limited and differenced once per axis and every face evaluated
 // once, by one warp; two rows of warm-up and two of look-ahead per chunk.
 // A row's last cells take a strip of their own; where they are twelve or fewer, a
-// warp walks several of its row chunks side by side (strip_plan), so a row of 29
-// cells costs 28 + 5 lanes, not 64: a step of 50000 rows of 29 cells 121 -> 81 us
+// warp on a long walk takes several of its row chunks side by side (strip_plan), so a row
+// of 29 cells costs 28 + 5 lanes, not 64: a step of 50000 rows of 29 cells 121 -> 81 us
 // (block tiles: 96), FP64 5.97 -> 3.25 ms (5.05); 2048 batched problems of 29 to 32
 // cells a side, five steps, 0.80 -> 0.62 ms (0.62).
 //
@@ -19,7 +19,7 @@
 // small meshes the latency of one strip.  It replaces a 32 x 8 tile per block
 // (primitives and both face fluxes through shared memory, two barriers, every
 // slope twice): 757 issue slots per cell-stage there.  Measured, bit-identical: 4096 batched
-// problems, five steps, 15.45 -> 10.12 ms; 100 FP64 steps of a 400-cell mesh
+// problems, five steps, 15.45 -> 10.07 ms; 100 FP64 steps of a 400-cell mesh
 // (15 SMs instead of 4) 4.73 -> 3.09 ms; 50 FP32 steps at 256^2 0.92 -> 0.84 ms.
 //
 // strip_rows evaluates the same expressions in the same order whatever the
@@ -228,35 +228,40 @@ __device__ __forceinline__ void strip_item(const StageArgs<T>& A, const StripPla
 }
 
 // Block reductions of what the block's warps accumulated: the non-physical
-// flag, the rate maximum (one atomic per block: the slot takes about one a
-// nanosecond from the whole chip), and the block's row of the totals partial array.
+// flag, the rate maximum, and the block's row of the totals partial array.  Blocks
+// of many warps send one atomic to the rate slot, which takes about one a
+// nanosecond from the whole chip; the small blocks of small meshes need not wait.
 template <typename T, int NWARP, bool ERR>
 __device__ __forceinline__ void strip_epilogue(const StageArgs<T>& A, const TileAcc<T>& acc) {
+    constexpr bool COMBINE = NWARP > 2;
     __shared__ double red_tot[NWARP][NF];
     __shared__ unsigned long long red_rate[NWARP];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool any_bad = __any_sync(FULL, acc.bad);
     if (any_bad && lane == 0) atomicOr(A.status, 1);
-    unsigned long long b = 0;
     if (A.rate_slot) {
-        b = rate_bits(acc.rate_max);
+        unsigned long long b = rate_bits(acc.rate_max);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             const unsigned long long v = __shfl_xor_sync(FULL, b, o);
             b = v > b ? v : b;
         }
-        if (NWARP > 1 && lane == 0) red_rate[warp] = b;
+        if (lane == 0) {
+            if (COMBINE) red_rate[warp] = b;
+            else atomicMax(A.rate_slot, b);
+        }
     }
     if (A.tot_partial) {
         const double s = warp_totals<ERR>(acc.tot, lane);
         if (sum5_writer(lane)) red_tot[warp][sum5_field(lane)] = s;
     }
-    if (!A.rate_slot && !A.tot_partial) return;
-    if (NWARP > 1) __syncthreads();
-    else __syncwarp();
-    if (A.rate_slot && threadIdx.x == 0) {
-        if (NWARP > 1)
-            for (int w = 1; w < NWARP; ++w) b = red_rate[w] > b ? red_rate[w] : b;
+    if (A.tot_partial || (COMBINE && A.rate_slot)) {
+        if (NWARP > 1) __syncthreads();
+        else __syncwarp();
+    }
+    if (COMBINE && A.rate_slot && threadIdx.x == 0) {
+        unsigned long long b = red_rate[0];
+        for (int w = 1; w < NWARP; ++w) b = red_rate[w] > b ? red_rate[w] : b;
         atomicMax(A.rate_slot, b);
     }
     if (A.tot_partial && threadIdx.x < NF) {
@@ -276,7 +281,7 @@ __global__ void __launch_bounds__(32 * NWARP) strip_kernel(const StageArgs<T> A)
         if (item * STRIP < A.n[0])
             strip_rows<T, DIM, PX, PY, RR>(A, (int)item * STRIP, threadIdx.x & 31, 0, 1, 1, acc);
     } else {
-        const StripPlan p = strip_plan(A.n[0]);
+        const StripPlan p = strip_plan(A.n[0], RR == 0);
         const int chunks = (A.n[1] + A.zchunk - 1) / A.zchunk;
         if (item < strip_warps<long long>(p, chunks)) strip_item<T, PX, PY, RR>(A, p, item, chunks, A.zchunk, acc);
     }
