@@ -254,18 +254,20 @@ cudaError_t run_stage_ws(const MeshDesc& m, const TileDesc& td, const StageCall&
         const char* starve = std::getenv("HARD_HYDRO_STARVE_TMA");
         A.starve_tma = TMA && starve && starve[0] == '1';
         dim3 grid(cdiv(m.n[0], 32), cdiv(m.n[1], TY), cdiv(A.zhi - A.zlo, A.zchunk));
-        static std::atomic<unsigned long long> attr1{0}, attr2{0};
+        static std::atomic<unsigned long long> attr1{0}, attr2[2] = {{0}, {0}};
         cudaError_t e;
         if (c.stage == 1) {
-            e = smem_attr_once(stage_ws_kernel<32, TY, NCW, 1, RPW, TMA>, L1::bytes, attr1);
+            e = smem_attr_once(stage_ws_kernel<32, TY, NCW, 1, RPW, TMA, false>, L1::bytes, attr1);
             if (e != cudaSuccess) return e;
-            e = launch_pdl(stage_ws_kernel<32, TY, NCW, 1, RPW, TMA>, grid, dim3(L1::NT), L1::bytes, s, A,
+            e = launch_pdl(stage_ws_kernel<32, TY, NCW, 1, RPW, TMA, false>, grid, dim3(L1::NT), L1::bytes, s, A,
                            maps);
         } else {
-            e = smem_attr_once(stage_ws_kernel<32, TY, NCW, 2, RPW, TMA>, L2::bytes, attr2);
+            const bool tot = c.tot_partial != nullptr;
+            auto kern = tot ? stage_ws_kernel<32, TY, NCW, 2, RPW, TMA, true>
+                            : stage_ws_kernel<32, TY, NCW, 2, RPW, TMA, false>;
+            e = smem_attr_once(kern, L2::bytes, attr2[tot]);
             if (e != cudaSuccess) return e;
-            e = launch_pdl(stage_ws_kernel<32, TY, NCW, 2, RPW, TMA>, grid, dim3(L2::NT), L2::bytes, s, A,
-                           maps);
+            e = launch_pdl(kern, grid, dim3(L2::NT), L2::bytes, s, A, maps);
         }
         used = true;
         return e;

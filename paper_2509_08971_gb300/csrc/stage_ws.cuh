@@ -221,7 +221,11 @@ __device__ __forceinline__ float ws_rate(const float U[NF], float gamma, float g
 // consecutive tile rows: with two, the y slope of a row is shared by the two
 // y faces around it and the iteration's control work is spread over two
 // cells per thread.
-template <int TX, int TY, int NCW, int STAGE, int RPW, bool TMA>
+// TOT: with the totals epilogue (stage 2).  Its lane sums and their error words are ten
+// registers and four operations a field and cell; a form of its own keeps them out of
+// steps without the log (256^3, four steps, 3.352 ms against 3.387 with one form for both; two
+// steps of the 512^3 blast with the log 13.52 ms, 13.41 with plain FP32 lane sums).
+template <int TX, int TY, int NCW, int STAGE, int RPW, bool TMA, bool TOT>
 __global__ void __launch_bounds__(32 * (TY / RPW + NCW), TY >= 16 ? 1 : (TY >= 8 ? 2 : 3))
 stage_ws_kernel(const __grid_constant__ StageArgs<float> A, const __grid_constant__ WsMaps M) {
     using L = WsLayout<TX, TY, NCW, STAGE, RPW, TMA>;
@@ -583,7 +587,7 @@ stage_ws_kernel(const __grid_constant__ StageArgs<float> A, const __grid_constan
                                 const bool up = own[r] && (rr > rate_max || rr != rr);
                                 rate_max = up ? rr : rate_max;
                             }
-                            if (EPI && A.tot_partial) {
+                            if (TOT) {
 #pragma unroll
                                 for (int f = 0; f < NF; ++f) tot[f].add_down(RPW == 1 || own[r] ? Uo[f] : 0.f);
                             }
@@ -735,7 +739,7 @@ stage_ws_kernel(const __grid_constant__ StageArgs<float> A, const __grid_constan
         }
         if (lane == 0) red_rate[warp] = b;
     }
-    if (EPI && A.tot_partial && facew) {
+    if (TOT && facew) {
         if (RPW == 1 && !own[0])                        // a lane's row is its own or it is not
 #pragma unroll
             for (int f = 0; f < NF; ++f) tot[f] = LaneSum<float>();
@@ -751,7 +755,7 @@ stage_ws_kernel(const __grid_constant__ StageArgs<float> A, const __grid_constan
             atomicMax(A.rate_slot, b);
         }
     }
-    if (EPI && A.tot_partial && tid < NF) {
+    if (TOT && tid < NF) {
         const long long bz = A.zlo / A.zchunk + blockIdx.z;
         const long long blk = (bz * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
         double s = 0.0;
