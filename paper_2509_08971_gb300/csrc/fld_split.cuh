@@ -19,7 +19,7 @@
 // What bounds it: memory.  A half-sweep of a 256^3 FP32 level moves 168 MB (x
 // of one colour, b and x of the other, D of both) in 34 us against 242 MB in 52 us
 // in mesh order; the prolongation corrects one colour only (19 us against 36), the
-// residual norm takes 34 us (53), the step to 1e-5 (four cycles) 2.23 ms (3.11).
+// residual norm takes 34 us (53), the step to 1e-5 (four cycles) 2.20 ms (3.11).
 #pragma once
 #include "pdl.h"
 
@@ -275,8 +275,8 @@ __global__ void __launch_bounds__(128, 4) split_smooth_kernel(const SplitArgs<T>
 }
 
 // sum r^2 over the cells of colour c, r = b - A x, into *out.  The 2 V terms of two
-// planes are summed in the element type, everything after them in FP64 (with the FP64
-// addition at each plane the 256^3 step took 2.216 ms, without any 2.205).
+// planes are summed in the element type, everything after them in FP64 (the 256^3 FP32
+// step 2.204 ms; with an FP64 addition at each plane 2.216, with none before the warp 2.196).
 template <typename T, bool WALLS>
 __global__ void __launch_bounds__(128) split_norm_kernel(const SplitArgs<T> a, int c, int chunk,
                                                          double* out) {

@@ -144,8 +144,8 @@ struct StageCall {
     unsigned long long* rate_slot; // nullptr = no rate epilogue
     double* tot_partial;           // nullptr = no totals epilogue
     int* status;
-    int zlo = 0, zhi = -1;         // 3D: the kernel-z cells [zlo, zhi) to update (-1: to nz);
-                                   // zlo a multiple of the tile's z-chunk
+    int zlo = 0, zhi = -1;         // 3D: the kernel-z cells [zlo, zhi) to update (-1: to nz; every
+                                   // call takes all of them); zlo a multiple of launch_tile's zc
     const void* zg[2] = {nullptr, nullptr};  // ghost planes of BC_HALO z faces (below, above),
                                              // each [5][2][ny][nx]
     void* scratch = nullptr;       // WENO on 3D meshes: [5][N] flux-difference buffer of the

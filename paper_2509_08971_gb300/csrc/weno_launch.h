@@ -33,7 +33,7 @@ inline constexpr int WENO_TX1 = 128, WENO_TX2 = 32, WENO_TY2 = 8, WENO_ZC = 32;
 
 // Blocks of the launch that carries a WENO stage's epilogue (rows of the
 // totals partial array): the combining z' march of the sweeps, or the fused
-// kernel's grid (the first tile of the mesh's tile table).
+// kernel's grid.
 inline long long weno_stage_blocks(const MeshDesc& m, bool sweeps, bool f64) {
     if (m.dim == 3 && sweeps) {
         const long long columns = (long long)m.n[0] * m.n[1];
