@@ -837,14 +837,28 @@ int split_chunk(const SplitArgs<T>& a) {
     return c;
 }
 
+// Threads per block of a half-sweep: FP64 ones last as long as the SM with the most
+// blocks, whose pipe they fill; 64 where that SM's share is so at least 6 % smaller (61^3
+// between walls 2.77 -> 2.55 ms, mesh order 2.54; 121^3 16.3 -> 14.5, 15.6; at 96^3, where it
+// would be 4 %, 2.30 -> 2.38).
+template <typename T>
+int smooth_threads(const SplitArgs<T>& a, int chunk) {
+    const auto share = [&](int nt) {
+        const long long blocks = ((long long)a.groups * a.n[1] + nt - 1) / nt * ((a.n[2] + chunk - 1) / chunk);
+        return (double)((blocks + 151) / 152) * nt;
+    };
+    return sizeof(T) == 8 && share(64) < 0.94 * share(128) ? 64 : 128;
+}
+
 template <typename T>
 cudaError_t smooth_split(const FldHierarchy* H, int l, double dt, int sweeps, cudaStream_t s) {
     const SplitArgs<T> a = split_args<T>(H, l, dt);
     const int chunk = split_chunk(a);
-    const dim3 g = flat_grid(a.groups, a.n[1], (a.n[2] + chunk - 1) / chunk);
+    const int nt = smooth_threads(a, chunk);
+    const dim3 g((unsigned)(((long long)a.groups * a.n[1] + nt - 1) / nt), (unsigned)((a.n[2] + chunk - 1) / chunk));
     auto kern = a.per[0] ? split_smooth_kernel<T, false> : split_smooth_kernel<T, true>;
     for (int it = 0; it < 2 * sweeps; ++it) {
-        const cudaError_t e = launch_pdl(kern, g, dim3(128), 0, s, a, it & 1, chunk);
+        const cudaError_t e = launch_pdl(kern, g, dim3((unsigned)nt), 0, s, a, it & 1, chunk);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
